@@ -203,16 +203,20 @@ __global__ void __launch_bounds__(Shape<EPI, PAIR, TBN>::THREADS, 1)
 
   if (warp == 0) {
     // ------------------------------------------------------------ producer
-    if (lane == 0) {
-      int stage = 0;
-      uint32_t phase = 0;
-      int issued = 0;
-      bool ok = true;
-      for (int it = 0; ok && work_item(sched, it, w); ++it) {
-        const int m0 = (w.tile / p.n_tiles) * TILE_M + static_cast<int>(rank) * BM;
-        const int n0 = (w.tile % p.n_tiles) * TBN + static_cast<int>(rank) * (TBN - B_ROWS);
-        for (int kb = w.kb0; kb < w.kb1; ++kb) {
-          if (!ptx::mbar_wait(&empty[stage], phase ^ 1u, lim, p.status)) { ok = false; break; }
+    // The whole warp walks the loop and one elected lane issues, so that the
+    // addresses and coordinates stay warp-uniform (as in the MMA warp below).
+    const bool issuer = ptx::elect_one();
+    int stage = 0;
+    uint32_t phase = 0;
+    int issued = 0;
+    bool ok = true;
+    for (int it = 0; ok && work_item(sched, it, w); ++it) {
+      const int m0 = (w.tile / p.n_tiles) * TILE_M + static_cast<int>(rank) * BM;
+      const int n0 = (w.tile % p.n_tiles) * TBN + static_cast<int>(rank) * (TBN - B_ROWS);
+      for (int kb = w.kb0; kb < w.kb1; ++kb) {
+        ok = __all_sync(0xffffffffu, ptx::mbar_wait(&empty[stage], phase ^ 1u, lim, p.status));
+        if (!ok) break;
+        if (issuer) {
           uint8_t* sa = smem + stage * SBYTES;
           uint8_t* sb = sa + A_BYTES;
           // the leader's stage barrier expects both CTAs' bytes
@@ -240,27 +244,41 @@ __global__ void __launch_bounds__(Shape<EPI, PAIR, TBN>::THREADS, 1)
               load(sb, &tmB, k0, n0);
             }
           }
-          ++issued;
-          if (++stage == NST) { stage = 0; phase ^= 1u; }
         }
+        __syncwarp();
+        ++issued;
+        if (++stage == NST) { stage = 0; phase ^= 1u; }
       }
-      // Drain: wait (bounded) for the loads still in flight before exiting.
-      // The leader's stage barriers count the peer's loads too; the peer
-      // stays resident until the leader has drained (final cluster barrier).
-      const int n_tail = !leader ? 0 : (issued < NST ? issued : NST);
-      for (int i = 0; i < n_tail; ++i) {
-        if (--stage < 0) { stage = NST - 1; phase ^= 1u; }
-        ptx::mbar_wait(&full[stage], phase, lim, p.status);
-      }
+    }
+    // Drain: wait (bounded) for the loads still in flight before exiting.
+    // The leader's stage barriers count the peer's loads too; the peer
+    // stays resident until the leader has drained (final cluster barrier).
+    const int n_tail = !leader ? 0 : (issued < NST ? issued : NST);
+    for (int i = 0; i < n_tail; ++i) {
+      if (--stage < 0) { stage = NST - 1; phase ^= 1u; }
+      ptx::mbar_wait(&full[stage], phase, lim, p.status);
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------- MMA issue
-    if (lane == 0 && leader) {
+    // A tcgen05.mma takes its descriptors from uniform registers.  With the
+    // loop inside one lane's branch they were built per lane for every
+    // instruction, about 130 cycles each: as long as the tensor pipe works on
+    // one (M = 256, N = 256, K = 16).  FFN forward of the large width, 4999
+    // rows: 106.8 -> 105.1 us; two base-width layers on 74 rows 139.4 -> 137.1.
+    if (leader) {
       constexpr uint32_t idesc = ptx::idesc_bf16_f32(TILE_M, TBN, A_MN, B_MN);
+      const bool issuer = ptx::elect_one();
       auto commit = [&](uint64_t* bar) {  // to this barrier in both CTAs of a pair
         if constexpr (PAIR) ptx::tc_commit_pair(bar, 3);
         else ptx::tc_commit(bar);
       };
+      // descriptors of stage 0; a stage or K step further adds to the address
+      // field (16-byte units), which never carries out of it
+      const uint32_t s0 = ptx::smem_u32(smem);
+      const uint64_t da = A_MN ? ptx::smem_desc_sw128(s0, MN_CHUNK_BYTES, 1024)
+                               : ptx::smem_desc_sw128(s0, 16, 1024);
+      const uint64_t db = B_MN ? ptx::smem_desc_sw128(s0 + A_BYTES, MN_CHUNK_BYTES, 1024)
+                               : ptx::smem_desc_sw128(s0 + A_BYTES, 16, 1024);
       int stage = 0;
       uint32_t phase = 0;
       int acc = 0;
@@ -268,37 +286,41 @@ __global__ void __launch_bounds__(Shape<EPI, PAIR, TBN>::THREADS, 1)
       bool ok = true;
       for (int it = 0; ok && work_item(sched, it, w); ++it) {
         // both CTAs' epilogues have drained this accumulator
-        if (!(PAIR ? ptx::mbar_wait_cluster(&tempty[acc], aphase ^ 1u, lim, p.status)
-                   : ptx::mbar_wait(&tempty[acc], aphase ^ 1u, lim, p.status)))
-          break;
+        const bool freed = PAIR ? ptx::mbar_wait_cluster(&tempty[acc], aphase ^ 1u, lim, p.status)
+                                : ptx::mbar_wait(&tempty[acc], aphase ^ 1u, lim, p.status);
+        if (!__all_sync(0xffffffffu, freed)) break;
         ptx::tc_fence_after();
         const uint32_t d_tmem = tmem_base + acc * TBN;
         for (int kb = w.kb0; kb < w.kb1; ++kb) {
-          if (!ptx::mbar_wait(&full[stage], phase, lim, p.status)) { ok = false; break; }
+          ok = __all_sync(0xffffffffu, ptx::mbar_wait(&full[stage], phase, lim, p.status));
+          if (!ok) break;
           ptx::tc_fence_after();
-          const uint32_t sa = ptx::smem_u32(smem + stage * SBYTES);
-          const uint32_t sb = sa + A_BYTES;
+          if (issuer) {
+            const uint64_t off = static_cast<uint64_t>(stage * (SBYTES >> 4));
 #pragma unroll
-          for (int kk = 0; kk < BK / 16; ++kk) {
-            const uint64_t ad = A_MN ? ptx::smem_desc_sw128(sa + kk * 2048, MN_CHUNK_BYTES, 1024)
-                                     : ptx::smem_desc_sw128(sa + kk * 32, 16, 1024);
-            const uint64_t bd = B_MN ? ptx::smem_desc_sw128(sb + kk * 2048, MN_CHUNK_BYTES, 1024)
-                                     : ptx::smem_desc_sw128(sb + kk * 32, 16, 1024);
-            if constexpr (PAIR)
-              ptx::tc_mma_f16_pair(d_tmem, ad, bd, idesc, (kb > w.kb0 || kk > 0) ? 1u : 0u);
-            else
-              ptx::tc_mma_f16(d_tmem, ad, bd, idesc, (kb > w.kb0 || kk > 0) ? 1u : 0u);
+            for (int kk = 0; kk < BK / 16; ++kk) {
+              const uint64_t ad = da + off + kk * (A_MN ? 128 : 2), bd = db + off + kk * (B_MN ? 128 : 2);
+              if constexpr (PAIR)
+                ptx::tc_mma_f16_pair(d_tmem, ad, bd, idesc, (kb > w.kb0 || kk > 0) ? 1u : 0u);
+              else
+                ptx::tc_mma_f16(d_tmem, ad, bd, idesc, (kb > w.kb0 || kk > 0) ? 1u : 0u);
+            }
+            commit(&empty[stage]);
           }
-          commit(&empty[stage]);
+          __syncwarp();
           if (++stage == NST) { stage = 0; phase ^= 1u; }
         }
         if (!ok) break;
-        commit(&tfull[acc]);
+        if (issuer) commit(&tfull[acc]);
+        __syncwarp();
         if (++acc == 2) { acc = 0; aphase ^= 1u; }
       }
       // All issued MMAs must finish before TMEM is released.
-      if constexpr (PAIR) ptx::tc_commit_pair(done, 1);
-      else ptx::tc_commit(done);
+      if (issuer) {
+        if constexpr (PAIR) ptx::tc_commit_pair(done, 1);
+        else ptx::tc_commit(done);
+      }
+      __syncwarp();
       ptx::mbar_wait(done, 0, lim, p.status);
     }
   } else {
