@@ -142,75 +142,89 @@ __global__ void __launch_bounds__(NTHR, 2) attn_fwd_tc(const __grid_constant__ C
     // Loads Q and the first F_STAGES K/V tiles, then per tile j: issues
     // O += P_j V_j once the softmax warps have written P_j, and refills the
     // ring slot of tile j with tile j + F_STAGES once S_j and P_j V_j have
-    // read it.  (Two threads issue this CTA's MMAs: one thread issues a
-    // tcgen05.mma only about every 100 cycles.)
-    if (lane == 0) {
-      constexpr uint32_t idO = ptx::idesc_bf16_f32(BQ, HD, false, true);
-      const uint32_t skv = ptx::smem_u32(smem + F_KV_OFF);
-      auto load_kv = [&](int j) {
-        const int st = j % F_STAGES;
-        uint8_t* kv = smem + F_KV_OFF + st * 2 * KV_BYTES;
-        ptx::mbar_arrive_expect_tx(&kv_full[st], 2 * KV_BYTES);
-        ptx::tma_load_2d(kv, &tmKV, &kv_full[st], H + a * HD, row0 + j * BKV);
-        ptx::tma_load_2d(kv + KV_BYTES, &tmKV, &kv_full[st], 2 * H + a * HD, row0 + j * BKV);
-      };
+    // read it.
+    // The whole warp walks the loop and one elected lane issues: a
+    // tcgen05.mma takes its descriptors from uniform registers, and built
+    // inside one lane's branch they were moved there instruction by
+    // instruction, slower than the tensor pipe works on these products.
+    constexpr uint32_t idO = ptx::idesc_bf16_f32(BQ, HD, false, true);
+    const bool issuer = ptx::elect_one();
+    const uint64_t dv0 = ptx::smem_desc_sw128(ptx::smem_u32(smem + F_KV_OFF + KV_BYTES), 8192, 1024);
+    auto wait = [&](uint64_t* bar, uint32_t parity) {
+      return __all_sync(0xffffffffu, ptx::mbar_wait(bar, parity, lim, p.status, kWaitHint));
+    };
+    auto load_kv = [&](int j) {
+      const int st = j % F_STAGES;
+      uint8_t* kv = smem + F_KV_OFF + st * 2 * KV_BYTES;
+      ptx::mbar_arrive_expect_tx(&kv_full[st], 2 * KV_BYTES);
+      ptx::tma_load_2d(kv, &tmKV, &kv_full[st], H + a * HD, row0 + j * BKV);
+      ptx::tma_load_2d(kv + KV_BYTES, &tmKV, &kv_full[st], 2 * H + a * HD, row0 + j * BKV);
+    };
+    if (issuer) {
       ptx::mbar_arrive_expect_tx(q_full, Q_BYTES);
       ptx::tma_load_2d(smem + F_Q_OFF, &tmQ, q_full, a * HD, row0 + q0);
-      int issued = 0;
-      for (; issued < n_kt && issued < F_STAGES; ++issued) load_kv(issued);
-      for (int j = 0; j < n_kt; ++j) {
-        if (!ptx::mbar_wait(&p_full[j & 1], (j >> 1) & 1, lim, p.status, kWaitHint)) break;
-        if (!ptx::mbar_wait(&kv_full[j % F_STAGES], (j / F_STAGES) & 1, lim, p.status, kWaitHint))
-          break;
-        ptx::tc_fence_after();
-        const uint32_t sv = skv + (j % F_STAGES) * 2 * KV_BYTES + KV_BYTES;
+    }
+    int issued = 0;
+    for (; issued < n_kt && issued < F_STAGES; ++issued)
+      if (issuer) load_kv(issued);
+    __syncwarp();
+    for (int j = 0; j < n_kt; ++j) {
+      if (!wait(&p_full[j & 1], (j >> 1) & 1)) break;
+      if (!wait(&kv_full[j % F_STAGES], (j / F_STAGES) & 1)) break;
+      ptx::tc_fence_after();
+      if (issuer) {
+        const uint64_t dv = dv0 + static_cast<uint64_t>((j % F_STAGES) * (2 * KV_BYTES >> 4));
         const uint32_t tpj = tP + (j & 1) * (BKV / 2);
 #pragma unroll
         for (int kk = 0; kk < BKV / 16; ++kk)
-          ptx::tc_mma_f16_tmem_a(tO, tpj + kk * 8, ptx::smem_desc_sw128(sv + kk * 2048, 8192, 1024),
-                                 idO, (j > 0 || kk > 0) ? 1u : 0u);
+          ptx::tc_mma_f16_tmem_a(tO, tpj + kk * 8, dv + kk * 128, idO, (j > 0 || kk > 0) ? 1u : 0u);
         ptx::tc_commit(&pv_done[j & 1]);
         ptx::tc_commit(&kv_empty[j % F_STAGES]);
-        if (issued < n_kt) {  // the slot of tile j takes tile j + F_STAGES
-          const int st = issued % F_STAGES;
-          if (!ptx::mbar_wait(&kv_empty[st], ((issued / F_STAGES) & 1) ^ 1u, lim, p.status, kWaitHint))
-            break;
-          load_kv(issued++);
-        }
       }
-      ptx::tc_commit(&done[1]);
-      ptx::mbar_wait(&done[1], 0, lim, p.status, kWaitHint);
-      // drain: bounded waits for the copies still in flight
-      ptx::mbar_wait(q_full, 0, lim, p.status, kWaitHint);
-      for (int j = issued - 1; j >= 0 && j >= issued - F_STAGES; --j)
-        ptx::mbar_wait(&kv_full[j % F_STAGES], (j / F_STAGES) & 1, lim, p.status, kWaitHint);
+      __syncwarp();
+      if (issued < n_kt) {  // the slot of tile j takes tile j + F_STAGES
+        if (!wait(&kv_empty[issued % F_STAGES], ((issued / F_STAGES) & 1) ^ 1u)) break;
+        if (issuer) load_kv(issued);
+        __syncwarp();
+        ++issued;
+      }
     }
+    if (issuer) ptx::tc_commit(&done[1]);
+    __syncwarp();
+    ptx::mbar_wait(&done[1], 0, lim, p.status, kWaitHint);
+    // drain: bounded waits for the copies still in flight
+    ptx::mbar_wait(q_full, 0, lim, p.status, kWaitHint);
+    for (int j = issued - 1; j >= 0 && j >= issued - F_STAGES; --j)
+      ptx::mbar_wait(&kv_full[j % F_STAGES], (j / F_STAGES) & 1, lim, p.status, kWaitHint);
   } else if (warp == 1) {
     // --------------------------------------------- S = Q K^T issue (warp 1)
     // S_j goes into buffer j & 1 as soon as K_j has landed and the softmax
     // warps hold S_{j-2} in registers (s_free)
-    if (lane == 0) {
-      constexpr uint32_t idS = ptx::idesc_bf16_f32(BQ, BKV, false, false);
-      const uint32_t sq = ptx::smem_u32(smem + F_Q_OFF);
-      const uint32_t skv = ptx::smem_u32(smem + F_KV_OFF);
-      bool ok = ptx::mbar_wait(q_full, 0, lim, p.status, kWaitHint);
-      for (int j = 0; j < n_kt && ok; ++j) {
-        if (j >= 2 && !ptx::mbar_wait(&s_free[j & 1], ((j - 2) >> 1) & 1, lim, p.status, kWaitHint))
-          break;
-        if (!ptx::mbar_wait(&kv_full[j % F_STAGES], (j / F_STAGES) & 1, lim, p.status, kWaitHint))
-          break;
-        ptx::tc_fence_after();
-        const uint32_t sk = skv + (j % F_STAGES) * 2 * KV_BYTES;
+    constexpr uint32_t idS = ptx::idesc_bf16_f32(BQ, BKV, false, false);
+    const bool issuer = ptx::elect_one();
+    const uint64_t dq = ptx::smem_desc_sw128(ptx::smem_u32(smem + F_Q_OFF), 16, 1024);
+    const uint64_t dk0 = ptx::smem_desc_sw128(ptx::smem_u32(smem + F_KV_OFF), 16, 1024);
+    auto wait = [&](uint64_t* bar, uint32_t parity) {
+      return __all_sync(0xffffffffu, ptx::mbar_wait(bar, parity, lim, p.status, kWaitHint));
+    };
+    bool ok = wait(q_full, 0);
+    for (int j = 0; j < n_kt && ok; ++j) {
+      if (j >= 2 && !wait(&s_free[j & 1], ((j - 2) >> 1) & 1)) break;
+      if (!wait(&kv_full[j % F_STAGES], (j / F_STAGES) & 1)) break;
+      ptx::tc_fence_after();
+      if (issuer) {
+        const uint64_t dk = dk0 + static_cast<uint64_t>((j % F_STAGES) * (2 * KV_BYTES >> 4));
 #pragma unroll
         for (int kk = 0; kk < HD / 16; ++kk)
-          ptx::tc_mma_f16(tS + (j & 1) * BKV, ptx::smem_desc_sw128(sq + kk * 32, 16, 1024),
-                          ptx::smem_desc_sw128(sk + kk * 32, 16, 1024), idS, kk > 0 ? 1u : 0u);
+          ptx::tc_mma_f16(tS + (j & 1) * BKV, dq + kk * 2, dk + kk * 2, idS, kk > 0 ? 1u : 0u);
         ptx::tc_commit(&s_full[j & 1]);
         ptx::tc_commit(&kv_empty[j % F_STAGES]);
       }
-      ptx::tc_commit(&done[0]);
-      ptx::mbar_wait(&done[0], 0, lim, p.status, kWaitHint);
+      __syncwarp();
     }
+    if (issuer) ptx::tc_commit(&done[0]);
+    __syncwarp();
+    ptx::mbar_wait(&done[0], 0, lim, p.status, kWaitHint);
   } else {
     // --------------------------------------------------- softmax / epilogue
     const int q4 = warp & 3;
@@ -478,56 +492,63 @@ __global__ void __maxnreg__(80) attn_bwd_dq_tc(const __grid_constant__ CUtensorM
         ptx::mbar_wait(&kv_full[j % DQ_STAGES], (j / DQ_STAGES) & 1, lim, p.status, kWaitHint);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      constexpr uint32_t idS = ptx::idesc_bf16_f32(BQ, BKV, false, false);
-      const uint32_t sq = ptx::smem_u32(smem + DQ_Q_OFF), so = ptx::smem_u32(smem + DQ_DO_OFF);
-      const uint32_t skv = ptx::smem_u32(smem + DQ_KV_OFF);
-      // S_j = Q K_j^T and dP_j = dO V_j^T, as soon as the softmax warps hold
-      // S_{j-1} / dP_{j-1} in registers (s_free) and K_j / V_j have landed
-      bool ok = ptx::mbar_wait(qd_full, 0, lim, p.status, kWaitHint);
-      for (int j = 0; j < n_kt && ok; ++j) {
-        if (j >= 1 && !ptx::mbar_wait(s_free, (j - 1) & 1, lim, p.status, kWaitHint)) break;
-        if (!ptx::mbar_wait(&kv_full[j % DQ_STAGES], (j / DQ_STAGES) & 1, lim, p.status, kWaitHint))
-          break;
-        ptx::tc_fence_after();
-        const uint32_t sk = skv + (j % DQ_STAGES) * 2 * KV_BYTES, sv = sk + KV_BYTES;
+    constexpr uint32_t idS = ptx::idesc_bf16_f32(BQ, BKV, false, false);
+    const bool issuer = ptx::elect_one();
+    const uint64_t dq = ptx::smem_desc_sw128(ptx::smem_u32(smem + DQ_Q_OFF), 16, 1024);
+    const uint64_t dd = ptx::smem_desc_sw128(ptx::smem_u32(smem + DQ_DO_OFF), 16, 1024);
+    const uint64_t dk0 = ptx::smem_desc_sw128(ptx::smem_u32(smem + DQ_KV_OFF), 16, 1024);
+    auto wait = [&](uint64_t* bar, uint32_t parity) {
+      return __all_sync(0xffffffffu, ptx::mbar_wait(bar, parity, lim, p.status, kWaitHint));
+    };
+    // S_j = Q K_j^T and dP_j = dO V_j^T, as soon as the softmax warps hold
+    // S_{j-1} / dP_{j-1} in registers (s_free) and K_j / V_j have landed
+    bool ok = wait(qd_full, 0);
+    for (int j = 0; j < n_kt && ok; ++j) {
+      if (j >= 1 && !wait(s_free, (j - 1) & 1)) break;
+      if (!wait(&kv_full[j % DQ_STAGES], (j / DQ_STAGES) & 1)) break;
+      ptx::tc_fence_after();
+      if (issuer) {
+        const uint64_t dk = dk0 + static_cast<uint64_t>((j % DQ_STAGES) * (2 * KV_BYTES >> 4));
 #pragma unroll
         for (int kk = 0; kk < HD / 16; ++kk)
-          ptx::tc_mma_f16(tS, ptx::smem_desc_sw128(sq + kk * 32, 16, 1024),
-                          ptx::smem_desc_sw128(sk + kk * 32, 16, 1024), idS, kk > 0 ? 1u : 0u);
+          ptx::tc_mma_f16(tS, dq + kk * 2, dk + kk * 2, idS, kk > 0 ? 1u : 0u);
 #pragma unroll
         for (int kk = 0; kk < HD / 16; ++kk)
-          ptx::tc_mma_f16(tdP, ptx::smem_desc_sw128(so + kk * 32, 16, 1024),
-                          ptx::smem_desc_sw128(sv + kk * 32, 16, 1024), idS, kk > 0 ? 1u : 0u);
+          ptx::tc_mma_f16(tdP, dd + kk * 2, dk + (KV_BYTES >> 4) + kk * 2, idS, kk > 0 ? 1u : 0u);
         ptx::tc_commit(s_full);
         ptx::tc_commit(&kv_empty[j % DQ_STAGES]);
       }
-      ptx::tc_commit(&done[0]);
-      ptx::mbar_wait(&done[0], 0, lim, p.status, kWaitHint);
+      __syncwarp();
     }
+    if (issuer) ptx::tc_commit(&done[0]);
+    __syncwarp();
+    ptx::mbar_wait(&done[0], 0, lim, p.status, kWaitHint);
   } else if (warp == 10) {
-    // dQ += dS_j K_j, in tile order, from a warp of its own: one thread
-    // issues a tcgen05.mma only about every 100 cycles, so the dQ products
-    // and the score products of the next tile go in side by side
-    if (lane == 0) {
-      constexpr uint32_t idQ = ptx::idesc_bf16_f32(BQ, HD, false, true);
-      const uint32_t skv = ptx::smem_u32(smem + DQ_KV_OFF);
-      for (int j = 0; j < n_kt; ++j) {
-        if (!ptx::mbar_wait(ds_full, j & 1, lim, p.status, kWaitHint)) break;
-        if (!ptx::mbar_wait(&kv_full[j % DQ_STAGES], (j / DQ_STAGES) & 1, lim, p.status, kWaitHint))
-          break;
-        ptx::tc_fence_after();
-        const uint32_t sk = skv + (j % DQ_STAGES) * 2 * KV_BYTES;
+    // dQ += dS_j K_j, in tile order, from a warp of its own, so that the dQ
+    // products and the score products of the next tile go in side by side
+    constexpr uint32_t idQ = ptx::idesc_bf16_f32(BQ, HD, false, true);
+    const bool issuer = ptx::elect_one();
+    const uint64_t dk0 = ptx::smem_desc_sw128(ptx::smem_u32(smem + DQ_KV_OFF), 8192, 1024);
+    auto wait = [&](uint64_t* bar, uint32_t parity) {
+      return __all_sync(0xffffffffu, ptx::mbar_wait(bar, parity, lim, p.status, kWaitHint));
+    };
+    for (int j = 0; j < n_kt; ++j) {
+      if (!wait(ds_full, j & 1)) break;
+      if (!wait(&kv_full[j % DQ_STAGES], (j / DQ_STAGES) & 1)) break;
+      ptx::tc_fence_after();
+      if (issuer) {
+        const uint64_t dk = dk0 + static_cast<uint64_t>((j % DQ_STAGES) * (2 * KV_BYTES >> 4));
 #pragma unroll
         for (int kk = 0; kk < BKV / 16; ++kk)
-          ptx::tc_mma_f16_tmem_a(tdQ, tdS + kk * 8, ptx::smem_desc_sw128(sk + kk * 2048, 8192, 1024),
-                                 idQ, (j > 0 || kk > 0) ? 1u : 0u);
+          ptx::tc_mma_f16_tmem_a(tdQ, tdS + kk * 8, dk + kk * 128, idQ, (j > 0 || kk > 0) ? 1u : 0u);
         ptx::tc_commit(dq_done);
         ptx::tc_commit(&kv_empty[j % DQ_STAGES]);
       }
-      ptx::tc_commit(&done[1]);
-      ptx::mbar_wait(&done[1], 0, lim, p.status, kWaitHint);
+      __syncwarp();
     }
+    if (issuer) ptx::tc_commit(&done[1]);
+    __syncwarp();
+    ptx::mbar_wait(&done[1], 0, lim, p.status, kWaitHint);
   } else {
     const int q4 = warp & 3;
     const int hf = (warp - 2) >> 2;  // column half: keys [32 hf, 32 hf + 32) of a tile
@@ -801,50 +822,59 @@ __global__ void __maxnreg__(80) attn_bwd_dkdv_tc(const __grid_constant__ CUtenso
     // goes in once its accumulating product of tile i - 1 has read the
     // columns it overwrites; the accumulating product once the softmax warps
     // have stored P^T_i / dS^T_i.
-    if (lane == 0) {
-      const bool v_side = warp == 1;
-      constexpr uint32_t idS = ptx::idesc_bf16_f32(BK2, BQ2, false, false);
-      constexpr uint32_t idG = ptx::idesc_bf16_f32(BK2, HD, false, true);
-      const uint32_t skv = ptx::smem_u32(smem + (v_side ? KV_K_OFF : KV_V_OFF));
-      const uint32_t tscore = v_side ? tST : tdPT, tacc = v_side ? tdV : tdK;
-      uint64_t* score_full = v_side ? st_full : dpt_full;
-      uint64_t* acc_done = v_side ? dv_done : dk_done;
-      // K-major operand of the score product (Q_i or dO_i) and MN-major
-      // operand of the accumulating product (dO_i or Q_i)
-      const int score_off = v_side ? KV_Q_OFF : KV_O_OFF, acc_off = v_side ? KV_O_OFF : KV_Q_OFF;
-      const uint32_t se = ptx::smem_u32(smem + KV_E_OFF), sz = ptx::smem_u32(smem + KV_Z_OFF);
-      const uint32_t sx = ptx::smem_u32(smem + KV_X_OFF + (v_side ? 0 : X_BYTES));
-      bool ok = ptx::mbar_wait(kv_full, 0, lim, p.status, kWaitHint);
-      for (int i = 0; i < n_qt && ok; ++i) {
-        const int st = i % KV_STAGES;
-        if (i >= 1 && !ptx::mbar_wait(acc_done, (i - 1) & 1, lim, p.status, kWaitHint)) break;
-        if (!ptx::mbar_wait(&q_full[st], (i / KV_STAGES) & 1, lim, p.status, kWaitHint)) break;
-        ptx::tc_fence_after();
-        const uint32_t sb = ptx::smem_u32(smem + score_off + st * QO2_BYTES);
+    // (whole warp in the loop, one elected lane issuing: as in the forward)
+    const bool v_side = warp == 1;
+    const bool issuer = ptx::elect_one();
+    constexpr uint32_t idS = ptx::idesc_bf16_f32(BK2, BQ2, false, false);
+    constexpr uint32_t idG = ptx::idesc_bf16_f32(BK2, HD, false, true);
+    const uint32_t tscore = v_side ? tST : tdPT, tacc = v_side ? tdV : tdK;
+    uint64_t* score_full = v_side ? st_full : dpt_full;
+    uint64_t* acc_done = v_side ? dv_done : dk_done;
+    // K-major operand of the score product (Q_i or dO_i) and MN-major
+    // operand of the accumulating product (dO_i or Q_i)
+    const int score_off = v_side ? KV_Q_OFF : KV_O_OFF, acc_off = v_side ? KV_O_OFF : KV_Q_OFF;
+    const uint64_t dkv = ptx::smem_desc_sw128(ptx::smem_u32(smem + (v_side ? KV_K_OFF : KV_V_OFF)), 16, 1024);
+    const uint64_t dsc = ptx::smem_desc_sw128(ptx::smem_u32(smem + score_off), 16, 1024);
+    const uint64_t dac = ptx::smem_desc_sw128(ptx::smem_u32(smem + acc_off), 8192, 1024);
+    const uint32_t se = ptx::smem_u32(smem + KV_E_OFF), sz = ptx::smem_u32(smem + KV_Z_OFF);
+    const uint32_t sx = ptx::smem_u32(smem + KV_X_OFF + (v_side ? 0 : X_BYTES));
+    const uint64_t de = ptx::smem_desc_noswizzle(se, sz - se, 128);
+    auto wait = [&](uint64_t* bar, uint32_t parity) {
+      return __all_sync(0xffffffffu, ptx::mbar_wait(bar, parity, lim, p.status, kWaitHint));
+    };
+    bool ok = wait(kv_full, 0);
+    for (int i = 0; i < n_qt && ok; ++i) {
+      const int st = i % KV_STAGES;
+      if (i >= 1 && !wait(acc_done, (i - 1) & 1)) break;
+      if (!wait(&q_full[st], (i / KV_STAGES) & 1)) break;
+      ptx::tc_fence_after();
+      const uint64_t soff = static_cast<uint64_t>(st * (QO2_BYTES >> 4));
+      if (issuer) {
+        const uint32_t sxs = sx + st * 2 * X_BYTES;
+        const uint64_t dx = ptx::smem_desc_noswizzle(sxs, sz - sxs, 128);
 #pragma unroll
         for (int kk = 0; kk < HD / 16; ++kk)
-          ptx::tc_mma_f16(tscore, ptx::smem_desc_sw128(skv + kk * 32, 16, 1024),
-                          ptx::smem_desc_sw128(sb + kk * 32, 16, 1024), idS, kk > 0 ? 1u : 0u);
-        // the per-query term: E X^T
-        const uint32_t sxs = sx + st * 2 * X_BYTES;
-        ptx::tc_mma_f16(tscore, ptx::smem_desc_noswizzle(se, sz - se, 128),
-                        ptx::smem_desc_noswizzle(sxs, sz - sxs, 128), idS, 1u);
+          ptx::tc_mma_f16(tscore, dkv + kk * 2, dsc + soff + kk * 2, idS, kk > 0 ? 1u : 0u);
+        ptx::tc_mma_f16(tscore, de, dx, idS, 1u);  // the per-query term: E X^T
         ptx::tc_commit(score_full);
-        if (!ptx::mbar_wait(pds_full, i & 1, lim, p.status, kWaitHint)) break;
-        ptx::tc_fence_after();
-        const uint32_t sa = ptx::smem_u32(smem + acc_off + st * QO2_BYTES);
+      }
+      __syncwarp();
+      if (!wait(pds_full, i & 1)) break;
+      ptx::tc_fence_after();
+      if (issuer) {
 #pragma unroll
         for (int kk = 0; kk < BQ2 / 16; ++kk)  // queries 16 kk ..: half kk / 2, packed column 8 (kk % 2)
-          ptx::tc_mma_f16_tmem_a(tacc, tscore + (kk >> 1) * 32 + (kk & 1) * 8,
-                                 ptx::smem_desc_sw128(sa + kk * 2048, 8192, 1024), idG,
+          ptx::tc_mma_f16_tmem_a(tacc, tscore + (kk >> 1) * 32 + (kk & 1) * 8, dac + soff + kk * 128, idG,
                                  (i > 0 || kk > 0) ? 1u : 0u);
         ptx::tc_commit(acc_done);
         ptx::tc_commit(&q_empty[st]);
       }
-      uint64_t* fin = &done[v_side ? 0 : 1];
-      ptx::tc_commit(fin);
-      ptx::mbar_wait(fin, 0, lim, p.status, kWaitHint);
+      __syncwarp();
     }
+    uint64_t* fin = &done[v_side ? 0 : 1];
+    if (issuer) ptx::tc_commit(fin);
+    __syncwarp();
+    ptx::mbar_wait(fin, 0, lim, p.status, kWaitHint);
   } else {
     const int q4 = warp & 3;
     const int hf = (warp - 2) >> 2;  // column half: queries [32 hf, 32 hf + 32) of a tile
