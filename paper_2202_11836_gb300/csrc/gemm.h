@@ -1,5 +1,6 @@
 // Internal GEMM launchers (bf16 tensor-core and fp32 SIMT).
 #pragma once
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include "../../include/sky_ops.h"
@@ -32,6 +33,28 @@ sky_status launch_bf16(sky_gemm_form form, int M, int N, int K, const void* A, c
                        cudaStream_t stream, float* colsum = nullptr, float* colpart = nullptr,
                        size_t colpart_bytes = 0, int* deferred_rows = nullptr,
                        const float* resid = nullptr, const LnResid* ln = nullptr);
+// 2-D bf16 tensor map over a row-major [rows, cols] matrix, box {64, box_rows},
+// 128-byte swizzle; out-of-range elements read as zero.
+bool make_map(CUtensorMap* map, const void* base, int64_t rows, int64_t cols, int box_rows);
+
+// The cluster kernel (gemm_cluster.cu): tiles of 128 x bn (pair: 256 x bn on an
+// SM pair), each tile's k-blocks split over ks CTAs (pairs) of one cluster.
+struct ClusterPlan {
+  bool pair;
+  int bn, ks;
+};
+// Whether a product goes to the cluster kernel, and with which tiles.
+// may_split: an fp32 output without bias or residual; colpart: column sums per
+// 32 rows are wanted.
+bool plan_cluster(sky_gemm_form form, int M, int N, int K, bool may_split, bool colpart, int sms,
+                  ClusterPlan* out);
+// Arguments as launch_bf16, already checked there.
+sky_status launch_cluster(sky_gemm_form form, const ClusterPlan& pl, int M, int N, int K, const void* A,
+                          const void* B, void* C, bool out_f32, int epi, const void* bias,
+                          const void* aux, void* aux_out, int32_t* status, uint64_t timeout_ns,
+                          int skip_loads, cudaStream_t stream, float* colpart, const float* resid,
+                          const LnResid* ln);
+
 // Rows of column partials a bf16 GEMM with M rows writes (upper bound).
 int colpart_rows_max(int M);
 // out[n] = sum over r of part[r][n] in order r = 0, 1, ... (rowwise.cu).

@@ -635,8 +635,8 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   return fn;
 }
 
-// 2-D bf16 tensor map over a row-major [rows, cols] matrix, box {64, box_rows},
-// 128-byte swizzle; out-of-range elements read as zero.
+}  // namespace
+
 bool make_map(CUtensorMap* map, const void* base, int64_t rows, int64_t cols, int box_rows) {
   auto fn = encode_fn();
   if (!fn) return false;
@@ -649,6 +649,7 @@ bool make_map(CUtensorMap* map, const void* base, int64_t rows, int64_t cols, in
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+namespace {
 // Launches the product's work units on a persistent grid: one CTA per SM, or
 // for the pair variant one two-CTA cluster per SM pair, capped by how many
 // such clusters the device holds at once (a single wave).
@@ -782,6 +783,24 @@ sky_status launch_bf16(sky_gemm_form form, int M, int N, int K, const void* A, c
   const int sms = sm_count();
   SKY_CHECK(sms > 0, SKY_ERR_CUDA, "no CUDA device");
 
+  const bool may_split = out_f32 && epi == SKY_EPI_STORE && bias == nullptr && resid == nullptr;
+  if (!colsum) {  // small and mid-sized products: the cluster kernel
+    ClusterPlan pl;
+    if (plan_cluster(form, M, N, K, may_split, deferred_rows != nullptr, sms, &pl)) {
+      float* part = nullptr;
+      if (deferred_rows) {
+        SKY_CHECK(!out_f32, SKY_ERR_UNSUPPORTED, "fused column sum needs a bf16 output");
+        const int rows = ceil_div(M, pl.pair ? 2 * BM : BM) * (pl.pair ? 8 : 4);  // one per 32 rows
+        SKY_CHECK(colpart && colpart_bytes >= static_cast<size_t>(rows) * N * sizeof(float),
+                  SKY_ERR_INVALID_ARG, "GEMM column-sum workspace too small");
+        part = colpart;
+        *deferred_rows = rows;
+      }
+      return launch_cluster(form, pl, M, N, K, A, B, C, out_f32, epi, bias, aux, aux_out, status,
+                            g_timeout_ns, g_skip_loads, stream, part, resid, ln);
+    }
+  }
+
   CUtensorMap ta, tb;
   const bool a_mn = form == SKY_GEMM_XTW;
   const bool b_mn = form != SKY_GEMM_XWT;
@@ -800,7 +819,6 @@ sky_status launch_bf16(sky_gemm_form form, int M, int N, int K, const void* A, c
   // narrower tile's main loop, which reuses each A tile for fewer columns,
   // lost more than the fuller last wave gained: QKV at T = 8192 took 47.1
   // instead of 43.1 us.)
-  const bool may_split = out_f32 && epi == SKY_EPI_STORE && bias == nullptr && resid == nullptr;
   const bool narrow = pair && form == SKY_GEMM_XWT && epi == SKY_EPI_STORE && !may_split &&
                       !colsum && !deferred_rows && N % 192 == 0 &&
                       m_t * ceil_div(N, BN) < clusters && m_t * (N / 192) <= clusters;
