@@ -99,6 +99,8 @@ __global__ void attn_delta_bf16(const bf16* __restrict__ ctx, const bf16* __rest
 template <typename T>
 __global__ void attn_delta(const T* __restrict__ ctx, const T* __restrict__ dctx, int S, int H,
                            int A, int D, int64_t rows, float* __restrict__ delta) {
+  pdl_trigger();
+  pdl_wait();
   const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int l = threadIdx.x & 31;
   if (w >= rows * A) return;
@@ -116,116 +118,289 @@ __global__ void attn_delta(const T* __restrict__ ctx, const T* __restrict__ dctx
 }
 
 // ----------------------------------------------------------------- fp32 path
-// One warp per (query row, head, sequence); p[] staged in shared memory.
-__global__ void attn_fwd_f32(const float* __restrict__ qkv, const int32_t* __restrict__ lens,
-                             int S, int H, int A, int D, float* __restrict__ ctx,
-                             float* __restrict__ lse, int32_t* status) {
-  extern __shared__ float sp[];
-  const int wpb = blockDim.x >> 5, warp = threadIdx.x >> 5, l = threadIdx.x & 31;
-  const int64_t w = (int64_t)blockIdx.x * wpb + warp;
-  if (w >= (int64_t)S * A) return;
-  const int b = blockIdx.y;
-  const int i = (int)(w % S), a = (int)(w / S);
-  float* p = sp + warp * S;
-  int len = lens[b];
-  if (len < 1 || len > S) {
-    if (status && l == 0) atomicOr(status, kStatusBadLength);
-    len = len < 1 ? 1 : S;
+// Exact fp32 arithmetic, head dim up to 128.  A CTA of four warps owns 16 rows
+// of one (sequence, head) and walks the other side in tiles of 64 rows staged in
+// shared memory.  Half a warp owns two rows, so row maxima and sums are
+// shuffles among 16 lanes and a row's probabilities go to shared memory and
+// back within the half warp.  Score products: 2 rows x 4 columns a thread (six
+// 16-byte shared loads for 32 FMAs); accumulating products: 2 rows x 4 dims.
+// Short sequences and few heads make these latency-bound; a warp per row with
+// scalar loads took 116 us forward and 182 us backward at 4 x 101 tokens, 12
+// heads of 64.
+constexpr int FR = 16, FC = 64, F_THR = 128;  // rows of a CTA, columns of a tile
+constexpr int FP_LD = FC + 4;                 // row stride of the probability tiles
+
+// Rows [r0, r0 + n) of X (row stride ld, D values each) into s[n][LD]; rows from
+// `rows` on and columns from D on are zeros.  vec: D, ld and X allow 16-byte loads.
+__device__ __forceinline__ void stage_rows(float* s, int LD, const float* __restrict__ X, int64_t ld, int r0,
+                                           int n, int rows, int D, bool vec) {
+  const int g4 = (D + 3) / 4;
+  for (int i = threadIdx.x; i < n * g4; i += F_THR) {
+    const int r = i / g4, c = (i - r * g4) * 4;
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (r0 + r < rows) {
+      const float* p = X + static_cast<int64_t>(r0 + r) * ld + c;
+      if (vec) {
+        v = *reinterpret_cast<const float4*>(p);
+      } else {
+        v.x = p[0];
+        if (c + 1 < D) v.y = p[1];
+        if (c + 2 < D) v.z = p[2];
+        if (c + 3 < D) v.w = p[3];
+      }
+    }
+    *reinterpret_cast<float4*>(s + r * LD + c) = v;
   }
-  const int64_t rs = 3 * (int64_t)H;
-  const float* q = qkv + ((int64_t)b * S + i) * rs + a * D;
-  const float sc = 1.f / sqrtf((float)D);
-  float mx = -INFINITY;
-  for (int j = l; j < len; j += 32) {
-    const float* k = qkv + ((int64_t)b * S + j) * rs + H + a * D;
-    float s = 0.f;
-    for (int d = 0; d < D; ++d) s = fmaf(q[d], k[d], s);
-    s *= sc;
-    p[j] = s;
-    mx = fmaxf(mx, s);
+}
+// acc[i][c] = row (2 ty + i) . column row (tx + 16 c), over D (a multiple of 4 in shared memory)
+__device__ __forceinline__ void scores(const float* rows, const float* cols, int LD, int D, float (&acc)[2][4]) {
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) acc[i][c] = 0.f;
+  for (int d = 0; d < D; d += 4) {
+    float4 r[2], k[4];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) r[i] = *reinterpret_cast<const float4*>(rows + (2 * ty + i) * LD + d);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) k[c] = *reinterpret_cast<const float4*>(cols + (tx + 16 * c) * LD + d);
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        acc[i][c] = fmaf(r[i].w, k[c].w, fmaf(r[i].z, k[c].z, fmaf(r[i].y, k[c].y, fmaf(r[i].x, k[c].x, acc[i][c]))));
   }
-  mx = warp_max(mx);
-  float sum = 0.f;
-  for (int j = l; j < len; j += 32) {
-    const float e = expf(p[j] - mx);
-    p[j] = e;
-    sum += e;
+}
+// o[i][cc] += sum_j w[2 ty + i][j] cols[j][4 tx + 64 cc ..] over the tile's first n columns (n <= 64)
+template <int CC>
+__device__ __forceinline__ void accumulate(const float* w, const float* cols, int LD, int D, int n, float4 (&o)[2][CC]) {
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  for (int j = 0; j < n; j += 4) {
+    float4 p[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) p[i] = *reinterpret_cast<const float4*>(w + (2 * ty + i) * FP_LD + j);
+#pragma unroll
+    for (int cc = 0; cc < CC; ++cc) {
+      const int d = 4 * tx + 64 * cc;
+      if (d >= D) continue;
+      float4 v[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) v[e] = *reinterpret_cast<const float4*>(cols + (j + e) * LD + d);
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const float pe[4] = {p[i].x, p[i].y, p[i].z, p[i].w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          o[i][cc].x = fmaf(pe[e], v[e].x, o[i][cc].x);
+          o[i][cc].y = fmaf(pe[e], v[e].y, o[i][cc].y);
+          o[i][cc].z = fmaf(pe[e], v[e].z, o[i][cc].z);
+          o[i][cc].w = fmaf(pe[e], v[e].w, o[i][cc].w);
+        }
+      }
+    }
   }
-  sum = warp_sum(sum);
-  __syncwarp();
-  const float inv = 1.f / sum;
-  for (int d = l; d < D; d += 32) {
-    float acc = 0.f;
-    for (int j = 0; j < len; ++j)
-      acc = fmaf(p[j], qkv[((int64_t)b * S + j) * rs + 2 * H + a * D + d], acc);
-    ctx[((int64_t)b * S + i) * H + a * D + d] = acc * inv;
+}
+template <int CC>
+__device__ __forceinline__ void store_rows(float* X, int64_t ld, int r0, int rows, int D, bool vec, float scale0,
+                                           float scale1, const float4 (&o)[2][CC]) {
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const int r = r0 + 2 * ty + i;
+    if (r >= rows) continue;
+    const float sc = i ? scale1 : scale0;
+#pragma unroll
+    for (int cc = 0; cc < CC; ++cc) {
+      const int d = 4 * tx + 64 * cc;
+      if (d >= D) continue;
+      const float4 v = make_float4(o[i][cc].x * sc, o[i][cc].y * sc, o[i][cc].z * sc, o[i][cc].w * sc);
+      float* p = X + static_cast<int64_t>(r) * ld + d;
+      if (vec) {
+        *reinterpret_cast<float4*>(p) = v;
+      } else {
+        p[0] = v.x;
+        if (d + 1 < D) p[1] = v.y;
+        if (d + 2 < D) p[2] = v.z;
+        if (d + 3 < D) p[3] = v.w;
+      }
+    }
   }
-  if (l == 0) lse[((int64_t)b * A + a) * S + i] = (mx + logf(sum)) * 1.4426950408889634f;  // base 2
+}
+__device__ __forceinline__ float half_warp_max(float v) {
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+__device__ __forceinline__ float half_warp_sum(float v) {
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
 }
 
-// dQ rows (mode 0) or dK/dV rows (mode 1), one warp per row.
-__global__ void attn_bwd_f32(const float* __restrict__ qkv, const float* __restrict__ dctx,
-                             const float* __restrict__ lse, const float* __restrict__ delta,
-                             const int32_t* __restrict__ lens, int S, int H, int A, int D,
-                             float* __restrict__ dqkv, int mode) {
-  const int wpb = blockDim.x >> 5, warp = threadIdx.x >> 5, l = threadIdx.x & 31;
-  const int64_t w = (int64_t)blockIdx.x * wpb + warp;
-  if (w >= (int64_t)S * A) return;
-  const int b = blockIdx.y;
-  const int r = (int)(w % S), a = (int)(w / S);
+template <int CC>
+__global__ void __launch_bounds__(F_THR) attn_fwd_f32(const float* __restrict__ qkv, const int32_t* __restrict__ lens,
+                                                      int S, int H, int A, int D, int LD, bool vec,
+                                                      float* __restrict__ ctx, float* __restrict__ lse,
+                                                      int32_t* status) {
+  pdl_trigger();
+  pdl_wait();
+  extern __shared__ __align__(16) float sm[];
+  float *sq = sm, *sk = sq + FR * LD, *sv = sk + FC * LD, *sp = sv + FC * LD;
+  const int tiles = (S + FR - 1) / FR;
+  const int a = static_cast<int>(blockIdx.x) / tiles, q0 = (static_cast<int>(blockIdx.x) % tiles) * FR, b = blockIdx.y;
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  int len = lens[b];
+  if (len < 1 || len > S) {
+    if (status && threadIdx.x == 0) atomicOr(status, kStatusBadLength);
+    len = len < 1 ? 1 : S;
+  }
+  const int64_t rs = 3 * static_cast<int64_t>(H);
+  const float* q = qkv + static_cast<int64_t>(b) * S * rs + a * D;
+  const float sc = 1.f / sqrtf((float)D);
+  stage_rows(sq, LD, q, rs, q0, FR, S, D, vec);
+  float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};
+  float4 o[2][CC] = {};
+  for (int k0 = 0; k0 < len; k0 += FC) {
+    __syncthreads();
+    stage_rows(sk, LD, q + H, rs, k0, FC, len, D, vec);
+    stage_rows(sv, LD, q + 2 * H, rs, k0, FC, len, D, vec);
+    __syncthreads();
+    float s[2][4];
+    scores(sq, sk, LD, D, s);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      float mx = -INFINITY;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        s[i][c] = k0 + tx + 16 * c < len ? s[i][c] * sc : -INFINITY;
+        mx = fmaxf(mx, s[i][c]);
+      }
+      const float mn = fmaxf(m[i], half_warp_max(mx));
+      const float al = expf(m[i] - mn);  // 0 in the first tile
+      m[i] = mn;
+      float sum = 0.f;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const float e = expf(s[i][c] - mn);  // masked: 0
+        sp[(2 * ty + i) * FP_LD + tx + 16 * c] = e;
+        sum += e;
+      }
+      l[i] = l[i] * al + half_warp_sum(sum);
+#pragma unroll
+      for (int cc = 0; cc < CC; ++cc) {
+        o[i][cc].x *= al; o[i][cc].y *= al; o[i][cc].z *= al; o[i][cc].w *= al;
+      }
+    }
+    __syncwarp();
+    accumulate<CC>(sp, sv, LD, D, min(FC, len - k0), o);
+    __syncwarp();
+  }
+  store_rows<CC>(ctx + static_cast<int64_t>(b) * S * H + a * D, H, q0, S, D, vec, 1.f / l[0], 1.f / l[1], o);
+  if (tx == 0)
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+      if (q0 + 2 * ty + i < S)
+        lse[(static_cast<int64_t>(b) * A + a) * S + q0 + 2 * ty + i] = (m[i] + logf(l[i])) * 1.4426950408889634f;  // base 2
+}
+
+// dQ (even blockIdx.x): own rows are queries (Q, dO), columns keys (K, V).
+// dK, dV (odd): own rows are keys (K, V), columns queries (Q, dO).  Either way
+//   P = exp2(s log2(e)/sqrt(D) - lse_q),  dS = P (dp - delta_q),
+// s and dp the products of the first and second operands; dQ or dK = dS . first
+// operand of the columns / sqrt(D), dV = P . dO.
+template <int CC>
+__global__ void __launch_bounds__(F_THR) attn_bwd_f32(const float* __restrict__ qkv, const float* __restrict__ dctx,
+                                                      const float* __restrict__ lse, const float* __restrict__ delta,
+                                                      const int32_t* __restrict__ lens, int S, int H, int A, int D,
+                                                      int LD, bool vec, float* __restrict__ dqkv) {
+  pdl_trigger();
+  pdl_wait();
+  extern __shared__ __align__(16) float sm[];
+  float *r0s = sm, *r1s = r0s + FR * LD, *c0s = r1s + FR * LD, *c1s = c0s + FC * LD;
+  float *sds = c1s + FC * LD, *sp = sds + FR * FP_LD, *sl = sp + FR * FP_LD, *sd = sl + FC;
+  const int tiles = (S + FR - 1) / FR;
+  const bool keys = blockIdx.x & 1;  // own rows are keys
+  const int u = static_cast<int>(blockIdx.x) >> 1;
+  const int a = u / tiles, r0 = (u % tiles) * FR, b = blockIdx.y;
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   int len = lens[b];
   len = len < 1 ? 1 : (len > S ? S : len);
-  const int64_t rs = 3 * (int64_t)H;
-  const float sc = 1.f / sqrtf((float)D);
-  auto Q = [&](int i, int d) { return qkv[((int64_t)b * S + i) * rs + a * D + d]; };
-  auto K = [&](int j, int d) { return qkv[((int64_t)b * S + j) * rs + H + a * D + d]; };
-  auto V = [&](int j, int d) { return qkv[((int64_t)b * S + j) * rs + 2 * H + a * D + d]; };
-  auto dO = [&](int i, int d) { return dctx[((int64_t)b * S + i) * H + a * D + d]; };
-  const float* lse_b = lse + ((int64_t)b * A + a) * S;
-  const float* del_b = delta + ((int64_t)b * A + a) * S;
-  constexpr int MAXD = 4;  // D <= 128
-  float acc0[MAXD] = {}, acc1[MAXD] = {};
-  if (mode == 0) {
-    const int i = r;
-    for (int j = 0; j < len; ++j) {
-      float s = 0.f, dp = 0.f;
-      for (int d = l; d < D; d += 32) {
-        s = fmaf(Q(i, d), K(j, d), s);
-        dp = fmaf(dO(i, d), V(j, d), dp);
-      }
-      s = warp_sum(s);
-      dp = warp_sum(dp);
-      const float p = exp2f(fmaf(s, sc * 1.4426950408889634f, -lse_b[i]));
-      const float ds = p * (dp - del_b[i]);
-      for (int d = l, c = 0; d < D; d += 32, ++c) acc0[c] = fmaf(ds, K(j, d), acc0[c]);
+  const int64_t rs = 3 * static_cast<int64_t>(H);
+  const float* q = qkv + static_cast<int64_t>(b) * S * rs + a * D;
+  const float* dO = dctx + static_cast<int64_t>(b) * S * H + a * D;
+  float* out = dqkv + static_cast<int64_t>(b) * S * rs + a * D;
+  const float *lse_b = lse + (static_cast<int64_t>(b) * A + a) * S, *del_b = delta + (static_cast<int64_t>(b) * A + a) * S;
+  const float sc = 1.f / sqrtf((float)D), sl2 = sc * 1.4426950408889634f;
+  float4 o0[2][CC] = {}, o1[2][CC] = {};
+  const int cols = keys ? S : len;
+  if (!keys || r0 < len) {
+    stage_rows(r0s, LD, keys ? q + H : q, rs, r0, FR, S, D, vec);
+    if (keys) stage_rows(r1s, LD, q + 2 * H, rs, r0, FR, S, D, vec);
+    else stage_rows(r1s, LD, dO, H, r0, FR, S, D, vec);
+    float lr[2], dr[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int r = min(r0 + 2 * ty + i, S - 1);
+      lr[i] = lse_b[r];
+      dr[i] = del_b[r];
     }
-    for (int d = l, c = 0; d < D; d += 32, ++c)
-      dqkv[((int64_t)b * S + i) * rs + a * D + d] = acc0[c] * sc;
-  } else {
-    const int j = r;
-    if (j < len) {
-      for (int i = 0; i < S; ++i) {
-        float s = 0.f, dp = 0.f;
-        for (int d = l; d < D; d += 32) {
-          s = fmaf(Q(i, d), K(j, d), s);
-          dp = fmaf(dO(i, d), V(j, d), dp);
+    for (int c0 = 0; c0 < cols; c0 += FC) {
+      __syncthreads();
+      if (keys) {
+        stage_rows(c0s, LD, q, rs, c0, FC, S, D, vec);
+        stage_rows(c1s, LD, dO, H, c0, FC, S, D, vec);
+        if (threadIdx.x < FC) {
+          const int c = min(c0 + static_cast<int>(threadIdx.x), S - 1);
+          sl[threadIdx.x] = lse_b[c];
+          sd[threadIdx.x] = del_b[c];
         }
-        s = warp_sum(s);
-        dp = warp_sum(dp);
-        const float p = exp2f(fmaf(s, sc * 1.4426950408889634f, -lse_b[i]));
-        const float ds = p * (dp - del_b[i]);
-        for (int d = l, c = 0; d < D; d += 32, ++c) {
-          acc0[c] = fmaf(ds, Q(i, d), acc0[c]);   // dK
-          acc1[c] = fmaf(p, dO(i, d), acc1[c]);    // dV
-        }
+      } else {
+        stage_rows(c0s, LD, q + H, rs, c0, FC, len, D, vec);
+        stage_rows(c1s, LD, q + 2 * H, rs, c0, FC, len, D, vec);
       }
-    }
-    for (int d = l, c = 0; d < D; d += 32, ++c) {
-      dqkv[((int64_t)b * S + j) * rs + H + a * D + d] = acc0[c] * sc;
-      dqkv[((int64_t)b * S + j) * rs + 2 * H + a * D + d] = acc1[c];
+      __syncthreads();
+      float s[2][4], dp[2][4];
+      scores(r0s, c0s, LD, D, s);
+      scores(r1s, c1s, LD, D, dp);
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const int cl = tx + 16 * c;
+          const bool live = c0 + cl < cols && (!keys || r0 + 2 * ty + i < len);
+          const float p = live ? exp2f(fmaf(s[i][c], sl2, -(keys ? sl[cl] : lr[i]))) : 0.f;
+          sds[(2 * ty + i) * FP_LD + cl] = live ? p * (dp[i][c] - (keys ? sd[cl] : dr[i])) : 0.f;
+          if (keys) sp[(2 * ty + i) * FP_LD + cl] = p;
+        }
+      __syncwarp();
+      const int n = min(FC, cols - c0);
+      accumulate<CC>(sds, c0s, LD, D, n, o0);
+      if (keys) accumulate<CC>(sp, c1s, LD, D, n, o1);
+      __syncwarp();
     }
   }
+  store_rows<CC>(keys ? out + H : out, rs, r0, S, D, vec, sc, sc, o0);
+  if (keys) store_rows<CC>(out + 2 * H, rs, r0, S, D, vec, 1.f, 1.f, o1);
 }
+
+// Launch shape of the fp32 kernels: the shared row stride (four floats past the
+// head dim, so the 16 lanes of a score product read different banks) and the
+// bytes it makes, 16-row units of all heads, and whether the head rows allow
+// 16-byte accesses.
+constexpr int row_stride(int D) { return (D + 3) / 4 * 4 + 4; }
+constexpr int fwd_smem(int D) { return ((FR + 2 * FC) * row_stride(D) + FR * FP_LD) * 4; }
+constexpr int bwd_smem(int D) { return ((2 * FR + 2 * FC) * row_stride(D) + 2 * FR * FP_LD + 2 * FC) * 4; }
+struct F32Shape {
+  unsigned units;
+  int LD;
+  bool vec;
+  F32Shape(int S, int H, int A, int D, const void* x, const void* y, const void* z)
+      : units((unsigned)ceil_div(S, FR) * A), LD(row_stride(D)) {
+    const auto a16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
+    vec = D % 4 == 0 && H % 4 == 0 && a16(x) && a16(y) && a16(z);
+  }
+};
 
 }  // namespace attn
 
@@ -248,13 +423,19 @@ sky_status attention_fwd(const void* qkv, const int32_t* lens, int B, int S, int
     return attention_fwd_tc(qkv, lens, B, S, H, A, ctx, lse, status, 2000000000ull, stream);
   } else {
     SKY_CHECK(D <= 128, SKY_ERR_UNSUPPORTED, "fp32 attention needs head dim <= 128");
-    const int wpb = 4;
-    dim3 grid(ceil_div((int64_t)S * A, wpb), B);
-    const size_t smem = (size_t)wpb * S * sizeof(float);
-    SKY_CHECK(smem <= 48 * 1024, SKY_ERR_UNSUPPORTED, "fp32 attention: sequence too long");
-    attn::attn_fwd_f32<<<grid, wpb * 32, smem, stream>>>(static_cast<const float*>(qkv), lens, S,
-                                                         H, A, D, static_cast<float*>(ctx), lse,
-                                                         status);
+    SKY_CHECK(S <= 3072, SKY_ERR_UNSUPPORTED, "fp32 attention: sequence too long");
+    const attn::F32Shape f(S, H, A, D, qkv, ctx, nullptr);
+    static const cudaError_t attr[2] = {  // once, for the largest head dim of each
+        cudaFuncSetAttribute(attn::attn_fwd_f32<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, attn::fwd_smem(64)),
+        cudaFuncSetAttribute(attn::attn_fwd_f32<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, attn::fwd_smem(128))};
+    const auto go = [&](auto kern) {
+      return launch_pdl(kern, dim3(f.units, B), dim3(attn::F_THR), attn::fwd_smem(D), stream, 1,
+                        static_cast<const float*>(qkv), lens, S, H, A, D, f.LD, f.vec, static_cast<float*>(ctx), lse,
+                        status);
+    };
+    cudaError_t le = attr[D > 64];
+    if (le == cudaSuccess) le = D <= 64 ? go(attn::attn_fwd_f32<1>) : go(attn::attn_fwd_f32<2>);
+    if (le != cudaSuccess) return cuda_fail(le, "attention forward launch");
   }
   count_launches(1);
   const cudaError_t e = cudaGetLastError();
@@ -296,17 +477,23 @@ sky_status attention_bwd(const void* qkv, const void* ctx, const void* dctx, con
                             stream, colpart);
   } else {
     SKY_CHECK(D <= 128, SKY_ERR_UNSUPPORTED, "fp32 attention needs head dim <= 128");
-    attn::attn_delta<float><<<dblocks, 256, 0, stream>>>(static_cast<const float*>(ctx),
-                                                         static_cast<const float*>(dctx), S, H, A,
-                                                         D, rows, delta);
-    const int wpb = 4;
-    dim3 grid(ceil_div((int64_t)S * A, wpb), B);
-    for (int mode = 0; mode < 2; ++mode)
-      attn::attn_bwd_f32<<<grid, wpb * 32, 0, stream>>>(
-          static_cast<const float*>(qkv), static_cast<const float*>(dctx), lse, delta, lens, S, H,
-          A, D, static_cast<float*>(dqkv), mode);
+    cudaError_t le = launch_pdl(attn::attn_delta<float>, dim3(dblocks), dim3(256), 0, stream, 1,
+                                static_cast<const float*>(ctx), static_cast<const float*>(dctx), S, H, A, D, rows,
+                                delta);
+    const attn::F32Shape f(S, H, A, D, qkv, dctx, dqkv);
+    static const cudaError_t attr[2] = {
+        cudaFuncSetAttribute(attn::attn_bwd_f32<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, attn::bwd_smem(64)),
+        cudaFuncSetAttribute(attn::attn_bwd_f32<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, attn::bwd_smem(128))};
+    if (le == cudaSuccess) le = attr[D > 64];
+    const auto go = [&](auto kern) {
+      return launch_pdl(kern, dim3(2 * f.units, B), dim3(attn::F_THR), attn::bwd_smem(D), stream, 1,
+                        static_cast<const float*>(qkv), static_cast<const float*>(dctx), lse,
+                        static_cast<const float*>(delta), lens, S, H, A, D, f.LD, f.vec, static_cast<float*>(dqkv));
+    };
+    if (le == cudaSuccess) le = D <= 64 ? go(attn::attn_bwd_f32<1>) : go(attn::attn_bwd_f32<2>);
+    if (le != cudaSuccess) return cuda_fail(le, "attention backward launch");
   }
-  count_launches(3);
+  count_launches(2);
   const cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? SKY_OK : cuda_fail(e, "attention backward launch");
 }
