@@ -33,8 +33,8 @@ template <int NV>
 __global__ void attn_delta_bf16(const bf16* __restrict__ ctx, const bf16* __restrict__ dctx, int S,
                                 int H, int A, int64_t rows, float* __restrict__ delta,
                                 const float* __restrict__ lse, uint4* __restrict__ xtab) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const int64_t row = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int l = threadIdx.x & 31;
   if (row >= rows) return;
@@ -99,8 +99,8 @@ __global__ void attn_delta_bf16(const bf16* __restrict__ ctx, const bf16* __rest
 template <typename T>
 __global__ void attn_delta(const T* __restrict__ ctx, const T* __restrict__ dctx, int S, int H,
                            int A, int D, int64_t rows, float* __restrict__ delta) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int l = threadIdx.x & 31;
   if (w >= rows * A) return;
@@ -243,7 +243,6 @@ __global__ void __launch_bounds__(F_THR) attn_fwd_f32(const float* __restrict__ 
                                                       int S, int H, int A, int D, int LD, bool vec,
                                                       float* __restrict__ ctx, float* __restrict__ lse,
                                                       int32_t* status) {
-  pdl_trigger();
   pdl_wait();
   extern __shared__ __align__(16) float sm[];
   float *sq = sm, *sk = sq + FR * LD, *sv = sk + FC * LD, *sp = sv + FC * LD;
@@ -296,6 +295,7 @@ __global__ void __launch_bounds__(F_THR) attn_fwd_f32(const float* __restrict__ 
     accumulate<CC>(sp, sv, LD, D, min(FC, len - k0), o);
     __syncwarp();
   }
+  pdl_trigger();
   store_rows<CC>(ctx + static_cast<int64_t>(b) * S * H + a * D, H, q0, S, D, vec, 1.f / l[0], 1.f / l[1], o);
   if (tx == 0)
 #pragma unroll
@@ -314,7 +314,6 @@ __global__ void __launch_bounds__(F_THR) attn_bwd_f32(const float* __restrict__ 
                                                       const float* __restrict__ lse, const float* __restrict__ delta,
                                                       const int32_t* __restrict__ lens, int S, int H, int A, int D,
                                                       int LD, bool vec, float* __restrict__ dqkv) {
-  pdl_trigger();
   pdl_wait();
   extern __shared__ __align__(16) float sm[];
   float *r0s = sm, *r1s = r0s + FR * LD, *c0s = r1s + FR * LD, *c1s = c0s + FC * LD;
@@ -380,6 +379,7 @@ __global__ void __launch_bounds__(F_THR) attn_bwd_f32(const float* __restrict__ 
       __syncwarp();
     }
   }
+  pdl_trigger();
   store_rows<CC>(keys ? out + H : out, rs, r0, S, D, vec, sc, sc, o0);
   if (keys) store_rows<CC>(out + 2 * H, rs, r0, S, D, vec, 1.f, 1.f, o1);
 }

@@ -101,7 +101,6 @@ __global__ void __launch_bounds__(C_THREADS, 2)
   uint64_t* tfull = empty + C_MAX_STAGES;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tfull + 1);
 
-  pdl_trigger();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int bn = p.bn;
   const int b_rows = PAIR ? bn >> 1 : bn;  // tile columns whose B operand this CTA loads
@@ -280,6 +279,7 @@ __global__ void __launch_bounds__(C_THREADS, 2)
       }
     }
   }
+  pdl_trigger();  // behind the main loop: see common.cuh
   ptx::tc_fence_before();
   __syncwarp();
   if (one_cta) __syncthreads();

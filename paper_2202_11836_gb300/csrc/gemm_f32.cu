@@ -101,7 +101,6 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
 template <bool AK, bool BK, bool VEC>
 __global__ void __launch_bounds__(F_THREADS) gemm_f32_kernel(const F32Params p) {
   __shared__ __align__(16) float sm[2][2][TK * 64];  // [buffer][A, B]; later the 64 x 64 partial tile
-  pdl_trigger();
   pdl_wait();
   const int t = threadIdx.x;
   const int split = static_cast<int>(blockIdx.x) % p.ks, tile = static_cast<int>(blockIdx.x) / p.ks;
@@ -139,6 +138,7 @@ __global__ void __launch_bounds__(F_THREADS) gemm_f32_kernel(const F32Params p) 
       }
     }
   }
+  pdl_trigger();
   auto finish = [&](int m, int n, float v) {
     if (m >= p.M || n >= p.N) return;
     const int64_t off = static_cast<int64_t>(m) * p.N + n;

@@ -157,7 +157,6 @@ __global__ void __launch_bounds__(Shape<EPI, PAIR, TBN>::THREADS, 1)
   uint64_t* done = tempty + 2;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
 
-  pdl_trigger();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = PAIR ? ptx::cluster_ctarank() : 0u;
   const bool leader = rank == 0;
@@ -569,6 +568,7 @@ __global__ void __launch_bounds__(Shape<EPI, PAIR, TBN>::THREADS, 1)
     }
   }
 
+  pdl_trigger();  // behind the last tile: see common.cuh
   ptx::tc_fence_before();
   __syncwarp();
   if constexpr (PAIR) ptx::cluster_sync();  // no CTA leaves while its peer may still signal it
@@ -587,8 +587,8 @@ __global__ void __launch_bounds__(Shape<EPI, PAIR, TBN>::THREADS, 1)
 template <int SPLITS>
 __global__ void splitk_reduce_kernel(const float* __restrict__ ws, int splits, int64_t n,
                                      float* __restrict__ out) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const int64_t n4 = n / 4;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n4;
        i += (int64_t)gridDim.x * blockDim.x) {

@@ -54,8 +54,8 @@ __global__ void __launch_bounds__(LN_WARPS * 32) ln_fwd_kernel(
     const T* __restrict__ beta, int rows, int H, float eps, float* u_out,
     float* __restrict__ y32, T* __restrict__ yT, float* __restrict__ mean_out,
     float* __restrict__ rstd_out) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const int lane = threadIdx.x & 31;
   const int warp = blockIdx.x * LN_WARPS + (threadIdx.x >> 5);
   const int nwarps = gridDim.x * LN_WARPS;
@@ -128,8 +128,8 @@ __global__ void __launch_bounds__(LN_WARPS * 32) ln_bwd_kernel(
     const T* __restrict__ gamma,
     const float* __restrict__ mean, const float* __restrict__ rstd, int rows, int H,
     float* __restrict__ du32, T* __restrict__ duT, float* __restrict__ part) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   extern __shared__ float red[];  // [LN_WARPS][3][H]
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int warp = blockIdx.x * LN_WARPS + wib;
@@ -211,8 +211,8 @@ __global__ void __launch_bounds__(LN_WARPS * 32) ln_bwd_kernel(
 template <typename T>
 __global__ void add_kernel(const float* __restrict__ a, const float* __restrict__ b, int64_t n,
                            T* __restrict__ out) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
     out[i] = from_f32<T>(a[i] + b[i]);
@@ -220,8 +220,8 @@ __global__ void add_kernel(const float* __restrict__ a, const float* __restrict_
 
 __global__ void to_bf16_kernel(const float* __restrict__ x, int64_t n,
                                __nv_bfloat16* __restrict__ out) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
     out[i] = __float2bfloat16_rn(x[i]);
@@ -229,8 +229,8 @@ __global__ void to_bf16_kernel(const float* __restrict__ x, int64_t n,
 
 template <typename T>
 __global__ void to_f32_kernel(const T* __restrict__ x, int64_t n, float* __restrict__ out) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
     out[i] = to_f32(x[i]);
@@ -282,8 +282,8 @@ __global__ void __launch_bounds__(32 * (SB_WARPS + 1), 1) ln_bwd_stream_kernel(
     const __nv_bfloat16* __restrict__ gamma, const float* __restrict__ mean,
     const float* __restrict__ rstd, int rows, int H, float* __restrict__ du32,
     __nv_bfloat16* __restrict__ duT, float* __restrict__ part, int32_t* status) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   extern __shared__ uint8_t sm_raw[];
   uint8_t* sm = sm_raw + ((128 - (ptx::smem_u32(sm_raw) & 127)) & 127);
   uint64_t* full = reinterpret_cast<uint64_t*>(sm + SB_RING * SB_ROW_BYTES);
@@ -422,8 +422,8 @@ constexpr int RP_WARPS = 16;
 __global__ void __launch_bounds__(RP_WARPS * 32) reduce_partials(const float* __restrict__ part,
                                                                  int nblk, int N, float* out0,
                                                                  float* out1, float* out2) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   __shared__ float red[RP_WARPS][33];
   const int k = blockIdx.y;
   float* out = k == 0 ? out0 : (k == 1 ? out1 : out2);
@@ -460,8 +460,8 @@ __global__ void __launch_bounds__(RP_WARPS * 32) reduce_partials(const float* __
 // computes segs[y].out[n] = sum_b segs[y].part[b][n] over its rows, exactly
 // as reduce_partials does (so the same partials give the same bits).
 __global__ void __launch_bounds__(RP_WARPS * 32) reduce_segments(const ColSegments segs) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   __shared__ float red[RP_WARPS][33];
   const ColSegment& sg = segs.seg[blockIdx.y];
   const int N = sg.cols, nblk = sg.rows;
@@ -500,8 +500,8 @@ __global__ void __launch_bounds__(RP_WARPS * 32) reduce_segments(const ColSegmen
 template <typename T>
 __global__ void __launch_bounds__(256) colsum_partial(const T* __restrict__ x, int rows, int N,
                                                       float* __restrict__ part) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   __shared__ float red[8][256];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int col = blockIdx.x * 256 + lane * 8;
@@ -556,11 +556,10 @@ __global__ void gelu_bwd_kernel(const T* __restrict__ dg, const T* __restrict__ 
     dh[i] = from_f32<T>(to_f32(dg[i]) * gelu_grad_f(to_f32(hpre[i])));
 }
 
-int ln_blocks(int rows) {
-  const int want = ceil_div(rows, LN_WARPS);
-  const int cap = 4 * (sm_count() > 0 ? sm_count() : 148);
-  return want < cap ? want : cap;
-}
+// A warp a row, every CTA launched: capped at four CTAs an SM (one wave, warps
+// taking one or two rows) 16384 rows of 1024 with a residual took 9 us longer
+// whenever the kernel before still held part of an SM.
+int ln_blocks(int rows) { return ceil_div(rows, LN_WARPS); }
 int stream_blocks() { return sm_count() > 0 ? sm_count() : 148; }
 // Backward CTAs also write column partials, so fewer, longer-lived CTAs.
 int ln_bwd_blocks(int rows) {
