@@ -38,11 +38,15 @@ def run_gemm(form, M, N, K, a, b, out_dtype, epi=L.SKY_EPI_STORE, bias=None, aux
 
 # (M, N, K) in (tiles of 128 x 64, k-blocks of 64): one tile and one k-block; a
 # ragged tail everywhere; two, three and six splits with uneven shares (the
-# k-blocks do not divide); 152 / 153 and 304 / 305 tiles; a pair with two splits
-# and a ragged last row tile; 128-wide weight-gradient tiles
+# k-blocks do not divide), 19 / 20 and 38 / 39 tiles of them; 76 / 77, 152 / 153
+# and 304 / 305 tiles; pairs with two splits and a ragged last row tile;
+# 128-wide weight-gradient tiles
 SHAPES = [(1, 8, 8), (129, 72, 200), (70, 136, 13 * 64 + 8), (257, 200, 17 * 64), (61, 72, 35 * 64 + 16),
+          (40, 19 * 64, 14 * 64), (40, 20 * 64, 14 * 64), (200, 19 * 64, 13 * 64), (200, 20 * 64, 13 * 64),
+          (128, 76 * 64, 136), (128, 77 * 64, 24 * 64), (260, 1664, 25 * 64 + 8),
           (128, 152 * 64, 136), (128, 153 * 64, 72), (2 * 128, 152 * 64, 64), (129, 19520, 64),
-          (1100, 1152, 35 * 64), (300, 1200, 33 * 64 + 24), (1000, 2496, 72)]
+          (1100, 1152, 35 * 64), (1100, 1152, 41 * 64), (300, 1200, 33 * 64 + 24), (1000, 2496, 72),
+          (130, 160, 97 * 64)]
 
 
 @pytest.mark.parametrize("form", [L.SKY_GEMM_XWT, L.SKY_GEMM_XW, L.SKY_GEMM_XTW])
