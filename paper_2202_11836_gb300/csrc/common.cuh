@@ -81,6 +81,59 @@ __device__ __forceinline__ void gelu_and_grad_as(float h, float& g, float& gp) {
   gp = fmaf(h * 0.3989422804014327f, E, Phi);
 }
 
+// Packed pairs of fp32: one instruction, each half rounded as its scalar form.
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(uint64_t v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+
+// gelu_and_grad_as of two values, in packed arithmetic where it pairs up, with
+// the sign handled without branches: with q = Phi(-|h|),
+//   GELU(h) = max(h, 0) - |h| q,   Phi(h) = 1/2 + sign(h) (1/2 - q).
+__device__ __forceinline__ void gelu_and_grad_as2(float h0, float h1, float2& g, float2& gp) {
+  const auto both = [](float v) { return pack2(v, v); };
+  float t0, t1, e0, e1;
+  const float den0 = fmaf(fabsf(h0), 0.47047f * 0.70710678118654752f, 1.f);
+  const float den1 = fmaf(fabsf(h1), 0.47047f * 0.70710678118654752f, 1.f);
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t0) : "f"(den0));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t1) : "f"(den1));
+  const uint64_t h = pack2(h0, h1), t = pack2(t0, t1);
+  const float2 x = unpack2(mul2(mul2(h, both(-0.72134752044448170f)), h));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e0) : "f"(x.x));  // exp(-h^2/2)
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e1) : "f"(x.y));
+  const uint64_t E = pack2(e0, e1);
+  uint64_t poly = fma2(t, both(0.5f * 0.7478556f), both(0.5f * -0.0958798f));
+  poly = mul2(t, fma2(t, poly, both(0.5f * 0.3480242f)));
+  const uint64_t q = mul2(poly, E);
+  const float2 qq = unpack2(q);
+  g.x = fmaf(-fabsf(h0), qq.x, fmaxf(h0, 0.f));
+  g.y = fmaf(-fabsf(h1), qq.y, fmaxf(h1, 0.f));
+  const uint64_t s = pack2(copysignf(1.f, h0), copysignf(1.f, h1));
+  const uint64_t Phi = fma2(s, fma2(q, both(-1.f), both(0.5f)), both(0.5f));
+  gp = unpack2(fma2(mul2(h, both(0.3989422804014327f)), E, Phi));
+}
+
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);

@@ -86,18 +86,6 @@ __device__ __forceinline__ float ld_cluster_f32(uint32_t addr) {
   return v;
 }
 
-// Two fp32 FMAs in one instruction (each rounded as fmaf).
-__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-
 template <bool AK, bool BK, bool VEC>
 __global__ void __launch_bounds__(F_THREADS) gemm_f32_kernel(const F32Params p) {
   __shared__ __align__(16) float sm[2][2][TK * 64];  // [buffer][A, B]; later the 64 x 64 partial tile

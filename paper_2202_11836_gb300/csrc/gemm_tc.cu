@@ -10,11 +10,12 @@
 //               K=16) into a TMEM accumulator; two accumulators (512 TMEM
 //               columns) let the epilogue of one tile overlap the next,
 //   warps 2..9  epilogue (two warps per TMEM lane quarter, one per half of
-//               the tile's columns; 2..17 and a quarter of the columns each
-//               for bias + GELU): tcgen05.ld of the accumulator, a
+//               the tile's columns): tcgen05.ld of the accumulator, a
 //               transpose through shared memory so stores coalesce, fused
-//               bias / GELU, store to global memory.  The forward GELU
-//               epilogue also stores GELU'(z) (fp16); the backward epilogue
+//               bias / residual, store to global memory.  The forward GELU
+//               epilogue (warps 2..17, a quarter of the columns each) computes
+//               GELU(z) and GELU'(z) (fp16) on the accumulator rows and
+//               writes both by TMA; the backward epilogue
 //               multiplies by it, loading it for the whole tile before the
 //               accumulator is waited on so its latency hides under the
 //               tile's main loop.
@@ -58,23 +59,25 @@ constexpr int PAIR_STAGES = 5;
 constexpr int PAIR_STAGES_WIDE = 6;  // all but the GELU' data-gradient epilogue
 
 // Launch shape per instantiation: epilogue warps (a multiple of 4, one group
-// per TMEM lane quarter), epilogue chunk width, ring stages and shared memory.
-// The bias+GELU epilogue is bound by its own math: it runs 16 warps (four per
-// lane quarter, 64 columns each) on 16-column chunks, which keeps it at about
-// 100 registers a thread (576 threads leave 112).
+// per TMEM lane quarter), ring stages and shared memory.  The bias+GELU epilogue
+// is bound by its own arithmetic: it runs 16 warps (four per lane quarter, 64
+// columns each), and stages its two 16-bit outputs for TMA (4 KiB a warp), which
+// takes one stage off the ring.
 // TBN: the tile's width (256, or 192 for K-major B operands whose output
 // width fills the SM pairs better in 192-wide tiles).
 template <int EPI, bool PAIR, int TBN = BN>
 struct Shape {
   static constexpr int EW = EPI == SKY_EPI_BIAS_GELU ? 16 : NUM_EPI_WARPS;
-  static constexpr int CW = EW == 16 ? 16 : 32;              // epilogue chunk width (columns)
+  static constexpr bool GELU = EPI == SKY_EPI_BIAS_GELU;
   static constexpr int THREADS = 64 + 32 * EW;
-  static constexpr int NST = PAIR ? (EPI == SKY_EPI_GELU_BWD ? PAIR_STAGES : PAIR_STAGES_WIDE) : STAGES;
+  static constexpr int NST = PAIR ? (EPI == SKY_EPI_GELU_BWD || GELU ? PAIR_STAGES : PAIR_STAGES_WIDE)
+                                  : (GELU ? STAGES - 1 : STAGES);
   static constexpr int SBYTES = A_BYTES + (PAIR ? TBN / 2 : TBN) * BK * 2;
   // two fp32 accumulators of 128 x TBN, in a power-of-two TMEM allocation
   static constexpr int TMEM_ALLOC = 2 * TBN <= 256 ? 256 : 512;
-  static constexpr int EPI_OFF = NST * SBYTES;               // per epilogue warp: 32 x CW fp32 staging
-  static constexpr int BAR_OFF = EPI_OFF + EW * 32 * CW * 4;
+  static constexpr int EPI_OFF = NST * SBYTES;  // per epilogue warp: 32 x 32 staging, fp32 or two 16-bit outputs
+  static constexpr int BIAS_OFF = EPI_OFF + EW * 4096;       // bias+GELU: the tile's bias, one copy per accumulator
+  static constexpr int BAR_OFF = BIAS_OFF + (GELU ? 2 * TBN * 2 : 0);
   static constexpr int SMEM = BAR_OFF + 256 /*barriers*/ + 1024 /*alignment slack*/;
   static_assert(SMEM <= 232448, "shared memory per CTA");
 };
@@ -139,7 +142,8 @@ __device__ __forceinline__ bool work_item(const Sched& sched, int it, Work& w) {
 template <bool A_MN, bool B_MN, int EPI, bool OUT_F32, bool PAIR, int TBN = BN>
 __global__ void __launch_bounds__(Shape<EPI, PAIR, TBN>::THREADS, 1)
     gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA,
-                   const __grid_constant__ CUtensorMap tmB, const Params p) {
+                   const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmC,
+                   const __grid_constant__ CUtensorMap tmX, const Params p) {
   using SH = Shape<EPI, PAIR, TBN>;
   constexpr int NST = SH::NST;
   constexpr int SBYTES = SH::SBYTES;
@@ -330,7 +334,7 @@ __global__ void __launch_bounds__(Shape<EPI, PAIR, TBN>::THREADS, 1)
     // row's 32 columns, then the fused epilogue and coalesced stores.
     constexpr int HALF = TBN / (EW / 4), CHUNKS = HALF / 32;  // columns of a warp, 32-column chunks
     const int q = warp & 3, hf = (warp - 2) >> 2;
-    float* stage = reinterpret_cast<float*>(smem + SH::EPI_OFF) + (warp - 2) * 32 * SH::CW;
+    float* stage = reinterpret_cast<float*>(smem + SH::EPI_OFF) + (warp - 2) * 1024;
     const int c4 = lane & 7;          // this lane's 4-column group in a chunk
     const int rsub = lane >> 3;       // row within each group of 4 rows
     int acc = 0;
@@ -391,6 +395,14 @@ __global__ void __launch_bounds__(Shape<EPI, PAIR, TBN>::THREADS, 1)
           }
         }
       }
+      if constexpr (EPI == SKY_EPI_BIAS_GELU) {
+        // this warp's 64 columns of bias (the four warps of a column group write the
+        // same values; a copy per accumulator, as a warp may be one tile ahead)
+        const int col = n0 + 2 * lane;
+        const uint32_t b2 = col < p.N ? *reinterpret_cast<const uint32_t*>(p.bias + col) : 0u;
+        *reinterpret_cast<uint32_t*>(smem + SH::BIAS_OFF + (acc * TBN + hf * HALF + 2 * lane) * 2) = b2;
+        __syncwarp();
+      }
       if (!ptx::mbar_wait(&tfull[acc], aphase, lim, p.status, kSleepNs)) break;
       ptx::tc_fence_after();
       const uint32_t taddr = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + acc * TBN + hf * HALF;
@@ -398,51 +410,57 @@ __global__ void __launch_bounds__(Shape<EPI, PAIR, TBN>::THREADS, 1)
                                   static_cast<int64_t>(w.split) * p.M * static_cast<int64_t>(p.N)
                             : nullptr;
       if constexpr (EPI == SKY_EPI_BIAS_GELU) {
-        // CW-column chunks: LPR lanes cover a row's CW columns, RPI rows per step
-        constexpr int CW = SH::CW, LPR = CW / 4, RPI = 32 / LPR, NI = 32 / RPI;
-        const int g4 = lane % LPR, grs = lane / LPR;
-        auto swz = [](int row) { return CW == 32 ? (row & 7) : ((row >> 1) & 3); };
-#pragma unroll 1
-        for (int c = 0; c < HALF; c += CW) {
-          uint32_t r[CW];
-          __syncwarp();
-          if constexpr (CW == 16) ptx::tmem_ld_32x32b_x16(taddr + c, *reinterpret_cast<uint32_t(*)[16]>(r));
-          else ptx::tmem_ld_32x32b_x32(taddr + c, *reinterpret_cast<uint32_t(*)[32]>(r));
+        // Thread = row: 32 columns at a time from TMEM, bias, GELU and GELU' in
+        // packed arithmetic, and both outputs as 16-bit rows of 64 bytes
+        // (64-byte-swizzled) into the warp's staging, which TMA writes out while
+        // the next chunk is computed.  The same tile transposed through fp32
+        // staging and stored 8 bytes a lane took 7 us, more than a K = 1024 main
+        // loop; this takes 4.  4096 x 3072 x 768: 25.3 -> 23.7 us, FFN forward block on
+        // 4999 rows, large width, 97.2 -> 94.8.
+        uint8_t* sg = reinterpret_cast<uint8_t*>(stage);
+        const uint32_t sbias = ptx::smem_u32(smem + SH::BIAS_OFF) + (acc * TBN + hf * HALF) * 2;
+        const uint32_t srow = ptx::smem_u32(sg) + lane * 64;
+#pragma unroll
+        for (int c = 0; c < HALF; c += 32) {
+          uint32_t r[32];
+          ptx::tmem_ld_32x32b_x32(taddr + c, r);
           ptx::tmem_ld_wait();
-          if (n0 + c >= p.N) continue;  // warp-uniform
+          if (c + 32 >= HALF) release_acc();  // the accumulator is in registers
+          if (n0 + c >= p.N) continue;        // warp-uniform
+          uint32_t og[16], ox[16];
 #pragma unroll
-          for (int j = 0; j < CW / 4; ++j)
-            *reinterpret_cast<float4*>(stage + lane * CW + ((j ^ swz(lane)) << 2)) =
-                make_float4(__uint_as_float(r[4 * j]), __uint_as_float(r[4 * j + 1]),
-                            __uint_as_float(r[4 * j + 2]), __uint_as_float(r[4 * j + 3]));
-          __syncwarp();
-          const int col = n0 + c + 4 * g4;
-          if (col >= p.N) continue;
-          const uint2 braw = *reinterpret_cast<const uint2*>(p.bias + col);
-          const __nv_bfloat162* bh = reinterpret_cast<const __nv_bfloat162*>(&braw);
-          const float2 bf0 = __bfloat1622float2(bh[0]), bf1 = __bfloat1622float2(bh[1]);
-          const float b4[4] = {bf0.x, bf0.y, bf1.x, bf1.y};
+          for (int j = 0; j < 32; j += 8) {
+            uint32_t bb[4];  // the bias of 8 columns, the same for every row
+            ptx::ld_shared_v4(sbias + (c + j) * 2, bb);
 #pragma unroll
-          for (int i = 0; i < NI; ++i) {
-            const int rl = RPI * i + grs;
-            const float4 t4 = *reinterpret_cast<const float4*>(stage + rl * CW + ((g4 ^ swz(rl)) << 2));
-            float z[4] = {t4.x + b4[0], t4.y + b4[1], t4.z + b4[2], t4.w + b4[3]}, gp[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) gelu_and_grad_as(z[j], z[j], gp[j]);
-            const int row = m0 + q * 32 + rl;
-            if (row < p.M) {
-              const int64_t off = static_cast<int64_t>(row) * p.N + col;
-              const __half2 h0 = __floats2half2_rn(gp[0], gp[1]), h1 = __floats2half2_rn(gp[2], gp[3]);
-              *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(p.C) + off) =
-                  make_uint2(ptx::pack_bf16(z[0], z[1]), ptx::pack_bf16(z[2], z[3]));
-              // GELU'(z) is read again only by the backward pass: a streaming
-              // store keeps it from displacing G, which FFN2 reads next, in L2
-              __stcs(reinterpret_cast<uint2*>(p.aux_out + off),
-                     make_uint2(*reinterpret_cast<const uint32_t*>(&h0),
-                                *reinterpret_cast<const uint32_t*>(&h1)));
+            for (int e = 0; e < 4; ++e) {
+              const float2 z = unpack2(add2(
+                  pack2(__uint_as_float(r[j + 2 * e]), __uint_as_float(r[j + 2 * e + 1])),
+                  pack2(__uint_as_float(bb[e] << 16), __uint_as_float(bb[e] & 0xffff0000u))));
+              float2 g, gp;
+              gelu_and_grad_as2(z.x, z.y, g, gp);
+              og[j / 2 + e] = ptx::pack_bf16(g.x, g.y);
+              const __half2 h = __floats2half2_rn(gp.x, gp.y);
+              ox[j / 2 + e] = *reinterpret_cast<const uint32_t*>(&h);
             }
           }
+          if (lane == 0) ptx::bulk_wait_group_read0();  // the chunk before has left the staging
+          __syncwarp();
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const uint32_t at = srow + ((j ^ ((lane >> 1) & 3)) << 4);
+            ptx::st_shared_v4(at, og[4 * j], og[4 * j + 1], og[4 * j + 2], og[4 * j + 3]);
+            ptx::st_shared_v4(at + 2048, ox[4 * j], ox[4 * j + 1], ox[4 * j + 2], ox[4 * j + 3]);
+          }
+          ptx::fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0 && m0 + q * 32 < p.M) {
+            ptx::tma_store_2d(&tmC, sg, n0 + c, m0 + q * 32);
+            ptx::tma_store_2d(&tmX, sg + 2048, n0 + c, m0 + q * 32);
+            ptx::bulk_commit_group();
+          }
         }
+        continue;  // (released above)
       } else
 #pragma unroll CHUNKS
       for (int cc = 0; cc < CHUNKS; ++cc) {
@@ -517,18 +535,6 @@ __global__ void __launch_bounds__(Shape<EPI, PAIR, TBN>::THREADS, 1)
             v[i][0] *= f0.x; v[i][1] *= f0.y; v[i][2] *= f1.x; v[i][3] *= f1.y;
           }
         }
-        uint2 gq[EPI == SKY_EPI_BIAS_GELU ? 8 : 1];
-        if constexpr (EPI == SKY_EPI_BIAS_GELU) {
-#pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            float gp[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) gelu_and_grad_as(v[i][j], v[i][j], gp[j]);
-            const __half2 h0 = __floats2half2_rn(gp[0], gp[1]), h1 = __floats2half2_rn(gp[2], gp[3]);
-            gq[i] = make_uint2(*reinterpret_cast<const uint32_t*>(&h0),
-                               *reinterpret_cast<const uint32_t*>(&h1));
-          }
-        }
         if (p.colpart) {
           // column sums of this warp's 32 rows (the bias gradient), fixed order
           float cs[4] = {0.f, 0.f, 0.f, 0.f};
@@ -558,14 +564,13 @@ __global__ void __launch_bounds__(Shape<EPI, PAIR, TBN>::THREADS, 1)
             } else {
               *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(p.C) + off) =
                   make_uint2(ptx::pack_bf16(v[i][0], v[i][1]), ptx::pack_bf16(v[i][2], v[i][3]));
-              if constexpr (EPI == SKY_EPI_BIAS_GELU)
-                __stcs(reinterpret_cast<uint2*>(p.aux_out + off), gq[i]);
             }
           }
         }
       }
       release_acc();
     }
+    if (EPI == SKY_EPI_BIAS_GELU && lane == 0) ptx::bulk_wait_group_read0();  // before the CTA's memory goes
   }
 
   pdl_trigger();  // behind the last tile: see common.cuh
@@ -650,12 +655,26 @@ bool make_map(CUtensorMap* map, const void* base, int64_t rows, int64_t cols, in
 }
 
 namespace {
+// 2-D map of a 16-bit output [rows, cols] for the bias+GELU epilogue's stores:
+// box {32, 32}, 64-byte swizzle; elements outside are not written.
+bool make_store_map(CUtensorMap* map, void* base, int64_t rows, int64_t cols, bool half) {
+  auto fn = encode_fn();
+  if (!fn) return false;
+  cuuint64_t dims[2] = {static_cast<cuuint64_t>(cols), static_cast<cuuint64_t>(rows)};
+  cuuint64_t strides[1] = {static_cast<cuuint64_t>(cols) * 2};
+  cuuint32_t box[2] = {32u, 32u};
+  cuuint32_t estr[2] = {1u, 1u};
+  return fn(map, half ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base, dims,
+            strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
+            CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // Launches the product's work units on a persistent grid: one CTA per SM, or
 // for the pair variant one two-CTA cluster per SM pair, capped by how many
 // such clusters the device holds at once (a single wave).
 template <bool A_MN, bool B_MN, int EPI, bool OUT_F32, bool PAIR, int TBN = BN>
 cudaError_t launch_variant(const Params& p, int sms, const CUtensorMap& ta, const CUtensorMap& tb,
-                           cudaStream_t stream) {
+                           cudaStream_t stream, const CUtensorMap* tc = nullptr, const CUtensorMap* tx = nullptr) {
   auto kern = gemm_tc_kernel<A_MN, B_MN, EPI, OUT_F32, PAIR, TBN>;
   using SH = Shape<EPI, PAIR, TBN>;
   static cudaError_t attr =
@@ -688,19 +707,20 @@ cudaError_t launch_variant(const Params& p, int sms, const CUtensorMap& ta, cons
   const int units = p.m_tiles * p.n_tiles * p.splits;
   const int grid = units < ctas ? units : ctas;
   return launch_pdl(kern, dim3((PAIR ? 2 : 1) * grid), dim3(SH::THREADS), SH::SMEM, stream,
-                    PAIR ? 2 : 1, ta, tb, p);
+                    PAIR ? 2 : 1, ta, tb, tc ? *tc : ta, tx ? *tx : ta, p);
 }
 
 // One instantiation per (operand majorness, epilogue, output type, pairing)
 // keeps every kernel's code to the epilogue it runs.
 template <bool A_MN, bool B_MN, bool PAIR>
 cudaError_t launch_form(const Params& p, int sms, const CUtensorMap& ta, const CUtensorMap& tb,
-                        int epi, bool out_f32, cudaStream_t stream) {
+                        int epi, bool out_f32, cudaStream_t stream, const CUtensorMap* tc,
+                        const CUtensorMap* tx) {
   if (out_f32)
     return launch_variant<A_MN, B_MN, SKY_EPI_STORE, true, PAIR>(p, sms, ta, tb, stream);
   switch (epi) {
     case SKY_EPI_BIAS_GELU:
-      return launch_variant<A_MN, B_MN, SKY_EPI_BIAS_GELU, false, PAIR>(p, sms, ta, tb, stream);
+      return launch_variant<A_MN, B_MN, SKY_EPI_BIAS_GELU, false, PAIR>(p, sms, ta, tb, stream, tc, tx);
     case SKY_EPI_GELU_BWD:
       return launch_variant<A_MN, B_MN, SKY_EPI_GELU_BWD, false, PAIR>(p, sms, ta, tb, stream);
     default:
@@ -786,7 +806,13 @@ sky_status launch_bf16(sky_gemm_form form, int M, int N, int K, const void* A, c
   const bool may_split = out_f32 && epi == SKY_EPI_STORE && bias == nullptr && resid == nullptr;
   if (!colsum) {  // small and mid-sized products: the cluster kernel
     ClusterPlan pl;
-    if (plan_cluster(form, M, N, K, may_split, deferred_rows != nullptr, sms, &pl)) {
+    bool here = plan_cluster(form, M, N, K, may_split, deferred_rows != nullptr, sms, &pl);
+    // GELU' off the 16-byte grid cannot be written by TMA: 8-byte stores do it
+    if (!here && epi == SKY_EPI_BIAS_GELU && (reinterpret_cast<uintptr_t>(aux_out) & 15) != 0) {
+      pl = ClusterPlan{false, 64, 1};
+      here = true;
+    }
+    if (here) {
       float* part = nullptr;
       if (deferred_rows) {
         SKY_CHECK(!out_f32, SKY_ERR_UNSUPPORTED, "fused column sum needs a bf16 output");
@@ -801,7 +827,7 @@ sky_status launch_bf16(sky_gemm_form form, int M, int N, int K, const void* A, c
     }
   }
 
-  CUtensorMap ta, tb;
+  CUtensorMap ta, tb, tc{}, tx{};
   const bool a_mn = form == SKY_GEMM_XTW;
   const bool b_mn = form != SKY_GEMM_XWT;
   const bool pair = use_pair(M, epi);
@@ -825,6 +851,8 @@ sky_status launch_bf16(sky_gemm_form form, int M, int N, int K, const void* A, c
   const int tbn = narrow ? 192 : BN;
   bool ok = a_mn ? make_map(&ta, A, K, M, 64) : make_map(&ta, A, M, K, BM);
   ok = ok && (b_mn ? make_map(&tb, B, K, N, 64) : make_map(&tb, B, N, K, pair ? tbn / 2 : tbn));
+  if (epi == SKY_EPI_BIAS_GELU)
+    ok = ok && make_store_map(&tc, C, M, N, false) && make_store_map(&tx, aux_out, M, N, true);
   SKY_CHECK(ok, SKY_ERR_CUDA, "cuTensorMapEncodeTiled failed (M=%d N=%d K=%d)", M, N, K);
 
   Params p{};
@@ -875,18 +903,18 @@ sky_status launch_bf16(sky_gemm_form form, int M, int N, int K, const void* A, c
                 : launch_variant<false, false, SKY_EPI_STORE, false, true, 192>(p, sms, ta, tb, stream);
   } else if (pair) {
     if (form == SKY_GEMM_XWT)
-      e = launch_form<false, false, true>(p, sms, ta, tb, epi, out_f32, stream);
+      e = launch_form<false, false, true>(p, sms, ta, tb, epi, out_f32, stream, &tc, &tx);
     else if (form == SKY_GEMM_XW)
-      e = launch_form<false, true, true>(p, sms, ta, tb, epi, out_f32, stream);
+      e = launch_form<false, true, true>(p, sms, ta, tb, epi, out_f32, stream, &tc, &tx);
     else
-      e = launch_form<true, true, true>(p, sms, ta, tb, epi, out_f32, stream);
+      e = launch_form<true, true, true>(p, sms, ta, tb, epi, out_f32, stream, &tc, &tx);
   } else {
     if (form == SKY_GEMM_XWT)
-      e = launch_form<false, false, false>(p, sms, ta, tb, epi, out_f32, stream);
+      e = launch_form<false, false, false>(p, sms, ta, tb, epi, out_f32, stream, &tc, &tx);
     else if (form == SKY_GEMM_XW)
-      e = launch_form<false, true, false>(p, sms, ta, tb, epi, out_f32, stream);
+      e = launch_form<false, true, false>(p, sms, ta, tb, epi, out_f32, stream, &tc, &tx);
     else
-      e = launch_form<true, true, false>(p, sms, ta, tb, epi, out_f32, stream);
+      e = launch_form<true, true, false>(p, sms, ta, tb, epi, out_f32, stream, &tc, &tx);
   }
   count_launches(1);
   if (e != cudaSuccess) return cuda_fail(e, "gemm_tc_kernel launch");

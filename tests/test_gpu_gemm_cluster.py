@@ -105,3 +105,23 @@ def test_slice_with_split_products(batch, seq):
     X, lens, dY = synth.activations(w), synth.lengths(w), synth.upstream_grad(w)
     Y, dX, grads = run_gpu_slice(w, X, lens, dY, params, None)
     compare_slice(w, Y, dX, grads, *oracle_slice(w, X, lens, dY, params))
+
+
+@pytest.mark.parametrize("M,N,K", [(300, 8008, 136), (129, 20000, 72), (1000, 2600, 200)])
+@pytest.mark.parametrize("shift", [0, 8])
+def test_wide_bias_gelu(M, N, K, shift):
+    """The persistent kernel's bias + GELU, whose outputs leave by TMA, with ragged
+    rows and columns (pair and single-CTA tiles), and GELU' off the 16-byte grid,
+    which the cluster kernel writes."""
+    g = np.random.default_rng(M + N)
+    A = round_bf16(g.normal(0, 1, (M, K)).astype(np.float32))
+    W = round_bf16(g.normal(0, 0.1, (N, K)).astype(np.float32))
+    bias = round_bf16(g.normal(0, 0.5, N).astype(np.float32))
+    a, w, b = to_device(A, "bf16"), to_device(W, "bf16"), to_device(bias, "bf16")
+    pre = (a.double() @ w.double().T).cpu().numpy() + bias
+    raw = torch.full((shift // 2 + M * N + 64,), -7.0, dtype=torch.float16, device="cuda")
+    gp = raw[shift // 2:shift // 2 + M * N]
+    c = run_gemm(L.SKY_GEMM_XWT, M, N, K, a, w, torch.bfloat16, L.SKY_EPI_BIAS_GELU, b, aux_out=gp)
+    assert bool((raw[:shift // 2] == -7.0).all()) and bool((raw[shift // 2 + M * N:] == -7.0).all())
+    assert l2rel(to_host(c), ORC.gelu(pre)) <= 4e-3
+    assert l2rel(to_host(gp).reshape(M, N), ORC.gelu_grad(pre)) <= 1e-3
