@@ -9,10 +9,12 @@
 // FMA.  8 x 8 a thread, or 16-deep slabs, were slower: fewer warps, and less in
 // flight.  The layer's products have few such tiles (404 x 768: 84 for 152 SMs,
 // each SM wanting four CTAs or more), so the K range is split over a cluster of
-// up to eight CTAs, whose partial tiles are added in split order through
-// distributed shared memory.  Against the kernel before (64 x 64, 4 x 4 a
+// up to eight CTAs.  Each owns a share of the tile's rows; the others send it
+// theirs through distributed shared memory, and it adds them in split order
+// (reading them from the peers, behind a second barrier, cost 0.7 us a launch:
+// 2-layer slice of width 128 219 -> 186 us).  Against the kernel before (64 x 64, 4 x 4 a
 // thread, scalar loads, no split), alone: 404 x 768 x 3072 196 -> 52 us (37
-// TFLOP/s), 1000 x 2304 x 768 -> 77 us (46 TFLOP/s), 128 x 384 x 128 -> 4.8 us;
+// TFLOP/s), 1000 x 2304 x 768 -> 77 us (46 TFLOP/s);
 // the error against float64 falls with the shorter sums (9.9e-7 -> 3.5e-7).
 #include "common.cuh"
 #include "gemm.h"
@@ -80,15 +82,11 @@ __device__ __forceinline__ void store_slab(float* s, const float (&r)[4 * LD4]) 
   }
 }
 
-__device__ __forceinline__ float ld_cluster_f32(uint32_t addr) {
-  float v;
-  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
-  return v;
-}
-
 template <bool AK, bool BK, bool VEC>
 __global__ void __launch_bounds__(F_THREADS) gemm_f32_kernel(const F32Params p) {
-  __shared__ __align__(16) float sm[2][2][TK * 64];  // [buffer][A, B]; later the 64 x 64 partial tile
+  __shared__ __align__(16) float sm[2][2][TK * 64];  // [buffer][A, B]; later, unsplit, the 64 x 64 tile
+  __shared__ __align__(16) float recv[TM * TN];      // split: this CTA's rows from every split
+  if (p.ks > 1) ptx::cluster_arrive();  // this CTA runs: its peers may write recv
   pdl_wait();
   const int t = threadIdx.x;
   const int split = static_cast<int>(blockIdx.x) % p.ks, tile = static_cast<int>(blockIdx.x) / p.ks;
@@ -138,39 +136,51 @@ __global__ void __launch_bounds__(F_THREADS) gemm_f32_kernel(const F32Params p) 
     }
     p.C[off] = v;
   };
-  // The partial tile goes to shared memory (row r at r * 64, no padding: a
-  // thread's four columns as one 16-byte store) and comes back with a warp on 32
-  // consecutive columns of a row, from every split in order.
-  float* st = &sm[0][0][0];  // 4096 floats: the two buffers
-  const int c = t & 63;
-  __syncthreads();
-#pragma unroll
-  for (int i = 0; i < RM; ++i) {
-    const int r = (i < 4 ? 0 : 32) + rg * 4 + (i & 3);
-    *reinterpret_cast<ulonglong2*>(st + r * 64 + cg * 4) = make_ulonglong2(acc[i][0], acc[i][1]);
-  }
   if (p.ks == 1) {
+    // through shared memory (row r at r * 64), so that a warp stores 32 consecutive
+    // columns of a row
+    float* st = &sm[0][0][0];
+    const int c = t & 63;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < RM; ++i) {
+      const int r = (i < 4 ? 0 : 32) + rg * 4 + (i & 3);
+      *reinterpret_cast<ulonglong2*>(st + r * 64 + cg * 4) = make_ulonglong2(acc[i][0], acc[i][1]);
+    }
     __syncthreads();
 #pragma unroll 4
     for (int r = t / 64; r < TM; r += F_THREADS / 64) finish(m0 + r, n0 + c, st[r * 64 + c]);
     return;
   }
+  // Each CTA owns 64 / ks rows of the tile: every split sends it its partial rows,
+  // half a warp a row, and it adds them in split order.
+  const int own = TM / p.ks;
+  ptx::cluster_wait();  // every peer runs
+  const uint32_t base = ptx::smem_u32(recv);
+#pragma unroll
+  for (int i = 0; i < RM; ++i) {
+    const int r = (i < 4 ? 0 : 32) + rg * 4 + (i & 3);
+    const float2 lo = unpack2(acc[i][0]), hi = unpack2(acc[i][1]);
+    ptx::st_cluster_v4(ptx::mapa_shared(base, r / own) + ((split * own + r % own) * 64 + cg * 4) * 4,
+                       __float_as_uint(lo.x), __float_as_uint(lo.y), __float_as_uint(hi.x), __float_as_uint(hi.y));
+  }
   ptx::cluster_sync();
-  const int r0 = TM * split / p.ks, r1 = TM * (split + 1) / p.ks;
-  const uint32_t base = ptx::smem_u32(st);
-#pragma unroll 2
-  for (int r = r0 + t / 64; r < r1; r += F_THREADS / 64) {
-    float part[8];
+  for (int g = t; g < own * 16; g += F_THREADS) {
+    const int r = g >> 4, c = (g & 15) * 4;
+    float4 part[8];
 #pragma unroll
     for (int s = 0; s < 8; ++s)
-      part[s] = s < p.ks ? ld_cluster_f32(ptx::mapa_shared(base + (r * 64 + c) * 4, s)) : 0.f;
-    float v = part[0];
+      part[s] = s < p.ks ? *reinterpret_cast<const float4*>(recv + (s * own + r) * 64 + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 v = part[0];
 #pragma unroll
     for (int s = 1; s < 8; ++s)
-      if (s < p.ks) v += part[s];
-    finish(m0 + r, n0 + c, v);
+      if (s < p.ks) { v.x += part[s].x; v.y += part[s].y; v.z += part[s].z; v.w += part[s].w; }
+    const int m = m0 + split * own + r;
+    finish(m, n0 + c, v.x);
+    finish(m, n0 + c + 1, v.y);
+    finish(m, n0 + c + 2, v.z);
+    finish(m, n0 + c + 3, v.w);
   }
-  ptx::cluster_sync();  // the peers have read this CTA's partial tile
 }
 }  // namespace
 
@@ -199,7 +209,8 @@ sky_status launch_f32(sky_gemm_form form, int M, int N, int K, const float* A, c
   // where the tiles are few); never two, whose pairs land on one SM.  us at 1 /
   // 2 / 4 / 8 splits: 404 x 768 x 3072 146 / 134 / 77 / 52, 404 x 2304 x 768
   // 65 / 44 / 40 / 41, 1000 x 2304 x 768 77 / 82 / 82 / 86, 128 x 384 x 128
-  // 5.6 / 7.7 / 4.8 / -, 512 x 2048 x 97 12.4 / 16.1 / 15.1 / -.
+  // 5.6 / 7.7 / 4.8 / -, 512 x 2048 x 97 12.4 / 16.1 / 15.1 / - (all before the
+  // partial rows were sent rather than read).
   p.ks = 1;
   for (int ks = 8; ks >= 4 && p.ks == 1; ks /= 2)
     if (tiles * ks <= 10 * sms && p.k_slabs >= (4 * tiles <= sms ? ks : 2 * ks)) p.ks = ks;
