@@ -207,33 +207,43 @@ __global__ void __launch_bounds__(LN_WARPS * 32) ln_bwd_kernel(
   }
 }
 
-// out = a + b (fp32 inputs) in fp32 or bf16.
-template <typename T>
-__global__ void add_kernel(const float* __restrict__ a, const float* __restrict__ b, int64_t n,
-                           T* __restrict__ out) {
-  pdl_wait();
-  pdl_trigger();
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x)
-    out[i] = from_f32<T>(a[i] + b[i]);
+// Element-wise passes, four elements a thread in 16-byte accesses when the
+// pointers allow it (VEC; the last n % 4 elements, or all without VEC, one by
+// one).  HBM-bound: accumulating a base-width layer's 7.1 M gradients, 12 bytes
+// each, took 18.7 us with 4-byte accesses against 13 at the copy rate; 4
+// micro-batches of 3 such layers, with nine of these passes, 1815 -> 1795 us.
+__device__ __forceinline__ float4 load4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ float4 load4(const __nv_bfloat16* p) {
+  const uint2 r = *reinterpret_cast<const uint2*>(p);
+  const float2 a = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(&r)[0]);
+  const float2 b = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(&r)[1]);
+  return make_float4(a.x, a.y, b.x, b.y);
+}
+__device__ __forceinline__ void store4(float* p, const float4& v) { *reinterpret_cast<float4*>(p) = v; }
+__device__ __forceinline__ void store4(__nv_bfloat16* p, const float4& v) {
+  *reinterpret_cast<uint2*>(p) = make_uint2(ptx::pack_bf16(v.x, v.y), ptx::pack_bf16(v.z, v.w));
 }
 
-__global__ void to_bf16_kernel(const float* __restrict__ x, int64_t n,
-                               __nv_bfloat16* __restrict__ out) {
+// out = a + b (ADD) or out = a, in the types given.
+template <typename TI, typename TO, bool ADD, bool VEC>
+__global__ void __launch_bounds__(256) map_kernel(const TI* a, const TI* b, int64_t n, TO* out) {
   pdl_wait();
   pdl_trigger();
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x)
-    out[i] = __float2bfloat16_rn(x[i]);
-}
-
-template <typename T>
-__global__ void to_f32_kernel(const T* __restrict__ x, int64_t n, float* __restrict__ out) {
-  pdl_wait();
-  pdl_trigger();
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x)
-    out[i] = to_f32(x[i]);
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, nt = (int64_t)gridDim.x * blockDim.x;
+  const int64_t n4 = VEC ? n / 4 : 0;
+  for (int64_t i = t; i < n4; i += nt) {
+    float4 v = load4(a + 4 * i);
+    if constexpr (ADD) {
+      const float4 w = load4(b + 4 * i);
+      v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
+    }
+    store4(out + 4 * i, v);
+  }
+  for (int64_t i = 4 * n4 + t; i < n; i += nt) {
+    float v = to_f32(a[i]);
+    if constexpr (ADD) v += to_f32(b[i]);
+    out[i] = from_f32<TO>(v);
+  }
 }
 
 // LayerNorm backward, streamed through shared memory (bf16 slices, H = 1024
@@ -754,39 +764,36 @@ cudaError_t reduce_rows_f32(const float* part, int rows, int N, float* out, cuda
 }
 }  // namespace gemm
 
+namespace {
+template <typename TI, typename TO, bool ADD>
+sky_status launch_map(const TI* a, const TI* b, int64_t n, TO* out, cudaStream_t st, const char* what) {
+  if (n <= 0) return SKY_OK;
+  const bool vec = aligned16(a) && aligned16(b) && aligned16(out);
+  const int sms = sm_count() > 0 ? sm_count() : 148;
+  const int blocks = (int)std::min<int64_t>(ceil_div(vec ? (n + 3) / 4 : n, 256), 16 * sms);
+  const cudaError_t e = vec ? launch_pdl(rw::map_kernel<TI, TO, ADD, true>, dim3(blocks), dim3(256), 0, st, 1, a, b, n, out)
+                            : launch_pdl(rw::map_kernel<TI, TO, ADD, false>, dim3(blocks), dim3(256), 0, st, 1, a, b, n, out);
+  count_launches(1);
+  return e == cudaSuccess ? SKY_OK : cuda_fail(e, what);
+}
+}  // namespace
+
 sky_status add_f32(const float* a, const float* b, int64_t n, sky_dtype out_dt, void* out,
                    cudaStream_t st) {
-  if (n <= 0) return SKY_OK;
-  const int blocks = (int)std::min<int64_t>(ceil_div(n, 256), 8 * 148);
-  if (out_dt == SKY_DTYPE_BF16)
-    launch_pdl(rw::add_kernel<__nv_bfloat16>, dim3(blocks), dim3(256), 0, st, 1, a, b, n, static_cast<__nv_bfloat16*>(out));
-  else
-    launch_pdl(rw::add_kernel<float>, dim3(blocks), dim3(256), 0, st, 1, a, b, n, static_cast<float*>(out));
-  count_launches(1);
-  const cudaError_t e = cudaGetLastError();
-  return e == cudaSuccess ? SKY_OK : cuda_fail(e, "add launch");
+  return out_dt == SKY_DTYPE_BF16
+             ? launch_map<float, __nv_bfloat16, true>(a, b, n, static_cast<__nv_bfloat16*>(out), st, "add launch")
+             : launch_map<float, float, true>(a, b, n, static_cast<float*>(out), st, "add launch");
 }
 
 sky_status f32_to_bf16(const float* x, int64_t n, void* out, cudaStream_t st) {
-  if (n <= 0) return SKY_OK;
-  const int blocks = (int)std::min<int64_t>(ceil_div(n, 256), 8 * 148);
-  launch_pdl(rw::to_bf16_kernel, dim3(blocks), dim3(256), 0, st, 1, x, n, static_cast<__nv_bfloat16*>(out));
-  count_launches(1);
-  const cudaError_t e = cudaGetLastError();
-  return e == cudaSuccess ? SKY_OK : cuda_fail(e, "narrow launch");
+  return launch_map<float, __nv_bfloat16, false>(x, nullptr, n, static_cast<__nv_bfloat16*>(out), st, "narrow launch");
 }
 
 sky_status to_f32(const void* x, int64_t n, sky_dtype dt, float* out, cudaStream_t st) {
-  if (n <= 0) return SKY_OK;
-  const int blocks = (int)std::min<int64_t>(ceil_div(n, 256), 8 * 148);
-  if (dt == SKY_DTYPE_BF16)
-    launch_pdl(rw::to_f32_kernel<__nv_bfloat16>, dim3(blocks), dim3(256), 0, st, 1, 
-        static_cast<const __nv_bfloat16*>(x), n, out);
-  else
-    launch_pdl(rw::to_f32_kernel<float>, dim3(blocks), dim3(256), 0, st, 1, static_cast<const float*>(x), n, out);
-  count_launches(1);
-  const cudaError_t e = cudaGetLastError();
-  return e == cudaSuccess ? SKY_OK : cuda_fail(e, "widen launch");
+  return dt == SKY_DTYPE_BF16
+             ? launch_map<__nv_bfloat16, float, false>(static_cast<const __nv_bfloat16*>(x), nullptr, n, out, st,
+                                                       "widen launch")
+             : launch_map<float, float, false>(static_cast<const float*>(x), nullptr, n, out, st, "widen launch");
 }
 
 namespace {
