@@ -409,6 +409,10 @@ sky_status attention_fwd_tc(const void* qkv, const int32_t* lens, int B, int S, 
                             void* ctx, float* lse, int32_t* status, uint64_t timeout_ns,
                             cudaStream_t stream);
 
+sky_status attention_bwd_short_tc(const void* qkv, const void* ctx, const void* dctx, const float* lse,
+                                  const int32_t* lens, int B, int S, int H, int A, void* dqkv, int32_t* status,
+                                  uint64_t timeout_ns, cudaStream_t stream, float* colpart);
+
 sky_status attention_bwd_tc(const void* qkv, const void* dctx, const float* lse, const float* delta,
                             const uint4* xtab, const int32_t* lens, int B, int S, int H, int A, void* dqkv,
                             int32_t* status, uint64_t timeout_ns, cudaStream_t stream,
@@ -460,6 +464,11 @@ sky_status attention_bwd(const void* qkv, const void* ctx, const void* dctx, con
     const auto a16 = [](const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15) == 0; };
     SKY_CHECK(a16(qkv) && a16(ctx) && a16(dctx) && a16(dqkv) && a16(delta), SKY_ERR_INVALID_ARG,
               "bf16 attention backward buffers and workspace must be 16-byte aligned");
+    // one tile a sequence: everything in one launch (grid y is the batch, at most
+    // 65535 as for the kernels below)
+    if (S <= 128 && B <= 65535)
+      return attention_bwd_short_tc(qkv, ctx, dctx, lse, lens, B, S, H, A, dqkv, status, 2000000000ull, stream,
+                                    colpart);
     const auto* c = static_cast<const __nv_bfloat16*>(ctx);
     const auto* dc = static_cast<const __nv_bfloat16*>(dctx);
     const dim3 g(ceil_div(rows * 32, 256)), blk(256);

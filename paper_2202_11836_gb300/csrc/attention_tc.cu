@@ -989,6 +989,267 @@ __global__ void __maxnreg__(80) attn_bwd_dkdv_tc(const __grid_constant__ CUtenso
   }
 }
 
+// ------------------------------------------- backward, sequences up to 128
+// One CTA per (b, a): its 128-row tile holds every query and every key, so the
+// scores, P and dS are formed once and all three gradients follow from them:
+//   S = Q K^T, dP = dO V^T (M = N = 128, K = 64); thread = query row:
+//   P = exp2(S log2(e)/sqrt(D) - lse2), dS = P (dP - delta), delta from the row's
+//   dO and O, both as bf16 into shared memory, 128-byte-swizzled, where they are
+//   read as they lie (dS K) and transposed (P^T dO, dS^T Q):
+//   dV = P^T dO, dK = dS^T Q / sqrt(D), dQ = dS K / sqrt(D)  (M = 128, N = 64, K = 128).
+// The dK/dV and dQ kernels above form P and dS twice, from tables of a delta
+// pre-pass; at one tile a sequence each of the three is mostly prologue and
+// tail.  Bound by that chain's latency: load, two products, softmax, three
+// products, store.  Two CTAs share an SM, one's waits under the other's work
+// (112 KiB of tiles and 256 TMEM columns each: the gradients go over the scores).
+constexpr int SH_Q = 0, SH_K = Q_BYTES, SH_O = 2 * Q_BYTES, SH_V = 3 * Q_BYTES;
+// P: two 64-key chunks of 128 rows, the first over V; dS: two more
+constexpr int SH_P = SH_V, SH_DS = SH_P + 2 * Q_BYTES, SH_BAR = SH_DS + 2 * Q_BYTES;
+constexpr int SH_SMEM = SH_BAR + 128;
+constexpr int SH_THR = 320;  // warp 0 TMA, warp 1 MMA issue, warps 2..9 softmax
+static_assert(2 * (SH_SMEM + 1024) <= 233472, "two CTAs per SM");
+
+__global__ void __launch_bounds__(SH_THR, 2) attn_bwd_short_tc(const __grid_constant__ CUtensorMap tmQKV,
+                                                               const __grid_constant__ CUtensorMap tmO,
+                                                               const __grid_constant__ CUtensorMap tmC,
+                                                               const __grid_constant__ CUtensorMap tmOut,
+                                                               const BwdParams p) {
+  extern __shared__ __align__(1024) uint8_t smem[];
+  uint64_t* qk_full = reinterpret_cast<uint64_t*>(smem + SH_BAR);
+  uint64_t* ov_full = qk_full + 1;
+  uint64_t* sc_full = ov_full + 1;   // S and dP complete
+  uint64_t* pds_full = sc_full + 1;  // P and dS in shared memory
+  uint64_t* g_full = pds_full + 1;   // dV, dK, dQ complete
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(g_full + 1);
+
+  const int a = blockIdx.x, b = blockIdx.y;
+  const int S = p.S, H = p.H;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int row0 = b * S;
+  const uint64_t lim = p.timeout_ns;
+  if (threadIdx.x == 0) {
+    ptx::mbar_init(qk_full, 1);
+    ptx::mbar_init(ov_full, 1);
+    ptx::mbar_init(sc_full, 1);
+    ptx::mbar_init(pds_full, NSM_B);
+    ptx::mbar_init(g_full, 1);
+    ptx::fence_mbar_init();
+    ptx::fence_proxy_async_smem();
+    ptx::prefetch_tensormap(&tmQKV);
+    ptx::prefetch_tensormap(&tmO);
+    ptx::prefetch_tensormap(&tmC);
+  }
+  if (warp == 1) {
+    ptx::tmem_alloc(tmem_slot, 256);
+    ptx::tmem_relinquish();
+  }
+  ptx::tc_fence_before();
+  __syncthreads();
+  ptx::tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  const uint32_t tS = tmem, tdP = tmem + 128;                      // 128 columns each
+  const uint32_t tdV = tmem, tdK = tmem + 64, tdQ = tmem + 128;    // over them, 64 each
+  pdl_wait();
+  int len = p.lens[b];
+  if (len < 1 || len > S) {
+    if (p.status && threadIdx.x == 0) atomicOr(p.status, kStatusBadLength);
+    len = len < 1 ? 1 : S;
+  }
+
+  if (warp == 0) {
+    if (lane == 0) {
+      ptx::mbar_arrive_expect_tx(qk_full, 2 * Q_BYTES);
+      ptx::tma_load_2d(smem + SH_Q, &tmQKV, qk_full, a * HD, row0);
+      ptx::tma_load_2d(smem + SH_K, &tmQKV, qk_full, H + a * HD, row0);
+      ptx::mbar_arrive_expect_tx(ov_full, 3 * Q_BYTES);
+      ptx::tma_load_2d(smem + SH_O, &tmO, ov_full, a * HD, row0);
+      ptx::tma_load_2d(smem + SH_DS, &tmC, ov_full, a * HD, row0);  // ctx, until dS is formed
+      ptx::tma_load_2d(smem + SH_V, &tmQKV, ov_full, 2 * H + a * HD, row0);
+      // bounded waits for the copies before the CTA may exit
+      ptx::mbar_wait(qk_full, 0, lim, p.status, kWaitHint);
+      ptx::mbar_wait(ov_full, 0, lim, p.status, kWaitHint);
+    }
+  } else if (warp == 1) {
+    // (whole warp, one elected lane issuing: as in the forward)
+    constexpr uint32_t idS = ptx::idesc_bf16_f32(128, 128, false, false);
+    constexpr uint32_t idT = ptx::idesc_bf16_f32(128, HD, true, true);   // P^T dO, dS^T Q
+    constexpr uint32_t idN = ptx::idesc_bf16_f32(128, HD, false, true);  // dS K
+    const bool issuer = ptx::elect_one();
+    const uint32_t s0 = ptx::smem_u32(smem);
+    auto kmaj = [&](int off) { return ptx::smem_desc_sw128(s0 + off, 16, 1024); };
+    auto mnmaj = [&](int off) { return ptx::smem_desc_sw128(s0 + off, Q_BYTES, 1024); };
+    auto wait = [&](uint64_t* bar) {
+      return __all_sync(0xffffffffu, ptx::mbar_wait(bar, 0, lim, p.status, kWaitHint));
+    };
+    const uint64_t dq = kmaj(SH_Q), dk = kmaj(SH_K), dO = kmaj(SH_O), dv = kmaj(SH_V);
+    bool ok = wait(qk_full);
+    if (ok) {
+      ptx::tc_fence_after();
+      if (issuer) {
+#pragma unroll
+        for (int kk = 0; kk < HD / 16; ++kk) ptx::tc_mma_f16(tS, dq + kk * 2, dk + kk * 2, idS, kk > 0 ? 1u : 0u);
+      }
+      __syncwarp();
+      ok = wait(ov_full);
+    }
+    if (ok) {
+      ptx::tc_fence_after();
+      if (issuer) {
+#pragma unroll
+        for (int kk = 0; kk < HD / 16; ++kk) ptx::tc_mma_f16(tdP, dO + kk * 2, dv + kk * 2, idS, kk > 0 ? 1u : 0u);
+        ptx::tc_commit(sc_full);
+      }
+      __syncwarp();
+      ok = wait(pds_full);
+    }
+    if (ok) {
+      ptx::tc_fence_after();
+      const uint64_t pt = mnmaj(SH_P), dst = mnmaj(SH_DS), ds = kmaj(SH_DS);
+      const uint64_t bo = mnmaj(SH_O), bq = mnmaj(SH_Q), bk = mnmaj(SH_K);
+      if (issuer) {
+#pragma unroll
+        for (int kk = 0; kk < 8; ++kk) ptx::tc_mma_f16(tdV, pt + kk * 128, bo + kk * 128, idT, kk > 0 ? 1u : 0u);
+#pragma unroll
+        for (int kk = 0; kk < 8; ++kk) ptx::tc_mma_f16(tdK, dst + kk * 128, bq + kk * 128, idT, kk > 0 ? 1u : 0u);
+#pragma unroll
+        for (int kk = 0; kk < 8; ++kk)  // keys 16 kk ..: chunk kk / 4
+          ptx::tc_mma_f16(tdQ, ds + (kk >> 2) * (Q_BYTES >> 4) + (kk & 3) * 2, bk + kk * 128, idN, kk > 0 ? 1u : 0u);
+      }
+      __syncwarp();
+    }
+    // also on a timeout: what was issued has to finish before TMEM is released
+    if (issuer) ptx::tc_commit(g_full);
+    __syncwarp();
+    ptx::mbar_wait(g_full, 0, lim, p.status, kWaitHint);
+  } else {
+    const int q4 = warp & 3, hf = (warp - 2) >> 2;  // keys [64 hf, 64 hf + 64) of the row
+    const int r = q4 * 32 + lane;                   // query row = TMEM lane
+    const uint32_t lane_base = static_cast<uint32_t>(q4 * 32) << 16;
+    const float sl2 = LOG2E * 0.125f;
+    const bool live = r < S;
+    const float nlse2 = live ? -p.lse[(static_cast<int64_t>(b) * p.A + a) * S + r] : 0.f;
+    auto wait_all = [&](uint64_t* bar) {
+      return __all_sync(0xffffffffu, ptx::mbar_wait(bar, 0, lim, p.status, kWaitHint));
+    };
+    // delta = dO . O of the row, from the swizzled tiles (loaded from global memory
+    // row by row, 16 bytes a lane, this took 8 us)
+    float dl = 0.f;
+    bool ok = wait_all(ov_full);
+    if (ok) {
+      const uint32_t so = ptx::smem_u32(smem + SH_O) + r * 128, sx = ptx::smem_u32(smem + SH_DS) + r * 128;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        uint32_t x[4], y[4];
+        ptx::ld_shared_v4(so + ((j ^ (r & 7)) << 4), x);
+        ptx::ld_shared_v4(sx + ((j ^ (r & 7)) << 4), y);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float2 u = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&x[e]));
+          const float2 w = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&y[e]));
+          dl += u.x * w.x + u.y * w.y;
+        }
+      }
+    }
+    softmax_warps_sync();  // every row's O is read: dS may be written
+    ok = ok && wait_all(sc_full);
+    if (ok) {
+      ptx::tc_fence_after();
+      const uint32_t sp = ptx::smem_u32(smem + SH_P) + hf * Q_BYTES + r * 128;
+      const uint32_t sd = ptx::smem_u32(smem + SH_DS) + hf * Q_BYTES + r * 128;
+#pragma unroll
+      for (int c = 0; c < 64; c += 32) {
+        uint32_t sv[32], dv[32];
+        ptx::tmem_ld_32x32b_x32(tS + lane_base + hf * 64 + c, sv);
+        ptx::tmem_ld_32x32b_x32(tdP + lane_base + hf * 64 + c, dv);
+        ptx::tmem_ld_wait();
+        const int left = live ? len - hf * 64 - c : 0;  // valid keys from this chunk's first on
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          uint32_t pp[4], dd[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const int i = 8 * u + 2 * e;
+            const float p0 = ptx::ex2_ftz(fmaf(__uint_as_float(sv[i]), sl2, nlse2));
+            const float p1 = ptx::ex2_ftz(fmaf(__uint_as_float(sv[i + 1]), sl2, nlse2));
+            pp[e] = ptx::pack_bf16(p0, p1);
+            dd[e] = ptx::pack_bf16(p0 * (__uint_as_float(dv[i]) - dl), p1 * (__uint_as_float(dv[i + 1]) - dl));
+            const uint32_t keep = (i < left ? 0x0000ffffu : 0u) | (i + 1 < left ? 0xffff0000u : 0u);
+            pp[e] &= keep;
+            dd[e] &= keep;
+          }
+          const uint32_t at = ((c / 8 + u) ^ (r & 7)) << 4;
+          ptx::st_shared_v4(sp + at, pp[0], pp[1], pp[2], pp[3]);
+          ptx::st_shared_v4(sd + at, dd[0], dd[1], dd[2], dd[3]);
+        }
+      }
+      ptx::fence_proxy_async_smem();  // P, dS -> the MMAs
+      ptx::tc_fence_before();
+      ptx::mbar_arrive(pds_full);
+      ok = wait_all(g_full);
+    }
+    pdl_trigger();
+    // the low-half warps stage dK / sqrt(D), the high-half warps dV, and each half
+    // of dQ / sqrt(D), as 128-byte-swizzled bf16 rows over tiles that the last
+    // products have read; one thread stores the three by TMA, which drops the
+    // rows past S
+    float* red = reinterpret_cast<float*>(smem + SH_DS);  // column sums: [3][4 quarters][64]
+    if (ok) {
+      ptx::tc_fence_after();
+      const float sc = hf == 0 ? 0.125f : 1.f;
+      const int sel = hf == 0 ? 1 : 2;  // block of dqkv: 0 dQ, 1 dK, 2 dV
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const bool is_q = c == 2;
+        const int col = is_q ? hf * 32 : c * 32;  // of the gradient's 64
+        uint32_t o[32];
+        ptx::tmem_ld_32x32b_x32((is_q ? tdQ : (hf == 0 ? tdK : tdV)) + lane_base + col, o);
+        ptx::tmem_ld_wait();
+        const float m = is_q ? 0.125f : sc;
+        const uint32_t orow = ptx::smem_u32(smem + (is_q ? SH_Q : (hf == 0 ? SH_K : SH_V))) + r * 128;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          uint32_t w[4];
+#pragma unroll
+          for (int t = 0; t < 4; ++t)
+            w[t] = ptx::pack_bf16(__uint_as_float(o[8 * u + 2 * t]) * m, __uint_as_float(o[8 * u + 2 * t + 1]) * m);
+          ptx::st_shared_v4(orow + (((col / 8 + u) ^ (r & 7)) << 4), w[0], w[1], w[2], w[3]);
+        }
+        if (p.colpart) {  // column sums of the stored values over this warp's 32 rows
+          float v[32];
+#pragma unroll
+          for (int j = 0; j < 32; ++j) v[j] = live ? bf16_round(__uint_as_float(o[j]) * m) : 0.f;
+          lanes_column_sum(v, lane);
+          red[((is_q ? 0 : sel) * 4 + q4) * 64 + col + lane] = v[0];
+        }
+      }
+    } else if (p.colpart) {
+      red[(hf == 0 ? 1 : 2) * 256 + q4 * 64 + lane] = red[(hf == 0 ? 1 : 2) * 256 + q4 * 64 + 32 + lane] = 0.f;
+      red[q4 * 64 + hf * 32 + lane] = 0.f;
+    }
+    ptx::fence_proxy_async_smem();  // the staged rows -> the TMA stores
+    softmax_warps_sync();
+    if (warp == 2 && lane == 0) {
+      ptx::tma_store_3d(&tmOut, smem + SH_Q, a * HD, 0, b);
+      ptx::tma_store_3d(&tmOut, smem + SH_K, H + a * HD, 0, b);
+      ptx::tma_store_3d(&tmOut, smem + SH_V, 2 * H + a * HD, 0, b);
+      ptx::bulk_commit_group();
+    }
+    const int t = static_cast<int>(threadIdx.x) - 64;
+    if (p.colpart && t < 3 * HD) {  // the four row quarters, added in order
+      const int g = t / HD, c = t % HD;
+      const float* x = red + g * 256 + c;
+      p.colpart[static_cast<int64_t>(b) * 3 * H + g * H + a * HD + c] = ((x[0] + x[64]) + x[128]) + x[192];
+    }
+    if (warp == 2 && lane == 0) ptx::bulk_wait_group_read0();  // before the CTA's memory goes
+  }
+  ptx::tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    ptx::tc_fence_after();
+    ptx::tmem_dealloc(tmem, 256);
+  }
+}
+
 namespace {
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
@@ -1061,6 +1322,27 @@ sky_status attention_fwd_tc(const void* qkv, const int32_t* lens, int B, int S, 
   const cudaError_t e = launch_pdl(attn_fwd_tc, grid, dim3(NTHR), F_SMEM, stream, 1, tq, tkv, tout, p);
   count_launches(1);
   return e == cudaSuccess ? SKY_OK : cuda_fail(e, "tensor-core attention forward launch");
+}
+
+// Backward of sequences up to 128 (bf16, D = 64) in one launch.
+sky_status attention_bwd_short_tc(const void* qkv, const void* ctx, const void* dctx, const float* lse,
+                                  const int32_t* lens, int B, int S, int H, int A, void* dqkv, int32_t* status,
+                                  uint64_t timeout_ns, cudaStream_t stream, float* colpart) {
+  using namespace attn_tc;
+  SKY_CHECK(H == A * HD, SKY_ERR_UNSUPPORTED, "tensor-core attention needs head dim 64");
+  const int64_t T = static_cast<int64_t>(B) * S;
+  CUtensorMap tq, to, tc, tout;
+  SKY_CHECK(head_map(&tq, qkv, T, 3 * H, BQ) && head_map(&to, dctx, T, H, BQ) && head_map(&tc, ctx, T, H, BQ) &&
+                seq_map(&tout, dqkv, B, S, 3 * H, BQ),
+            SKY_ERR_CUDA, "cuTensorMapEncodeTiled failed for the attention backward operands");
+  static cudaError_t attr =
+      cudaFuncSetAttribute(attn_bwd_short_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, SH_SMEM);
+  if (attr != cudaSuccess) return cuda_fail(attr, "attention backward smem attribute");
+  BwdParams p{S, H, A, lens, lse, nullptr, nullptr, static_cast<__nv_bfloat16*>(dqkv), colpart, status, timeout_ns};
+  const cudaError_t e = launch_pdl(attn_bwd_short_tc, dim3(A, B), dim3(SH_THR), SH_SMEM, stream, 1, tq, to, tc,
+                                   tout, p);
+  count_launches(1);
+  return e == cudaSuccess ? SKY_OK : cuda_fail(e, "tensor-core attention backward launch");
 }
 
 // Backward launchers (bf16, D = 64): delta must already hold rowsum(dO * O).
