@@ -292,19 +292,18 @@ __global__ void __launch_bounds__(NTHR, 2) attn_fwd_tc(const __grid_constant__ C
       }
       // P = exp2(s * sl2 - m) as bf16 pairs into this row's lane of P buffer
       // j & 1 in tensor memory
-      const float nm = -m;
-      float ls = 0.f;
+      const uint64_t nm = pack2(-m, -m), sc = pack2(sl2, sl2);
+      uint64_t ls[2] = {0, 0};  // pairs of zeros
       uint32_t pk[BKV / 2];
 #pragma unroll
-      for (int u = 0; u < BKV / 8; ++u) {
-        float e[8];
-#pragma unroll
-        for (int t = 0; t < 8; ++t) e[t] = ptx::ex2_ftz(fmaf(__uint_as_float(v[8 * u + t]), sl2, nm));
-        ls += ((e[0] + e[1]) + (e[2] + e[3])) + ((e[4] + e[5]) + (e[6] + e[7]));
-#pragma unroll
-        for (int t = 0; t < 4; ++t) pk[4 * u + t] = ptx::pack_bf16(e[2 * t], e[2 * t + 1]);
+      for (int u = 0; u < BKV / 2; ++u) {
+        const float2 x = unpack2(fma2(pack2(__uint_as_float(v[2 * u]), __uint_as_float(v[2 * u + 1])), sc, nm));
+        const float e0 = ptx::ex2_ftz(x.x), e1 = ptx::ex2_ftz(x.y);
+        ls[u & 1] = add2(ls[u & 1], pack2(e0, e1));
+        pk[u] = ptx::pack_bf16(e0, e1);
       }
-      l += ls;
+      const float2 lsum = unpack2(add2(ls[0], ls[1]));
+      l += lsum.x + lsum.y;
       // P buffer j & 1 was last read by P_{j-2} V_{j-2}
       if (j >= 2 && !wait_all(&pv_done[j & 1], ((j - 2) >> 1) & 1)) { ok = false; break; }
       ptx::tmem_st_32x32b_x32(tP + (j & 1) * (BKV / 2) + lane_base, pk);
@@ -560,6 +559,7 @@ __global__ void __maxnreg__(80) attn_bwd_dq_tc(const __grid_constant__ CUtensorM
     const int64_t sidx = (static_cast<int64_t>(b) * p.A + a) * S + (q < S ? q : 0);
     const float nlse2 = q < S ? -p.lse[sidx] : -INFINITY;  // P = 0 on rows past S
     const float dl = q < S ? p.delta[sidx] : 0.f;
+    const uint64_t sc2 = pack2(sl2, sl2), nlse = pack2(nlse2, nlse2), ndl = pack2(-dl, -dl);
     bool ok = true;
     auto wait_all = [&](uint64_t* bar, uint32_t parity) {
       const bool mine = ptx::mbar_wait(bar, parity, lim, p.status, kWaitHint);
@@ -578,13 +578,10 @@ __global__ void __maxnreg__(80) attn_bwd_dq_tc(const __grid_constant__ CUtensorM
       uint32_t pk[16];
 #pragma unroll
       for (int i = 0; i < 32; i += 2) {
-        float ds2[2];
-#pragma unroll
-        for (int t = 0; t < 2; ++t) {
-          const float pr = ptx::ex2_ftz(fmaf(__uint_as_float(sv[i + t]), sl2, nlse2));
-          ds2[t] = pr * (__uint_as_float(dv[i + t]) - dl);
-        }
-        pk[i >> 1] = ptx::pack_bf16(ds2[0], ds2[1]);
+        const float2 x = unpack2(fma2(pack2(__uint_as_float(sv[i]), __uint_as_float(sv[i + 1])), sc2, nlse));
+        const uint64_t pr = pack2(ptx::ex2_ftz(x.x), ptx::ex2_ftz(x.y));
+        const float2 ds = unpack2(mul2(pr, add2(pack2(__uint_as_float(dv[i]), __uint_as_float(dv[i + 1])), ndl)));
+        pk[i >> 1] = ptx::pack_bf16(ds.x, ds.y);
       }
       if (kbase + 32 > len) {  // warp-uniform: only the last tile holds masked keys
 #pragma unroll
@@ -882,9 +879,9 @@ __global__ void __maxnreg__(80) attn_bwd_dkdv_tc(const __grid_constant__ CUtenso
     const int hf = (warp - 2) >> 2;  // column half: queries [32 hf, 32 hf + 32) of a tile
     const int r = q4 * 32 + lane;    // key row within the tile == TMEM lane
     const int key = k0 + r;
-    const bool kvalid = key < len;
     const uint32_t lane_base = static_cast<uint32_t>(q4 * 32) << 16;
-    const float sl2 = LOG2E * 0.125f;
+    const float sl2 = LOG2E * 0.125f, pad = key < len ? 0.f : -INFINITY;
+    const uint64_t sc2 = pack2(sl2, sl2), off = pack2(pad, pad);
     bool ok = true;
     auto wait_all = [&](uint64_t* bar, uint32_t parity) {
       const bool mine = ptx::mbar_wait(bar, parity, lim, p.status, kWaitHint);
@@ -901,14 +898,12 @@ __global__ void __maxnreg__(80) attn_bwd_dkdv_tc(const __grid_constant__ CUtenso
       uint32_t pp[16], dd[16];
 #pragma unroll
       for (int t = 0; t < 32; t += 2) {
-        float pt[2], ds[2];
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          pt[e] = kvalid ? ptx::ex2_ftz(__uint_as_float(sv[t + e]) * sl2) : 0.f;
-          ds[e] = pt[e] * __uint_as_float(dv[t + e]);
-        }
-        pp[t >> 1] = ptx::pack_bf16(pt[0], pt[1]);
-        dd[t >> 1] = ptx::pack_bf16(ds[0], ds[1]);
+        // (a key past the valid length: exp2(-inf) = 0)
+        const float2 x = unpack2(fma2(pack2(__uint_as_float(sv[t]), __uint_as_float(sv[t + 1])), sc2, off));
+        const float2 pt = make_float2(ptx::ex2_ftz(x.x), ptx::ex2_ftz(x.y));
+        const float2 ds = unpack2(mul2(pack2(pt.x, pt.y), pack2(__uint_as_float(dv[t]), __uint_as_float(dv[t + 1]))));
+        pp[t >> 1] = ptx::pack_bf16(pt.x, pt.y);
+        dd[t >> 1] = ptx::pack_bf16(ds.x, ds.y);
       }
       const int nq = S - i * BQ2 - hf * 32;  // queries of this half inside the sequence
       if (nq < 32) {  // warp-uniform: queries past S
@@ -1150,6 +1145,7 @@ __global__ void __launch_bounds__(SH_THR, 2) attn_bwd_short_tc(const __grid_cons
         }
       }
     }
+    const uint64_t sc2 = pack2(sl2, sl2), nlse = pack2(nlse2, nlse2), ndl = pack2(-dl, -dl);
     softmax_warps_sync();  // every row's O is read: dS may be written
     ok = ok && wait_all(sc_full);
     if (ok) {
@@ -1169,10 +1165,12 @@ __global__ void __launch_bounds__(SH_THR, 2) attn_bwd_short_tc(const __grid_cons
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
             const int i = 8 * u + 2 * e;
-            const float p0 = ptx::ex2_ftz(fmaf(__uint_as_float(sv[i]), sl2, nlse2));
-            const float p1 = ptx::ex2_ftz(fmaf(__uint_as_float(sv[i + 1]), sl2, nlse2));
+            const float2 x = unpack2(fma2(pack2(__uint_as_float(sv[i]), __uint_as_float(sv[i + 1])), sc2, nlse));
+            const float p0 = ptx::ex2_ftz(x.x), p1 = ptx::ex2_ftz(x.y);
+            const float2 ds = unpack2(
+                mul2(pack2(p0, p1), add2(pack2(__uint_as_float(dv[i]), __uint_as_float(dv[i + 1])), ndl)));
             pp[e] = ptx::pack_bf16(p0, p1);
-            dd[e] = ptx::pack_bf16(p0 * (__uint_as_float(dv[i]) - dl), p1 * (__uint_as_float(dv[i + 1]) - dl));
+            dd[e] = ptx::pack_bf16(ds.x, ds.y);
             const uint32_t keep = (i < left ? 0x0000ffffu : 0u) | (i + 1 < left ? 0xffff0000u : 0u);
             pp[e] &= keep;
             dd[e] &= keep;
