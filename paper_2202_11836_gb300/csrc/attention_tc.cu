@@ -6,7 +6,7 @@
 //   S_j = Q K_j^T                  tcgen05.mma M=128 N=64 K=64 -> TMEM
 //   softmax (4 warps, thread = query row = TMEM lane): row max over the
 //     valid keys, P_j = exp2(S_j log2(e)/sqrt(D) - m) written as bf16 pairs
-//     back to tensor memory (tcgen05.st), where the next product reads it
+//     over the scores (tcgen05.st), where the next product reads it
 //   O += P_j V_j                   tcgen05.mma M=128 N=64 K=64, A = P_j from
 //                                  TMEM, B = V_j from shared memory -> TMEM
 // Q, K and V come straight out of the packed QKV activations by TMA (one
@@ -14,18 +14,19 @@
 // memory.  Because a thread owns a whole query row, the row max and row sum
 // need no shuffles.
 //
-// The steps are pipelined inside the CTA: S and P have two TMEM buffers each,
-// so the MMA warp computes S_{j+1} (issued one tile
-// ahead) and P_{j-1} V_{j-1} while the softmax warps work on tile j, and K/V
-// tiles stream through a 3-stage TMA ring.  The exponent offset m of a row
-// is only raised when the tile's max exceeds it by more than 2^8 (a factor
-// 256 in P): then O and the row sum are rescaled in TMEM once the pending
-// P V product has landed.  Otherwise P may exceed 1 by at most that factor,
-// which bf16 and the fp32 sums carry with the same relative precision; the
-// final O / l and the log-sum-exp do not depend on m.  The log-sum-exp is
-// kept in base-2 units, lse2 = log2 sum_j exp2(S_ij log2(e)/sqrt(D)), which
-// is what the backward kernels subtract in the exponent.  All mbarrier
-// waits are time-bounded.
+// The chain of a tile is serial inside a CTA; what overlaps it is other CTAs.
+// With P over S, a CTA needs 128 TMEM columns, 49 KiB of shared memory (two K/V
+// stages) and 80 registers a thread (half a row's scores at a time, the high
+// half read twice), so four share an SM.  Two CTAs with S and P double-buffered
+// inside each were 69.1 us at S = 2048 (16 heads, 4 sequences), three of these
+// 80.7, four 63.4.  No pipe is full then (ncu: issue 46%, tensor 37%, XU 37% of
+// the active cycles).  The exponent offset m of a row is only raised when the
+// tile's max exceeds it by more than 2^8 (a factor 256 in P): then O and the row
+// sum are rescaled in TMEM.  Otherwise P may exceed 1 by at most that factor,
+// which bf16 and the fp32 sums carry with the same relative precision; the final
+// O / l and the log-sum-exp do not depend on m.  The log-sum-exp is kept in
+// base-2 units, lse2 = log2 sum_j exp2(S_ij log2(e)/sqrt(D)), which is what the
+// backward kernels subtract in the exponent.  All mbarrier waits are time-bounded.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -40,8 +41,7 @@ namespace attn_tc {
 constexpr int BQ = 128, BKV = 64, HD = 64;
 constexpr int Q_BYTES = BQ * HD * 2;    // 16 KiB
 constexpr int KV_BYTES = BKV * HD * 2;  // 8 KiB per K or V tile
-// forward CTA: warp 0 TMA and O += P V issue, warp 1 S = Q K^T issue,
-// warps 2..5 softmax
+// forward CTA: warp 0 TMA, warp 1 MMA issue, warps 2..5 softmax
 constexpr int NTHR = 192;
 // The backward kernels run eight softmax warps: warps w and w + 4 share TMEM
 // lane quarter w % 4 and take the low / high 32 columns of each 64-wide tile.
@@ -59,14 +59,16 @@ constexpr float LOG2E = 1.4426950408889634f;
 constexpr uint32_t kWaitHint = 10000;
 
 // forward shared-memory layout (offsets from a 1024-byte aligned base)
-constexpr int F_STAGES = 3;
+constexpr int F_STAGES = 2;
 constexpr int F_Q_OFF = 0;
 constexpr int F_KV_OFF = F_Q_OFF + Q_BYTES;                  // [F_STAGES] x {K, V}
 constexpr int F_BAR_OFF = F_KV_OFF + F_STAGES * 2 * KV_BYTES;
 constexpr int F_SMEM = F_BAR_OFF + 256 + 1024;
-// S_0: [0, 64), S_1: [64, 128), O: [128, 192), P_0: [192, 224), P_1: [224, 256)
-// (P as bf16 pairs: the A operand of P V read from tensor memory)
-constexpr int F_TMEM_COLS = 256;
+// S: [0, 64), then P as bf16 pairs in [0, 32) (the A operand of P V, read from
+// tensor memory); O: [64, 128)
+constexpr int F_TMEM_COLS = 128;
+constexpr int F_CTAS = 4;  // per SM
+static_assert(F_CTAS * (F_SMEM + 1024) <= 233472, "four forward CTAs per SM");
 constexpr float kRescaleLog2 = 8.f;
 
 struct FwdParams {
@@ -76,37 +78,26 @@ struct FwdParams {
   float* lse;
   int32_t* status;
   uint64_t timeout_ns;
-  int late_trigger;  // let the next kernel start behind the last score product, not at once
 };
 
-__global__ void __launch_bounds__(NTHR, 2) attn_fwd_tc(const __grid_constant__ CUtensorMap tmQ,
+__global__ void __launch_bounds__(NTHR, F_CTAS) attn_fwd_tc(const __grid_constant__ CUtensorMap tmQ,
                                                     const __grid_constant__ CUtensorMap tmKV,
                                                     const __grid_constant__ CUtensorMap tmOut,
                                                     const FwdParams p) {
-  if (!p.late_trigger) pdl_trigger();
-  pdl_wait();
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw_addr = ptx::smem_u32(smem_raw);
   uint8_t* smem = smem_raw + (((raw_addr + 1023u) & ~1023u) - raw_addr);
   uint64_t* q_full = reinterpret_cast<uint64_t*>(smem + F_BAR_OFF);
   uint64_t* kv_full = q_full + 1;
   uint64_t* kv_empty = kv_full + F_STAGES;
-  uint64_t* s_full = kv_empty + F_STAGES;  // [2]
-  uint64_t* s_free = s_full + 2;           // [2]
-  uint64_t* p_full = s_free + 2;           // [2]
-  uint64_t* pv_done = p_full + 2;          // [2]
-  uint64_t* done = pv_done + 2;            // [2], one per issuing warp
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 2);
+  uint64_t* s_full = kv_empty + F_STAGES;  // S_j complete
+  uint64_t* p_full = s_full + 1;           // P_j in tensor memory
+  uint64_t* pv_done = p_full + 1;          // O += P_j V_j complete
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(pv_done + 1);
 
   const int qt = blockIdx.x, a = blockIdx.y, b = blockIdx.z;
   const int S = p.S, H = p.H;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int len = p.lens[b];
-  if (len < 1 || len > S) {
-    if (p.status && threadIdx.x == 0) atomicOr(p.status, kStatusBadLength);
-    len = len < 1 ? 1 : S;
-  }
-  const int n_kt = (len + BKV - 1) / BKV;
   const int row0 = b * S;  // first token row of this sequence
   const int q0 = qt * BQ;
   const uint64_t lim = p.timeout_ns;
@@ -115,18 +106,15 @@ __global__ void __launch_bounds__(NTHR, 2) attn_fwd_tc(const __grid_constant__ C
     ptx::mbar_init(q_full, 1);
     for (int s = 0; s < F_STAGES; ++s) {
       ptx::mbar_init(&kv_full[s], 1);
-      ptx::mbar_init(&kv_empty[s], 2);  // S_j has read K_j, P_j V_j has read V_j
+      ptx::mbar_init(&kv_empty[s], 1);
     }
-    for (int s = 0; s < 2; ++s) {
-      ptx::mbar_init(&s_full[s], 1);
-      ptx::mbar_init(&s_free[s], 128);
-      ptx::mbar_init(&p_full[s], 128);
-      ptx::mbar_init(&pv_done[s], 1);
-    }
-    ptx::mbar_init(&done[0], 1);
-    ptx::mbar_init(&done[1], 1);
+    ptx::mbar_init(s_full, 1);
+    ptx::mbar_init(p_full, 128);
+    ptx::mbar_init(pv_done, 1);
     ptx::fence_mbar_init();
     ptx::fence_proxy_async_smem();
+    ptx::prefetch_tensormap(&tmQ);
+    ptx::prefetch_tensormap(&tmKV);
   }
   if (warp == 1) {
     ptx::tmem_alloc(tmem_slot, F_TMEM_COLS);
@@ -136,97 +124,85 @@ __global__ void __launch_bounds__(NTHR, 2) attn_fwd_tc(const __grid_constant__ C
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  const uint32_t tS = tmem, tO = tmem + 128, tP = tmem + 192;
+  const uint32_t tS = tmem, tO = tmem + 64;
+  pdl_wait();
+  int len = p.lens[b];
+  if (len < 1 || len > S) {
+    if (p.status && threadIdx.x == 0) atomicOr(p.status, kStatusBadLength);
+    len = len < 1 ? 1 : S;
+  }
+  const int n_kt = (len + BKV - 1) / BKV;
 
   if (warp == 0) {
-    // --------------------------------- producer and O += P V issue (warp 0)
-    // Loads Q and the first F_STAGES K/V tiles, then per tile j: issues
-    // O += P_j V_j once the softmax warps have written P_j, and refills the
-    // ring slot of tile j with tile j + F_STAGES once S_j and P_j V_j have
-    // read it.
-    // The whole warp walks the loop and one elected lane issues: a
-    // tcgen05.mma takes its descriptors from uniform registers, and built
-    // inside one lane's branch they were moved there instruction by
-    // instruction, slower than the tensor pipe works on these products.
-    constexpr uint32_t idO = ptx::idesc_bf16_f32(BQ, HD, false, true);
+    // ------------------------------------------------------------- producer
     const bool issuer = ptx::elect_one();
-    const uint64_t dv0 = ptx::smem_desc_sw128(ptx::smem_u32(smem + F_KV_OFF + KV_BYTES), 8192, 1024);
-    auto wait = [&](uint64_t* bar, uint32_t parity) {
-      return __all_sync(0xffffffffu, ptx::mbar_wait(bar, parity, lim, p.status, kWaitHint));
-    };
-    auto load_kv = [&](int j) {
-      const int st = j % F_STAGES;
-      uint8_t* kv = smem + F_KV_OFF + st * 2 * KV_BYTES;
-      ptx::mbar_arrive_expect_tx(&kv_full[st], 2 * KV_BYTES);
-      ptx::tma_load_2d(kv, &tmKV, &kv_full[st], H + a * HD, row0 + j * BKV);
-      ptx::tma_load_2d(kv + KV_BYTES, &tmKV, &kv_full[st], 2 * H + a * HD, row0 + j * BKV);
-    };
     if (issuer) {
       ptx::mbar_arrive_expect_tx(q_full, Q_BYTES);
       ptx::tma_load_2d(smem + F_Q_OFF, &tmQ, q_full, a * HD, row0 + q0);
     }
-    int issued = 0;
-    for (; issued < n_kt && issued < F_STAGES; ++issued)
-      if (issuer) load_kv(issued);
     __syncwarp();
+    int issued = 0;
     for (int j = 0; j < n_kt; ++j) {
-      if (!wait(&p_full[j & 1], (j >> 1) & 1)) break;
-      if (!wait(&kv_full[j % F_STAGES], (j / F_STAGES) & 1)) break;
-      ptx::tc_fence_after();
+      const int st = j % F_STAGES;
+      if (!__all_sync(0xffffffffu,
+                      ptx::mbar_wait(&kv_empty[st], ((j / F_STAGES) & 1) ^ 1u, lim, p.status, kWaitHint)))
+        break;
       if (issuer) {
-        const uint64_t dv = dv0 + static_cast<uint64_t>((j % F_STAGES) * (2 * KV_BYTES >> 4));
-        const uint32_t tpj = tP + (j & 1) * (BKV / 2);
-#pragma unroll
-        for (int kk = 0; kk < BKV / 16; ++kk)
-          ptx::tc_mma_f16_tmem_a(tO, tpj + kk * 8, dv + kk * 128, idO, (j > 0 || kk > 0) ? 1u : 0u);
-        ptx::tc_commit(&pv_done[j & 1]);
-        ptx::tc_commit(&kv_empty[j % F_STAGES]);
+        uint8_t* kv = smem + F_KV_OFF + st * 2 * KV_BYTES;
+        ptx::mbar_arrive_expect_tx(&kv_full[st], 2 * KV_BYTES);
+        ptx::tma_load_2d(kv, &tmKV, &kv_full[st], H + a * HD, row0 + j * BKV);
+        ptx::tma_load_2d(kv + KV_BYTES, &tmKV, &kv_full[st], 2 * H + a * HD, row0 + j * BKV);
       }
       __syncwarp();
-      if (issued < n_kt) {  // the slot of tile j takes tile j + F_STAGES
-        if (!wait(&kv_empty[issued % F_STAGES], ((issued / F_STAGES) & 1) ^ 1u)) break;
-        if (issuer) load_kv(issued);
-        __syncwarp();
-        ++issued;
-      }
+      ++issued;
     }
-    if (issuer) ptx::tc_commit(&done[1]);
-    __syncwarp();
-    ptx::mbar_wait(&done[1], 0, lim, p.status, kWaitHint);
     // drain: bounded waits for the copies still in flight
     ptx::mbar_wait(q_full, 0, lim, p.status, kWaitHint);
     for (int j = issued - 1; j >= 0 && j >= issued - F_STAGES; --j)
       ptx::mbar_wait(&kv_full[j % F_STAGES], (j / F_STAGES) & 1, lim, p.status, kWaitHint);
   } else if (warp == 1) {
-    // --------------------------------------------- S = Q K^T issue (warp 1)
-    // S_j goes into buffer j & 1 as soon as K_j has landed and the softmax
-    // warps hold S_{j-2} in registers (s_free)
+    // ------------------------------------------------------------ MMA issue
+    // The whole warp walks the loop and one elected lane issues: a
+    // tcgen05.mma takes its descriptors from uniform registers, and built
+    // inside one lane's branch they were moved there instruction by
+    // instruction, slower than the tensor pipe works on these products.
     constexpr uint32_t idS = ptx::idesc_bf16_f32(BQ, BKV, false, false);
+    constexpr uint32_t idO = ptx::idesc_bf16_f32(BQ, HD, false, true);
     const bool issuer = ptx::elect_one();
     const uint64_t dq = ptx::smem_desc_sw128(ptx::smem_u32(smem + F_Q_OFF), 16, 1024);
     const uint64_t dk0 = ptx::smem_desc_sw128(ptx::smem_u32(smem + F_KV_OFF), 16, 1024);
+    const uint64_t dv0 = ptx::smem_desc_sw128(ptx::smem_u32(smem + F_KV_OFF + KV_BYTES), 8192, 1024);
     auto wait = [&](uint64_t* bar, uint32_t parity) {
       return __all_sync(0xffffffffu, ptx::mbar_wait(bar, parity, lim, p.status, kWaitHint));
     };
     bool ok = wait(q_full, 0);
     for (int j = 0; j < n_kt && ok; ++j) {
-      if (j >= 2 && !wait(&s_free[j & 1], ((j - 2) >> 1) & 1)) break;
-      if (!wait(&kv_full[j % F_STAGES], (j / F_STAGES) & 1)) break;
+      const uint64_t off = static_cast<uint64_t>((j % F_STAGES) * (2 * KV_BYTES >> 4));
+      // K_j, V_j are here, and P_{j-1}, whose columns S_j takes, has been read
+      if (!wait(&kv_full[j % F_STAGES], (j / F_STAGES) & 1)) { ok = false; break; }
+      if (j > 0 && !wait(pv_done, (j - 1) & 1)) { ok = false; break; }
       ptx::tc_fence_after();
       if (issuer) {
-        const uint64_t dk = dk0 + static_cast<uint64_t>((j % F_STAGES) * (2 * KV_BYTES >> 4));
 #pragma unroll
         for (int kk = 0; kk < HD / 16; ++kk)
-          ptx::tc_mma_f16(tS + (j & 1) * BKV, dq + kk * 2, dk + kk * 2, idS, kk > 0 ? 1u : 0u);
-        ptx::tc_commit(&s_full[j & 1]);
+          ptx::tc_mma_f16(tS, dq + kk * 2, dk0 + off + kk * 2, idS, kk > 0 ? 1u : 0u);
+        ptx::tc_commit(s_full);
+      }
+      __syncwarp();
+      if (!wait(p_full, j & 1)) { ok = false; break; }
+      ptx::tc_fence_after();
+      if (issuer) {
+#pragma unroll
+        for (int kk = 0; kk < BKV / 16; ++kk)
+          ptx::tc_mma_f16_tmem_a(tO, tS + kk * 8, dv0 + off + kk * 128, idO, (j > 0 || kk > 0) ? 1u : 0u);
+        ptx::tc_commit(pv_done);
         ptx::tc_commit(&kv_empty[j % F_STAGES]);
       }
       __syncwarp();
     }
-    if (p.late_trigger) pdl_trigger();
-    if (issuer) ptx::tc_commit(&done[0]);
+    if (!ok && issuer) ptx::tc_commit(pv_done);  // a timeout: what was issued still has to finish
     __syncwarp();
-    ptx::mbar_wait(&done[0], 0, lim, p.status, kWaitHint);
+    ptx::mbar_wait(pv_done, (n_kt - 1) & 1, lim, p.status, kWaitHint);
   } else {
     // --------------------------------------------------- softmax / epilogue
     const int q4 = warp & 3;
@@ -241,96 +217,93 @@ __global__ void __launch_bounds__(NTHR, 2) attn_fwd_tc(const __grid_constant__ C
       const bool mine = ptx::mbar_wait(bar, parity, lim, p.status, kWaitHint);
       return __all_sync(0xffffffffu, mine);
     };
+    uint32_t v[32];  // half a row's scores at a time: registers for four CTAs an SM
     for (int j = 0; j < n_kt; ++j) {
-      if (!wait_all(&s_full[j & 1], (j >> 1) & 1)) { ok = false; break; }
+      const int left = len - j * BKV;  // valid keys of this tile
+      auto load_half = [&](int h) {
+        ptx::tmem_ld_32x32b_x32(tS + lane_base + h * 32, v);
+        ptx::tmem_ld_wait();
+        if (left < (h + 1) * 32) {  // CTA-uniform: only the last tile holds masked keys
+#pragma unroll
+          for (int i = 0; i < 32; ++i)
+            if (h * 32 + i >= left) v[i] = 0xff800000u;  // -inf: excluded from the max, P = 0
+        }
+      };
+      auto half_max = [&](float mx) {
+        float m4[4] = {mx, __uint_as_float(v[0]), __uint_as_float(v[1]), __uint_as_float(v[2])};
+#pragma unroll
+        for (int i = 3; i < 32; ++i) m4[i & 3] = fmaxf(m4[i & 3], __uint_as_float(v[i]));
+        return fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
+      };
+      if (!wait_all(s_full, j & 1)) { ok = false; break; }
       ptx::tc_fence_after();
-      uint32_t v[BKV];
-      {
-        uint32_t (&v0)[32] = *reinterpret_cast<uint32_t(*)[32]>(&v[0]);
-        uint32_t (&v1)[32] = *reinterpret_cast<uint32_t(*)[32]>(&v[32]);
-        ptx::tmem_ld_32x32b_x32(tS + (j & 1) * BKV + lane_base, v0);
-        ptx::tmem_ld_32x32b_x32(tS + (j & 1) * BKV + lane_base + 32, v1);
-      }
-      ptx::tmem_ld_wait();
-      // S_j is in registers: its buffer may take S_{j+2}
-      ptx::tc_fence_before();
-      ptx::mbar_arrive(&s_free[j & 1]);
-      const int kbase = j * BKV;
-      if (kbase + BKV > len) {  // CTA-uniform: only the last tile holds masked keys
-#pragma unroll
-        for (int i = 0; i < BKV; ++i)
-          if (kbase + i >= len) v[i] = 0xff800000u;  // -inf: excluded from the max, P = 0
-      }
-      // row max of the raw scores (scaling by log2(e)/sqrt(D) > 0 commutes with max)
-      float mx8[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) mx8[i] = __uint_as_float(v[i]);
-#pragma unroll
-      for (int i = 8; i < BKV; ++i) mx8[i & 7] = fmaxf(mx8[i & 7], __uint_as_float(v[i]));
-      const float mx = fmaxf(fmaxf(fmaxf(mx8[0], mx8[1]), fmaxf(mx8[2], mx8[3])),
-                             fmaxf(fmaxf(mx8[4], mx8[5]), fmaxf(mx8[6], mx8[7]))) * sl2;
+      // row max of the raw scores (scaling by log2(e)/sqrt(D) > 0 commutes with
+      // max): the high half, then the low half, which stays in registers
+      load_half(1);
+      float mx = half_max(-INFINITY);
+      load_half(0);
+      mx = half_max(mx) * sl2;
       if (j == 0) {
         m = mx;
       } else if (__any_sync(0xffffffffu, mx > m + kRescaleLog2)) {
-        // O must hold P_{j-1} V_{j-1} before it is rescaled
-        if (!wait_all(&pv_done[(j - 1) & 1], ((j - 1) >> 1) & 1)) { ok = false; break; }
-        ptx::tc_fence_after();
+        // O holds P_{j-1} V_{j-1}: S_j was issued behind it
         const float m_new = fmaxf(m, mx);
         const float alpha = exp2f(m - m_new);
 #pragma unroll
-        for (int c = 0; c < HD / 32; ++c) {
-          uint32_t o[32];
-          ptx::tmem_ld_32x32b_x32(tO + lane_base + c * 32, o);
+        for (int c = 0; c < HD / 16; ++c) {
+          uint32_t o[16];
+          ptx::tmem_ld_32x32b_x16(tO + lane_base + c * 16, o);
           ptx::tmem_ld_wait();
 #pragma unroll
-          for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
-          ptx::tmem_st_32x32b_x32(tO + lane_base + c * 32, o);
+          for (int i = 0; i < 16; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
+          ptx::tmem_st_32x32b_x16(tO + lane_base + c * 16, o);
         }
-        ptx::tmem_st_wait();
         l *= alpha;
         m = m_new;
       }
-      // P = exp2(s * sl2 - m) as bf16 pairs into this row's lane of P buffer
-      // j & 1 in tensor memory
+      // P = exp2(s * sl2 - m) as bf16 pairs over the scores: the low half's into
+      // the columns it was read from, then the high half's behind it
       const uint64_t nm = pack2(-m, -m), sc = pack2(sl2, sl2);
       uint64_t ls[2] = {0, 0};  // pairs of zeros
-      uint32_t pk[BKV / 2];
 #pragma unroll
-      for (int u = 0; u < BKV / 2; ++u) {
-        const float2 x = unpack2(fma2(pack2(__uint_as_float(v[2 * u]), __uint_as_float(v[2 * u + 1])), sc, nm));
-        const float e0 = ptx::ex2_ftz(x.x), e1 = ptx::ex2_ftz(x.y);
-        ls[u & 1] = add2(ls[u & 1], pack2(e0, e1));
-        pk[u] = ptx::pack_bf16(e0, e1);
+      for (int h = 0; h < 2; ++h) {
+        if (h == 1) load_half(1);
+        uint32_t pk[16];
+#pragma unroll
+        for (int u = 0; u < 16; ++u) {
+          const float2 x = unpack2(fma2(pack2(__uint_as_float(v[2 * u]), __uint_as_float(v[2 * u + 1])), sc, nm));
+          const float e0 = ptx::ex2_ftz(x.x), e1 = ptx::ex2_ftz(x.y);
+          ls[u & 1] = add2(ls[u & 1], pack2(e0, e1));
+          pk[u] = ptx::pack_bf16(e0, e1);
+        }
+        ptx::tmem_st_32x32b_x16(tS + lane_base + h * 16, pk);
       }
       const float2 lsum = unpack2(add2(ls[0], ls[1]));
       l += lsum.x + lsum.y;
-      // P buffer j & 1 was last read by P_{j-2} V_{j-2}
-      if (j >= 2 && !wait_all(&pv_done[j & 1], ((j - 2) >> 1) & 1)) { ok = false; break; }
-      ptx::tmem_st_32x32b_x32(tP + (j & 1) * (BKV / 2) + lane_base, pk);
       ptx::tmem_st_wait();
       ptx::tc_fence_before();
-      ptx::mbar_arrive(&p_full[j & 1]);
+      ptx::mbar_arrive(p_full);
     }
+    pdl_trigger();  // behind the main loop: see common.cuh
     // epilogue: O / l -> ctx (bf16) as 128-byte-swizzled rows over the Q
     // tile (the last S product has read it), stored by one TMA that drops the
     // rows past S; the log-sum-exp directly
-    if (ok && wait_all(&pv_done[(n_kt - 1) & 1], ((n_kt - 1) >> 1) & 1)) {
+    if (ok && wait_all(pv_done, (n_kt - 1) & 1)) {
       ptx::tc_fence_after();
       const float inv = 1.f / l;
       const int q = q0 + r;
       const uint32_t orow = ptx::smem_u32(smem + F_Q_OFF) + r * 128;
 #pragma unroll
       for (int c = 0; c < HD / 32; ++c) {
-        uint32_t o[32];
-        ptx::tmem_ld_32x32b_x32(tO + lane_base + c * 32, o);
+        ptx::tmem_ld_32x32b_x32(tO + lane_base + c * 32, v);
         ptx::tmem_ld_wait();
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           uint32_t w[4];
 #pragma unroll
           for (int t = 0; t < 4; ++t)
-            w[t] = ptx::pack_bf16(__uint_as_float(o[8 * u + 2 * t]) * inv,
-                                  __uint_as_float(o[8 * u + 2 * t + 1]) * inv);
+            w[t] = ptx::pack_bf16(__uint_as_float(v[8 * u + 2 * t]) * inv,
+                                  __uint_as_float(v[8 * u + 2 * t + 1]) * inv);
           ptx::st_shared_v4(orow + (((c * 4 + u) ^ (r & 7)) << 4), w[0], w[1], w[2], w[3]);
         }
       }
@@ -340,6 +313,197 @@ __global__ void __launch_bounds__(NTHR, 2) attn_fwd_tc(const __grid_constant__ C
     asm volatile("bar.sync 1, 128;" ::: "memory");  // the four softmax warps
     if (warp == 2 && lane == 0) {
       ptx::tma_store_3d(&tmOut, smem + F_Q_OFF, a * HD, q0, b);
+      ptx::bulk_commit_group();
+      ptx::bulk_wait_group_read0();  // before the CTA's memory goes
+    }
+  }
+  ptx::tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    ptx::tc_fence_after();
+    ptx::tmem_dealloc(tmem, F_TMEM_COLS);
+  }
+}
+
+// ----------------------------------------- forward, sequences up to 128
+// One 128-key tile: S = Q K^T (N = 128), one softmax pass, O = P V.  P (bf16
+// pairs) goes over the scores' first 64 columns as they are consumed, O over the
+// rest: 128 TMEM columns and 48 KiB, four CTAs an SM.  Latency-bound: it saves the
+// second tile's round trip through the tensor pipe.
+constexpr int FS_Q = 0, FS_K = Q_BYTES, FS_V = 2 * Q_BYTES, FS_BAR = 3 * Q_BYTES;
+constexpr int FS_SMEM = FS_BAR + 64 + 1024;
+static_assert(F_CTAS * (FS_SMEM + 1024) <= 233472, "four forward CTAs per SM");
+
+__global__ void __launch_bounds__(NTHR, F_CTAS) attn_fwd_short_tc(const __grid_constant__ CUtensorMap tmQKV,
+                                                                  const __grid_constant__ CUtensorMap tmOut,
+                                                                  const FwdParams p) {
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t raw_addr = ptx::smem_u32(smem_raw);
+  uint8_t* smem = smem_raw + (((raw_addr + 1023u) & ~1023u) - raw_addr);
+  uint64_t* qk_full = reinterpret_cast<uint64_t*>(smem + FS_BAR);
+  uint64_t* v_full = qk_full + 1;
+  uint64_t* s_full = v_full + 1;   // S complete
+  uint64_t* p_full = s_full + 1;   // P in tensor memory
+  uint64_t* o_full = p_full + 1;   // O complete
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(o_full + 1);
+
+  const int a = blockIdx.x, b = blockIdx.y;
+  const int S = p.S, H = p.H;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int row0 = b * S;
+  const uint64_t lim = p.timeout_ns;
+  if (threadIdx.x == 0) {
+    ptx::mbar_init(qk_full, 1);
+    ptx::mbar_init(v_full, 1);
+    ptx::mbar_init(s_full, 1);
+    ptx::mbar_init(p_full, 128);
+    ptx::mbar_init(o_full, 1);
+    ptx::fence_mbar_init();
+    ptx::fence_proxy_async_smem();
+    ptx::prefetch_tensormap(&tmQKV);
+  }
+  if (warp == 1) {
+    ptx::tmem_alloc(tmem_slot, F_TMEM_COLS);
+    ptx::tmem_relinquish();
+  }
+  ptx::tc_fence_before();
+  __syncthreads();
+  ptx::tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  const uint32_t tS = tmem, tO = tmem + 64;
+  pdl_wait();
+  int len = p.lens[b];
+  if (len < 1 || len > S) {
+    if (p.status && threadIdx.x == 0) atomicOr(p.status, kStatusBadLength);
+    len = len < 1 ? 1 : S;
+  }
+  const int chunks = (len + 31) / 32;  // 32-key chunks with a valid key
+
+  if (warp == 0) {
+    if (lane == 0) {
+      ptx::mbar_arrive_expect_tx(qk_full, 2 * Q_BYTES);
+      ptx::tma_load_2d(smem + FS_Q, &tmQKV, qk_full, a * HD, row0);
+      ptx::tma_load_2d(smem + FS_K, &tmQKV, qk_full, H + a * HD, row0);
+      ptx::mbar_arrive_expect_tx(v_full, Q_BYTES);
+      ptx::tma_load_2d(smem + FS_V, &tmQKV, v_full, 2 * H + a * HD, row0);
+      // bounded waits for the copies before the CTA may exit
+      ptx::mbar_wait(qk_full, 0, lim, p.status, kWaitHint);
+      ptx::mbar_wait(v_full, 0, lim, p.status, kWaitHint);
+    }
+  } else if (warp == 1) {
+    // (whole warp, one elected lane issuing: as above)
+    constexpr uint32_t idS = ptx::idesc_bf16_f32(BQ, 128, false, false);
+    constexpr uint32_t idO = ptx::idesc_bf16_f32(BQ, HD, false, true);
+    const bool issuer = ptx::elect_one();
+    const uint64_t dq = ptx::smem_desc_sw128(ptx::smem_u32(smem + FS_Q), 16, 1024);
+    const uint64_t dk = ptx::smem_desc_sw128(ptx::smem_u32(smem + FS_K), 16, 1024);
+    const uint64_t dv = ptx::smem_desc_sw128(ptx::smem_u32(smem + FS_V), 8192, 1024);
+    auto wait = [&](uint64_t* bar) {
+      return __all_sync(0xffffffffu, ptx::mbar_wait(bar, 0, lim, p.status, kWaitHint));
+    };
+    bool ok = wait(qk_full);
+    if (ok) {
+      ptx::tc_fence_after();
+      if (issuer) {
+#pragma unroll
+        for (int kk = 0; kk < HD / 16; ++kk) ptx::tc_mma_f16(tS, dq + kk * 2, dk + kk * 2, idS, kk > 0 ? 1u : 0u);
+        ptx::tc_commit(s_full);
+      }
+      __syncwarp();
+      ok = wait(v_full) && wait(p_full);
+    }
+    if (ok) {
+      ptx::tc_fence_after();
+      if (issuer) {
+        for (int kk = 0; kk < 2 * chunks; ++kk)
+          ptx::tc_mma_f16_tmem_a(tO, tS + kk * 8, dv + kk * 128, idO, kk > 0 ? 1u : 0u);
+      }
+      __syncwarp();
+    }
+    // also on a timeout: what was issued has to finish before TMEM is released
+    if (issuer) ptx::tc_commit(o_full);
+    __syncwarp();
+    ptx::mbar_wait(o_full, 0, lim, p.status, kWaitHint);
+  } else {
+    const int q4 = warp & 3;
+    const int r = q4 * 32 + lane;  // query row == TMEM lane
+    const uint32_t lane_base = static_cast<uint32_t>(q4 * 32) << 16;
+    const float sl2 = LOG2E * 0.125f;
+    auto wait_all = [&](uint64_t* bar) {
+      return __all_sync(0xffffffffu, ptx::mbar_wait(bar, 0, lim, p.status, kWaitHint));
+    };
+    float m = -INFINITY, l = 0.f;
+    uint32_t v[32];
+    auto load_chunk = [&](int c) {
+      ptx::tmem_ld_32x32b_x32(tS + lane_base + c * 32, v);
+      ptx::tmem_ld_wait();
+      if (len < (c + 1) * 32) {  // CTA-uniform
+#pragma unroll
+        for (int i = 0; i < 32; ++i)
+          if (c * 32 + i >= len) v[i] = 0xff800000u;  // -inf: excluded from the max, P = 0
+      }
+    };
+    bool ok = wait_all(s_full);
+    if (ok) {
+      ptx::tc_fence_after();
+      // row max, the first chunk last: it stays in registers
+#pragma unroll 1
+      for (int c = chunks - 1; c >= 0; --c) {
+        load_chunk(c);
+        float m4[4] = {m, __uint_as_float(v[0]), __uint_as_float(v[1]), __uint_as_float(v[2])};
+#pragma unroll
+        for (int i = 3; i < 32; ++i) m4[i & 3] = fmaxf(m4[i & 3], __uint_as_float(v[i]));
+        m = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
+      }
+      m *= sl2;
+      const uint64_t nm = pack2(-m, -m), sc = pack2(sl2, sl2);
+      uint64_t ls[2] = {0, 0};  // pairs of zeros
+#pragma unroll 1
+      for (int c = 0; c < chunks; ++c) {
+        if (c > 0) load_chunk(c);
+        uint32_t pk[16];
+#pragma unroll
+        for (int u = 0; u < 16; ++u) {
+          const float2 x = unpack2(fma2(pack2(__uint_as_float(v[2 * u]), __uint_as_float(v[2 * u + 1])), sc, nm));
+          const float e0 = ptx::ex2_ftz(x.x), e1 = ptx::ex2_ftz(x.y);
+          ls[u & 1] = add2(ls[u & 1], pack2(e0, e1));
+          pk[u] = ptx::pack_bf16(e0, e1);
+        }
+        ptx::tmem_st_32x32b_x16(tS + lane_base + c * 16, pk);  // over chunk c / 2, which has been read
+      }
+      const float2 lsum = unpack2(add2(ls[0], ls[1]));
+      l = lsum.x + lsum.y;
+      ptx::tmem_st_wait();
+      ptx::tc_fence_before();
+      ptx::mbar_arrive(p_full);
+      ok = wait_all(o_full);
+    }
+    pdl_trigger();  // behind the products: see common.cuh
+    // O / l -> ctx as in the kernel above
+    if (ok) {
+      ptx::tc_fence_after();
+      const float inv = 1.f / l;
+      const uint32_t orow = ptx::smem_u32(smem + FS_Q) + r * 128;
+#pragma unroll
+      for (int c = 0; c < HD / 32; ++c) {
+        ptx::tmem_ld_32x32b_x32(tO + lane_base + c * 32, v);
+        ptx::tmem_ld_wait();
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          uint32_t w[4];
+#pragma unroll
+          for (int t = 0; t < 4; ++t)
+            w[t] = ptx::pack_bf16(__uint_as_float(v[8 * u + 2 * t]) * inv,
+                                  __uint_as_float(v[8 * u + 2 * t + 1]) * inv);
+          ptx::st_shared_v4(orow + (((c * 4 + u) ^ (r & 7)) << 4), w[0], w[1], w[2], w[3]);
+        }
+      }
+      if (r < S) p.lse[(static_cast<int64_t>(b) * p.A + a) * S + r] = m + log2f(l);
+    }
+    ptx::fence_proxy_async_smem();  // the staged rows -> the TMA store
+    asm volatile("bar.sync 1, 128;" ::: "memory");  // the four softmax warps
+    if (warp == 2 && lane == 0) {
+      ptx::tma_store_3d(&tmOut, smem + FS_Q, a * HD, 0, b);
       ptx::bulk_commit_group();
       ptx::bulk_wait_group_read0();  // before the CTA's memory goes
     }
@@ -1304,6 +1468,16 @@ sky_status attention_fwd_tc(const void* qkv, const int32_t* lens, int B, int S, 
             SKY_ERR_UNSUPPORTED, "attention buffers must be 16-byte aligned");
   CUtensorMap tq, tkv, tout;
   const int64_t T = static_cast<int64_t>(B) * S;
+  if (S <= 128 && B <= 65535) {  // one tile a sequence
+    SKY_CHECK(head_map(&tq, qkv, T, 3 * H, BQ) && seq_map(&tout, ctx, B, S, H, BQ), SKY_ERR_CUDA,
+              "cuTensorMapEncodeTiled failed for the attention operands");
+    static cudaError_t at = cudaFuncSetAttribute(attn_fwd_short_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, FS_SMEM);
+    if (at != cudaSuccess) return cuda_fail(at, "attention smem attribute");
+    FwdParams p{S, H, A, lens, static_cast<__nv_bfloat16*>(ctx), lse, status, timeout_ns};
+    const cudaError_t e = launch_pdl(attn_fwd_short_tc, dim3(A, B), dim3(NTHR), FS_SMEM, stream, 1, tq, tout, p);
+    count_launches(1);
+    return e == cudaSuccess ? SKY_OK : cuda_fail(e, "tensor-core attention forward launch");
+  }
   SKY_CHECK(head_map(&tq, qkv, T, 3 * H, BQ) && head_map(&tkv, qkv, T, 3 * H, BKV) &&
                 seq_map(&tout, ctx, B, S, H, BQ),
             SKY_ERR_CUDA,
@@ -1312,11 +1486,7 @@ sky_status attention_fwd_tc(const void* qkv, const int32_t* lens, int B, int S, 
                                                  F_SMEM);
   if (attr != cudaSuccess) return cuda_fail(attr, "attention smem attribute");
   dim3 grid(ceil_div(S, BQ), A, B);
-  // one wave of CTAs: the next kernel's would only crowd in beside them; over
-  // several waves it starts when the last CTAs have (S = 2048, 1024 CTAs: 72.0
-  // us a launch, 73.4 with the late trigger)
-  const bool one_wave = static_cast<int64_t>(grid.x) * A * B <= 2 * sm_count();
-  FwdParams p{S, H, A, lens, static_cast<__nv_bfloat16*>(ctx), lse, status, timeout_ns, one_wave};
+  FwdParams p{S, H, A, lens, static_cast<__nv_bfloat16*>(ctx), lse, status, timeout_ns};
   const cudaError_t e = launch_pdl(attn_fwd_tc, grid, dim3(NTHR), F_SMEM, stream, 1, tq, tkv, tout, p);
   count_launches(1);
   return e == cudaSuccess ? SKY_OK : cuda_fail(e, "tensor-core attention forward launch");
