@@ -16,6 +16,7 @@ namespace gemm {
 // possibly on another stream ordered after this launch).
 // resid (optional, fp32 output of the STORE epilogue, no split): C = acc +
 // bias + resid[m, n], added in that order (the residual branch of Sec. II-C).
+// resid == C (XTW form, no bias): C += product, which may be split.
 // With `ln`, resid holds the pre-LayerNorm sum u of the previous sub-layer and
 // the residual added is its LayerNorm output, recomputed in the epilogue from
 // the row statistics: gamma[n] * ((u[m, n] - mean[m]) * rstd[m]) + beta[n]
@@ -44,7 +45,7 @@ struct ClusterPlan {
   int bn, ks;
 };
 // Whether a product goes to the cluster kernel, and with which tiles.
-// may_split: an fp32 output without bias or residual; colpart: column sums per
+// may_split: an fp32 output without bias or residual (C += product is none); colpart: column sums per
 // 32 rows are wanted.
 bool plan_cluster(sky_gemm_form form, int M, int N, int K, bool may_split, bool colpart, int sms,
                   ClusterPlan* out);

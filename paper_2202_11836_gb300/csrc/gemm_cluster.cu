@@ -106,6 +106,14 @@ __device__ __forceinline__ float4 ld_stream_f4(const float* p) {
                : "l"(p));
   return v;
 }
+// (also of what the kernel itself overwrites later)
+__device__ __forceinline__ float4 ld_own_f4(const float* p) {
+  float4 v;
+  asm volatile("ld.global.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "l"(p));
+  return v;
+}
 __device__ __forceinline__ float4 bf4(const __nv_bfloat16* p) {
   const uint2 raw = *reinterpret_cast<const uint2*>(p);
   const float2 a = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(&raw)[0]);
@@ -114,8 +122,9 @@ __device__ __forceinline__ float4 bf4(const __nv_bfloat16* p) {
 }
 
 // Epilogues, one instantiation each: bias only (fp32 or bf16 output), bias +
-// GELU, GELU', and bias + fp32 residual or LayerNorm residual (fp32 output).
-enum { E_STORE, E_GELU, E_GELU_BWD, E_RESID };
+// GELU, GELU', bias + fp32 residual or LayerNorm residual (fp32 output), and
+// C += product (fp32).
+enum { E_STORE, E_GELU, E_GELU_BWD, E_RESID, E_ADD };
 
 template <bool A_MN, bool B_MN, class TL, int EP>
 __global__ void __launch_bounds__(C_THREADS, 2)
@@ -180,7 +189,7 @@ __global__ void __launch_bounds__(C_THREADS, 2)
   bool ok = true;
   // what the epilogue needs beside the sums, fetched under the main loop
   float4 bias4 = make_float4(0.f, 0.f, 0.f, 0.f), gm4 = bias4, be4 = bias4;
-  float4 pre[EP == E_RESID ? TL::GT : 1];
+  float4 pre[EP == E_RESID || EP == E_ADD ? TL::GT : 1];
   float mu[EP == E_RESID ? TL::GT : 1], rs[EP == E_RESID ? TL::GT : 1];
   uint2 pre_g[EP == E_GELU_BWD ? TL::GT : 1];
 
@@ -280,7 +289,7 @@ __global__ void __launch_bounds__(C_THREADS, 2)
         be4 = bf4(p.ln_beta + col);
       }
     }
-    if constexpr (EP == E_RESID || EP == E_GELU_BWD) {
+    if constexpr (EP == E_RESID || EP == E_GELU_BWD || EP == E_ADD) {
 #pragma unroll
       for (int i = 0; i < TL::GT; ++i) {
         const int rl = row_lo + et / GPR + i * RSTEP, row = m0 + rl;
@@ -290,6 +299,8 @@ __global__ void __launch_bounds__(C_THREADS, 2)
           pre[i] = in ? ld_stream_f4(p.resid + off) : make_float4(0.f, 0.f, 0.f, 0.f);
           mu[i] = in && p.ln_mean ? __ldg(p.ln_mean + row) : 0.f;
           rs[i] = in && p.ln_mean ? __ldg(p.ln_rstd + row) : 0.f;
+        } else if constexpr (EP == E_ADD) {
+          pre[i] = in ? ld_own_f4(static_cast<const float*>(p.C) + off) : make_float4(0.f, 0.f, 0.f, 0.f);
         } else {
           pre_g[i] = in ? __ldg(reinterpret_cast<const uint2*>(p.aux + off)) : make_uint2(0u, 0u);
         }
@@ -420,9 +431,11 @@ __global__ void __launch_bounds__(C_THREADS, 2)
           } else {
             v[u].x += pre[i].x; v[u].y += pre[i].y; v[u].z += pre[i].z; v[u].w += pre[i].w;
           }
+        } else if constexpr (EP == E_ADD) {
+          v[u].x += pre[i].x; v[u].y += pre[i].y; v[u].z += pre[i].z; v[u].w += pre[i].w;
         }
         if (!ok) continue;
-        if (EP == E_RESID || (EP == E_STORE && p.out_f32))
+        if (EP == E_RESID || EP == E_ADD || (EP == E_STORE && p.out_f32))
           *reinterpret_cast<float4*>(static_cast<float*>(p.C) + off) = v[u];
         else
           *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(p.C) + off) =
@@ -479,6 +492,9 @@ template <bool A_MN, bool B_MN, class TL>
 cudaError_t launch_epi(int epi, ClusterParams& p, const CUtensorMap& ta, const CUtensorMap& tb, cudaStream_t st) {
   if (epi == SKY_EPI_BIAS_GELU) return launch_one<A_MN, B_MN, TL, E_GELU>(p, ta, tb, st);
   if (epi == SKY_EPI_GELU_BWD) return launch_one<A_MN, B_MN, TL, E_GELU_BWD>(p, ta, tb, st);
+  if constexpr (A_MN) {
+    if (p.resid && p.resid == p.C) return launch_one<A_MN, B_MN, TL, E_ADD>(p, ta, tb, st);
+  }
   if (p.resid) return launch_one<A_MN, B_MN, TL, E_RESID>(p, ta, tb, st);
   return launch_one<A_MN, B_MN, TL, E_STORE>(p, ta, tb, st);
 }
@@ -488,7 +504,9 @@ cudaError_t launch_plan(const ClusterPlan& pl, int epi, ClusterParams& p, const 
                         const CUtensorMap& tb, cudaStream_t st) {
   if (pl.pair) return launch_epi<A_MN, B_MN, Tiling<true, 128, 2>>(epi, p, ta, tb, st);
   if constexpr (A_MN) {
-    if (pl.bn == 128) return launch_one<A_MN, B_MN, Tiling<false, 128, 1>, E_STORE>(p, ta, tb, st);
+    if (pl.bn == 128)
+      return p.resid ? launch_one<A_MN, B_MN, Tiling<false, 128, 1>, E_ADD>(p, ta, tb, st)
+                     : launch_one<A_MN, B_MN, Tiling<false, 128, 1>, E_STORE>(p, ta, tb, st);
   }
   switch (pl.ks) {
     case 6: return launch_epi<A_MN, B_MN, Tiling<false, 64, 6>>(epi, p, ta, tb, st);

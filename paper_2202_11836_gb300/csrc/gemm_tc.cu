@@ -109,9 +109,9 @@ __device__ __forceinline__ uint2 ld_nc_u2(const void* p) {
                : "l"(p));
   return v;
 }
-__device__ __forceinline__ float4 ld_nc_f4(const float* p) {
+__device__ __forceinline__ float4 ld_own_f4(const float* p) {
   float4 v;
-  asm volatile("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
+  asm volatile("ld.global.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
                : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
                : "l"(p));
   return v;
@@ -374,7 +374,7 @@ __global__ void __launch_bounds__(Shape<EPI, PAIR, TBN>::THREADS, 1)
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
           const int row = m0 + q * 32 + 4 * i + rsub;
-          d[i] = (col < p.N && row < p.M) ? ld_nc_f4(rp + static_cast<int64_t>(row) * p.N + col)
+          d[i] = (col < p.N && row < p.M) ? ld_own_f4(rp + static_cast<int64_t>(row) * p.N + col)
                                           : make_float4(0.f, 0.f, 0.f, 0.f);
         }
       };
@@ -586,11 +586,11 @@ __global__ void __launch_bounds__(Shape<EPI, PAIR, TBN>::THREADS, 1)
 }
 
 // Fixed-order sum of split-K partials: out[i] = sum_s ws[s][i], added in
-// split order.  SPLITS > 0: every split's load of a vector is issued before
+// split order (add: out[i] += that sum).  SPLITS > 0: every split's load of a vector is issued before
 // the first add (a loop over a run-time count would wait for each load in
 // turn); SPLITS == 0: any count.
 template <int SPLITS>
-__global__ void splitk_reduce_kernel(const float* __restrict__ ws, int splits, int64_t n,
+__global__ void splitk_reduce_kernel(const float* __restrict__ ws, int splits, int64_t n, bool add,
                                      float* __restrict__ out) {
   pdl_wait();
   pdl_trigger();
@@ -614,13 +614,17 @@ __global__ void splitk_reduce_kernel(const float* __restrict__ ws, int splits, i
         acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
       }
     }
+    if (add) {
+      const float4 v = reinterpret_cast<const float4*>(out)[i];
+      acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
+    }
     reinterpret_cast<float4*>(out)[i] = acc;
   }
   for (int64_t i = n4 * 4 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
     float acc = ws[i];
     for (int s = 1; s < splits; ++s) acc += ws[s * n + i];
-    out[i] = acc;
+    out[i] = add ? acc + out[i] : acc;
   }
 }
 
@@ -803,7 +807,10 @@ sky_status launch_bf16(sky_gemm_form form, int M, int N, int K, const void* A, c
   const int sms = sm_count();
   SKY_CHECK(sms > 0, SKY_ERR_CUDA, "no CUDA device");
 
-  const bool may_split = out_f32 && epi == SKY_EPI_STORE && bias == nullptr && resid == nullptr;
+  const bool add = resid && resid == C;  // C += product
+  SKY_CHECK(!add || (form == SKY_GEMM_XTW && !bias && !ln), SKY_ERR_UNSUPPORTED,
+            "only a weight gradient is added to its output");
+  const bool may_split = out_f32 && epi == SKY_EPI_STORE && bias == nullptr && (!resid || add);
   if (!colsum) {  // small and mid-sized products: the cluster kernel
     ClusterPlan pl;
     bool here = plan_cluster(form, M, N, K, may_split, deferred_rows != nullptr, sms, &pl);
@@ -884,7 +891,7 @@ sky_status launch_bf16(sky_gemm_form form, int M, int N, int K, const void* A, c
     if (deferred_rows) *deferred_rows = colpart_rows;
   }
   p.bias = static_cast<const __nv_bfloat16*>(bias);
-  p.resid = resid;
+  p.resid = add && p.splits > 1 ? nullptr : resid;
   if (ln) {
     p.ln_mean = ln->mean;
     p.ln_rstd = ln->rstd;
@@ -928,13 +935,13 @@ sky_status launch_bf16(sky_gemm_form form, int M, int N, int K, const void* A, c
     const float* wsf = static_cast<const float*>(ws);
     float* cf = static_cast<float*>(C);
     switch (p.splits) {
-      case 2: e = launch_pdl(splitk_reduce_kernel<2>, dim3(blocks), dim3(256), 0, stream, 1, wsf, p.splits, n, cf); break;
-      case 3: e = launch_pdl(splitk_reduce_kernel<3>, dim3(blocks), dim3(256), 0, stream, 1, wsf, p.splits, n, cf); break;
-      case 4: e = launch_pdl(splitk_reduce_kernel<4>, dim3(blocks), dim3(256), 0, stream, 1, wsf, p.splits, n, cf); break;
-      case 5: e = launch_pdl(splitk_reduce_kernel<5>, dim3(blocks), dim3(256), 0, stream, 1, wsf, p.splits, n, cf); break;
-      case 6: e = launch_pdl(splitk_reduce_kernel<6>, dim3(blocks), dim3(256), 0, stream, 1, wsf, p.splits, n, cf); break;
-      case 8: e = launch_pdl(splitk_reduce_kernel<8>, dim3(blocks), dim3(256), 0, stream, 1, wsf, p.splits, n, cf); break;
-      default: e = launch_pdl(splitk_reduce_kernel<0>, dim3(blocks), dim3(256), 0, stream, 1, wsf, p.splits, n, cf); break;
+      case 2: e = launch_pdl(splitk_reduce_kernel<2>, dim3(blocks), dim3(256), 0, stream, 1, wsf, p.splits, n, add, cf); break;
+      case 3: e = launch_pdl(splitk_reduce_kernel<3>, dim3(blocks), dim3(256), 0, stream, 1, wsf, p.splits, n, add, cf); break;
+      case 4: e = launch_pdl(splitk_reduce_kernel<4>, dim3(blocks), dim3(256), 0, stream, 1, wsf, p.splits, n, add, cf); break;
+      case 5: e = launch_pdl(splitk_reduce_kernel<5>, dim3(blocks), dim3(256), 0, stream, 1, wsf, p.splits, n, add, cf); break;
+      case 6: e = launch_pdl(splitk_reduce_kernel<6>, dim3(blocks), dim3(256), 0, stream, 1, wsf, p.splits, n, add, cf); break;
+      case 8: e = launch_pdl(splitk_reduce_kernel<8>, dim3(blocks), dim3(256), 0, stream, 1, wsf, p.splits, n, add, cf); break;
+      default: e = launch_pdl(splitk_reduce_kernel<0>, dim3(blocks), dim3(256), 0, stream, 1, wsf, p.splits, n, add, cf); break;
     }
     count_launches(1);
     if (e != cudaSuccess) return cuda_fail(e, "splitk_reduce launch");

@@ -209,9 +209,8 @@ __global__ void __launch_bounds__(LN_WARPS * 32) ln_bwd_kernel(
 
 // Element-wise passes, four elements a thread in 16-byte accesses when the
 // pointers allow it (VEC; the last n % 4 elements, or all without VEC, one by
-// one).  HBM-bound: accumulating a base-width layer's 7.1 M gradients, 12 bytes
-// each, took 18.7 us with 4-byte accesses against 13 at the copy rate; 4
-// micro-batches of 3 such layers, with nine of these passes, 1815 -> 1795 us.
+// one).  HBM-bound: adding a base-width layer's 7.1 M fp32 gradients to others, 12
+// bytes each, took 18.7 us with 4-byte accesses; so 12 to 13, the copy rate.
 __device__ __forceinline__ float4 load4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 __device__ __forceinline__ float4 load4(const __nv_bfloat16* p) {
   const uint2 r = *reinterpret_cast<const uint2*>(p);
@@ -467,7 +466,7 @@ __global__ void __launch_bounds__(RP_WARPS * 32) reduce_partials(const float* __
 }
 
 // Several fixed-order column reductions in one launch: segment y = blockIdx.y
-// computes segs[y].out[n] = sum_b segs[y].part[b][n] over its rows, exactly
+// computes segs[y].out[n] = (segs.add: +=) sum_b segs[y].part[b][n] over its rows, exactly
 // as reduce_partials does (so the same partials give the same bits).
 __global__ void __launch_bounds__(RP_WARPS * 32) reduce_segments(const ColSegments segs) {
   pdl_wait();
@@ -499,7 +498,7 @@ __global__ void __launch_bounds__(RP_WARPS * 32) reduce_segments(const ColSegmen
     float t = 0.f;
 #pragma unroll
     for (int j = 0; j < RP_WARPS; ++j) t += red[j][lane];
-    sg.out[n] = t;
+    sg.out[n] = segs.add ? sg.out[n] + t : t;
   }
 }
 

@@ -47,6 +47,7 @@ constexpr int kMaxColSegments = 8;
 struct ColSegments {
   ColSegment seg[kMaxColSegments];
   int n;
+  bool add;  // out += the sums
 };
 sky_status reduce_column_segments(const ColSegments& segs, cudaStream_t st);
 sky_status add_f32(const float* a, const float* b, int64_t n, sky_dtype out_dt, void* out,
