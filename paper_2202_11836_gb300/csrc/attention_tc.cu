@@ -14,13 +14,22 @@
 // memory.  Because a thread owns a whole query row, the row max and row sum
 // need no shuffles.
 //
-// The chain of a tile is serial inside a CTA; what overlaps it is other CTAs.
-// With P over S, a CTA needs 128 TMEM columns, 49 KiB of shared memory (two K/V
-// stages) and 80 registers a thread (half a row's scores at a time, the high
-// half read twice), so four share an SM.  Two CTAs with S and P double-buffered
-// inside each were 69.1 us at S = 2048 (16 heads, 4 sequences), three of these
-// 80.7, four 63.4.  No pipe is full then (ncu: issue 46%, tensor 37%, XU 37% of
-// the active cycles).  The exponent offset m of a row is only raised when the
+// A tile's chain (S, softmax, P V) is serial, so tiles have to overlap.  Two forms
+// of the kernel, chosen by the launcher, do it:
+//   two score buffers (NS = 2): S_{j+1} runs beside the softmax of tile j.  256
+//     TMEM columns, so two CTAs an SM; a tile takes 0.53 us alone (S = 2048).
+//   one (NS = 1): P over the only S; 128 TMEM columns, 49 KiB of shared memory and
+//     80 registers a thread (half a row's scores at a time, the high half read
+//     twice), so four CTAs overlap on an SM.  A tile takes 0.85 us alone, but a full
+//     SM finishes more of them: 16 heads x 4 full sequences of 2048, 81 us against
+//     86.  No pipe is full then (ncu: issue 46%, tensor 37%, XU 37% of the active
+//     cycles); three CTAs an SM were slower.
+// Where the query blocks are few, KS = 2 or 4 CTAs of a cluster share a block's keys:
+// each leaves its part of O, m and l in shared memory, and each finishes 128 / KS of
+// the rows from its peers' parts.  4 heads x 2048: 19.9 us before, 17.3 unsplit, 10.3
+// in four; the combination costs 2 us and more with more clusters.
+//
+// The exponent offset m of a row is only raised when the
 // tile's max exceeds it by more than 2^8 (a factor 256 in P): then O and the row
 // sum are rescaled in TMEM.  Otherwise P may exceed 1 by at most that factor,
 // which bf16 and the fp32 sums carry with the same relative precision; the final
@@ -30,7 +39,9 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
+#include <cfloat>
 #include <mutex>
+#include <type_traits>
 
 #include "common.cuh"
 #include "ptx.cuh"
@@ -48,9 +59,7 @@ constexpr int NTHR = 192;
 constexpr int NSM_B = 256;              // softmax threads in the backward kernels
 // Backward CTAs: warp 0 TMA, warp 1 issues the score products (S and dP),
 // warps 2..9 softmax, warp 10 issues the accumulating products (dQ, or dV
-// and dK).  One thread issues a tcgen05.mma only about every 100 cycles,
-// while an M=128, N=64, K=16 product keeps the tensor pipe busy for about
-// 32, so the two kinds of product are issued side by side by two warps.
+// and dK), so that neither kind waits behind the other's barriers.
 constexpr int NTHR_B = 352;
 constexpr float LOG2E = 1.4426950408889634f;
 // Suspend-time hint (ns) of every mbarrier wait: a waiting thread sleeps
@@ -58,17 +67,23 @@ constexpr float LOG2E = 1.4426950408889634f;
 // softmax warps (the critical path) share with the producer and MMA threads.
 constexpr uint32_t kWaitHint = 10000;
 
-// forward shared-memory layout (offsets from a 1024-byte aligned base)
-constexpr int F_STAGES = 2;
-constexpr int F_Q_OFF = 0;
-constexpr int F_KV_OFF = F_Q_OFF + Q_BYTES;                  // [F_STAGES] x {K, V}
-constexpr int F_BAR_OFF = F_KV_OFF + F_STAGES * 2 * KV_BYTES;
-constexpr int F_SMEM = F_BAR_OFF + 256 + 1024;
-// S: [0, 64), then P as bf16 pairs in [0, 32) (the A operand of P V, read from
-// tensor memory); O: [64, 128)
-constexpr int F_TMEM_COLS = 128;
-constexpr int F_CTAS = 4;  // per SM
-static_assert(F_CTAS * (F_SMEM + 1024) <= 233472, "four forward CTAs per SM");
+// Forward kernel with NS score buffers: four CTAs an SM with one, two with two.
+// Shared-memory layout (offsets from a 1024-byte aligned base).  TMEM: S_0, then
+// S_1, 64 columns each, of which P as bf16 pairs takes the first 32 (the A operand
+// of P V, read from tensor memory); O: 64 columns behind them.
+template <int NS>
+struct FwdShape {
+  static constexpr int CTAS = NS == 1 ? 4 : 2;  // per SM
+  static constexpr int STAGES = NS + 1;         // K/V ring
+  static constexpr int Q_OFF = 0;
+  static constexpr int KV_OFF = Q_OFF + Q_BYTES;  // [STAGES] x {K, V}
+  static constexpr int BAR_OFF = KV_OFF + STAGES * 2 * KV_BYTES;
+  static constexpr int ML_OFF = BAR_OFF + 256;    // split keys: m and l of each row
+  static constexpr int SMEM = ML_OFF + BQ * 8 + 1024;
+  static constexpr int TMEM_COLS = 128 * NS;
+};
+static_assert(FwdShape<1>::CTAS * (FwdShape<1>::SMEM + 1024) <= 233472, "four forward CTAs per SM");
+static_assert(FwdShape<1>::STAGES * 2 * KV_BYTES >= BQ * HD * 4, "a partial O goes over the K/V stages");
 constexpr float kRescaleLog2 = 8.f;
 
 struct FwdParams {
@@ -80,22 +95,24 @@ struct FwdParams {
   uint64_t timeout_ns;
 };
 
-__global__ void __launch_bounds__(NTHR, F_CTAS) attn_fwd_tc(const __grid_constant__ CUtensorMap tmQ,
+template <int KS, int NS>
+__global__ void __launch_bounds__(NTHR, FwdShape<NS>::CTAS) attn_fwd_tc(const __grid_constant__ CUtensorMap tmQ,
                                                     const __grid_constant__ CUtensorMap tmKV,
                                                     const __grid_constant__ CUtensorMap tmOut,
                                                     const FwdParams p) {
+  using SH = FwdShape<NS>;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw_addr = ptx::smem_u32(smem_raw);
   uint8_t* smem = smem_raw + (((raw_addr + 1023u) & ~1023u) - raw_addr);
-  uint64_t* q_full = reinterpret_cast<uint64_t*>(smem + F_BAR_OFF);
+  uint64_t* q_full = reinterpret_cast<uint64_t*>(smem + SH::BAR_OFF);
   uint64_t* kv_full = q_full + 1;
-  uint64_t* kv_empty = kv_full + F_STAGES;
-  uint64_t* s_full = kv_empty + F_STAGES;  // S_j complete
-  uint64_t* p_full = s_full + 1;           // P_j in tensor memory
-  uint64_t* pv_done = p_full + 1;          // O += P_j V_j complete
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(pv_done + 1);
+  uint64_t* kv_empty = kv_full + SH::STAGES;
+  uint64_t* s_full = kv_empty + SH::STAGES;  // [NS] S_j complete
+  uint64_t* p_full = s_full + NS;            // [NS] P_j in tensor memory
+  uint64_t* pv_done = p_full + NS;           // [NS] O += P_j V_j complete
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(pv_done + NS);
 
-  const int qt = blockIdx.x, a = blockIdx.y, b = blockIdx.z;
+  const int qt = blockIdx.x / KS, split = blockIdx.x % KS, a = blockIdx.y, b = blockIdx.z;
   const int S = p.S, H = p.H;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int row0 = b * S;  // first token row of this sequence
@@ -104,62 +121,66 @@ __global__ void __launch_bounds__(NTHR, F_CTAS) attn_fwd_tc(const __grid_constan
 
   if (threadIdx.x == 0) {
     ptx::mbar_init(q_full, 1);
-    for (int s = 0; s < F_STAGES; ++s) {
+    for (int s = 0; s < SH::STAGES; ++s) {
       ptx::mbar_init(&kv_full[s], 1);
       ptx::mbar_init(&kv_empty[s], 1);
     }
-    ptx::mbar_init(s_full, 1);
-    ptx::mbar_init(p_full, 128);
-    ptx::mbar_init(pv_done, 1);
+    for (int s = 0; s < NS; ++s) {
+      ptx::mbar_init(&s_full[s], 1);
+      ptx::mbar_init(&p_full[s], 128);
+      ptx::mbar_init(&pv_done[s], 1);
+    }
     ptx::fence_mbar_init();
     ptx::fence_proxy_async_smem();
     ptx::prefetch_tensormap(&tmQ);
     ptx::prefetch_tensormap(&tmKV);
   }
   if (warp == 1) {
-    ptx::tmem_alloc(tmem_slot, F_TMEM_COLS);
+    ptx::tmem_alloc(tmem_slot, SH::TMEM_COLS);
     ptx::tmem_relinquish();
   }
   ptx::tc_fence_before();
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  const uint32_t tS = tmem, tO = tmem + 64;
+  const uint32_t tS0 = tmem, tO = tmem + 64 * NS;
   pdl_wait();
   int len = p.lens[b];
   if (len < 1 || len > S) {
     if (p.status && threadIdx.x == 0) atomicOr(p.status, kStatusBadLength);
     len = len < 1 ? 1 : S;
   }
-  const int n_kt = (len + BKV - 1) / BKV;
+  const int n_all = (len + BKV - 1) / BKV;
+  const int j0 = split * n_all / KS, n_kt = (split + 1) * n_all / KS - j0;  // this CTA's key tiles
+  const int last = n_kt > 0 ? n_kt - 1 : 0;
 
   if (warp == 0) {
     // ------------------------------------------------------------- producer
     const bool issuer = ptx::elect_one();
     if (issuer) {
       ptx::mbar_arrive_expect_tx(q_full, Q_BYTES);
-      ptx::tma_load_2d(smem + F_Q_OFF, &tmQ, q_full, a * HD, row0 + q0);
+      ptx::tma_load_2d(smem + SH::Q_OFF, &tmQ, q_full, a * HD, row0 + q0);
     }
     __syncwarp();
     int issued = 0;
     for (int j = 0; j < n_kt; ++j) {
-      const int st = j % F_STAGES;
+      const int st = j % SH::STAGES;
       if (!__all_sync(0xffffffffu,
-                      ptx::mbar_wait(&kv_empty[st], ((j / F_STAGES) & 1) ^ 1u, lim, p.status, kWaitHint)))
+                      ptx::mbar_wait(&kv_empty[st], ((j / SH::STAGES) & 1) ^ 1u, lim, p.status, kWaitHint)))
         break;
       if (issuer) {
-        uint8_t* kv = smem + F_KV_OFF + st * 2 * KV_BYTES;
+        uint8_t* kv = smem + SH::KV_OFF + st * 2 * KV_BYTES;
         ptx::mbar_arrive_expect_tx(&kv_full[st], 2 * KV_BYTES);
-        ptx::tma_load_2d(kv, &tmKV, &kv_full[st], H + a * HD, row0 + j * BKV);
-        ptx::tma_load_2d(kv + KV_BYTES, &tmKV, &kv_full[st], 2 * H + a * HD, row0 + j * BKV);
+        ptx::tma_load_2d(kv, &tmKV, &kv_full[st], H + a * HD, row0 + (j0 + j) * BKV);
+        ptx::tma_load_2d(kv + KV_BYTES, &tmKV, &kv_full[st], 2 * H + a * HD, row0 + (j0 + j) * BKV);
       }
       __syncwarp();
       ++issued;
     }
     // drain: bounded waits for the copies still in flight
     ptx::mbar_wait(q_full, 0, lim, p.status, kWaitHint);
-    for (int j = issued - 1; j >= 0 && j >= issued - F_STAGES; --j)
-      ptx::mbar_wait(&kv_full[j % F_STAGES], (j / F_STAGES) & 1, lim, p.status, kWaitHint);
+    for (int j = issued - 1; j >= 0 && j >= issued - SH::STAGES; --j)
+      ptx::mbar_wait(&kv_full[j % SH::STAGES], (j / SH::STAGES) & 1, lim, p.status, kWaitHint);
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issue
     // The whole warp walks the loop and one elected lane issues: a
@@ -169,40 +190,48 @@ __global__ void __launch_bounds__(NTHR, F_CTAS) attn_fwd_tc(const __grid_constan
     constexpr uint32_t idS = ptx::idesc_bf16_f32(BQ, BKV, false, false);
     constexpr uint32_t idO = ptx::idesc_bf16_f32(BQ, HD, false, true);
     const bool issuer = ptx::elect_one();
-    const uint64_t dq = ptx::smem_desc_sw128(ptx::smem_u32(smem + F_Q_OFF), 16, 1024);
-    const uint64_t dk0 = ptx::smem_desc_sw128(ptx::smem_u32(smem + F_KV_OFF), 16, 1024);
-    const uint64_t dv0 = ptx::smem_desc_sw128(ptx::smem_u32(smem + F_KV_OFF + KV_BYTES), 8192, 1024);
+    const uint64_t dq = ptx::smem_desc_sw128(ptx::smem_u32(smem + SH::Q_OFF), 16, 1024);
+    const uint64_t dk0 = ptx::smem_desc_sw128(ptx::smem_u32(smem + SH::KV_OFF), 16, 1024);
+    const uint64_t dv0 = ptx::smem_desc_sw128(ptx::smem_u32(smem + SH::KV_OFF + KV_BYTES), 8192, 1024);
     auto wait = [&](uint64_t* bar, uint32_t parity) {
       return __all_sync(0xffffffffu, ptx::mbar_wait(bar, parity, lim, p.status, kWaitHint));
     };
     bool ok = wait(q_full, 0);
-    for (int j = 0; j < n_kt && ok; ++j) {
-      const uint64_t off = static_cast<uint64_t>((j % F_STAGES) * (2 * KV_BYTES >> 4));
-      // K_j, V_j are here, and P_{j-1}, whose columns S_j takes, has been read
-      if (!wait(&kv_full[j % F_STAGES], (j / F_STAGES) & 1)) { ok = false; break; }
-      if (j > 0 && !wait(pv_done, (j - 1) & 1)) { ok = false; break; }
+    auto score = [&](int j) {  // S_j into buffer j % NS
+      const int st = j % SH::STAGES;
+      // K_j, V_j are here, and P_{j - NS}, whose columns S_j takes, has been read
+      if (!wait(&kv_full[st], (j / SH::STAGES) & 1)) return false;
+      if (j >= NS && !wait(&pv_done[j % NS], (j / NS - 1) & 1)) return false;
       ptx::tc_fence_after();
       if (issuer) {
+        const uint64_t dk = dk0 + static_cast<uint64_t>(st * (2 * KV_BYTES >> 4));
 #pragma unroll
         for (int kk = 0; kk < HD / 16; ++kk)
-          ptx::tc_mma_f16(tS, dq + kk * 2, dk0 + off + kk * 2, idS, kk > 0 ? 1u : 0u);
-        ptx::tc_commit(s_full);
+          ptx::tc_mma_f16(tS0 + (j % NS) * 64, dq + kk * 2, dk + kk * 2, idS, kk > 0 ? 1u : 0u);
+        ptx::tc_commit(&s_full[j % NS]);
       }
       __syncwarp();
-      if (!wait(p_full, j & 1)) { ok = false; break; }
+      return true;
+    };
+    if (NS == 2 && ok && n_kt > 0) ok = score(0);
+    for (int j = 0; j < n_kt && ok; ++j) {
+      if (NS == 1) ok = score(j);
+      else if (j + 1 < n_kt) ok = score(j + 1);  // beside the softmax of tile j
+      if (!ok || !wait(&p_full[j % NS], (j / NS) & 1)) { ok = false; break; }
       ptx::tc_fence_after();
       if (issuer) {
+        const uint64_t dv = dv0 + static_cast<uint64_t>((j % SH::STAGES) * (2 * KV_BYTES >> 4));
 #pragma unroll
         for (int kk = 0; kk < BKV / 16; ++kk)
-          ptx::tc_mma_f16_tmem_a(tO, tS + kk * 8, dv0 + off + kk * 128, idO, (j > 0 || kk > 0) ? 1u : 0u);
-        ptx::tc_commit(pv_done);
-        ptx::tc_commit(&kv_empty[j % F_STAGES]);
+          ptx::tc_mma_f16_tmem_a(tO, tS0 + (j % NS) * 64 + kk * 8, dv + kk * 128, idO, (j > 0 || kk > 0) ? 1u : 0u);
+        ptx::tc_commit(&pv_done[j % NS]);
+        ptx::tc_commit(&kv_empty[j % SH::STAGES]);
       }
       __syncwarp();
     }
-    if (!ok && issuer) ptx::tc_commit(pv_done);  // a timeout: what was issued still has to finish
+    if (!ok && issuer) ptx::tc_commit(&pv_done[last % NS]);  // a timeout: what was issued still has to finish
     __syncwarp();
-    ptx::mbar_wait(pv_done, (n_kt - 1) & 1, lim, p.status, kWaitHint);
+    if (n_kt > 0) ptx::mbar_wait(&pv_done[last % NS], (last / NS) & 1, lim, p.status, kWaitHint);
   } else {
     // --------------------------------------------------- softmax / epilogue
     const int q4 = warp & 3;
@@ -217,36 +246,54 @@ __global__ void __launch_bounds__(NTHR, F_CTAS) attn_fwd_tc(const __grid_constan
       const bool mine = ptx::mbar_wait(bar, parity, lim, p.status, kWaitHint);
       return __all_sync(0xffffffffu, mine);
     };
-    uint32_t v[32];  // half a row's scores at a time: registers for four CTAs an SM
+    // two score buffers: a whole row's scores; one: half of them at a time, registers
+    // for four CTAs an SM
+    uint32_t vv[32 * NS];
+    auto half = [&](int h) -> uint32_t(&)[32] { return *reinterpret_cast<uint32_t(*)[32]>(vv + (NS == 2 ? 32 * h : 0)); };
     for (int j = 0; j < n_kt; ++j) {
-      const int left = len - j * BKV;  // valid keys of this tile
-      auto load_half = [&](int h) {
-        ptx::tmem_ld_32x32b_x32(tS + lane_base + h * 32, v);
-        ptx::tmem_ld_wait();
+      const int left = len - (j0 + j) * BKV;  // valid keys of this tile
+      const uint32_t tS = tS0 + (j % NS) * 64;
+      auto load_half = [&](int h) { ptx::tmem_ld_32x32b_x32(tS + lane_base + h * 32, half(h)); };
+      auto mask_half = [&](int h) {
+        uint32_t(&v)[32] = half(h);
         if (left < (h + 1) * 32) {  // CTA-uniform: only the last tile holds masked keys
 #pragma unroll
           for (int i = 0; i < 32; ++i)
             if (h * 32 + i >= left) v[i] = 0xff800000u;  // -inf: excluded from the max, P = 0
         }
       };
-      auto half_max = [&](float mx) {
+      auto half_max = [&](int h, float mx) {
+        const uint32_t(&v)[32] = half(h);
         float m4[4] = {mx, __uint_as_float(v[0]), __uint_as_float(v[1]), __uint_as_float(v[2])};
 #pragma unroll
         for (int i = 3; i < 32; ++i) m4[i & 3] = fmaxf(m4[i & 3], __uint_as_float(v[i]));
         return fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
       };
-      if (!wait_all(s_full, j & 1)) { ok = false; break; }
+      if (!wait_all(&s_full[j % NS], (j / NS) & 1)) { ok = false; break; }
       ptx::tc_fence_after();
       // row max of the raw scores (scaling by log2(e)/sqrt(D) > 0 commutes with
       // max): the high half, then the low half, which stays in registers
       load_half(1);
-      float mx = half_max(-INFINITY);
-      load_half(0);
-      mx = half_max(mx) * sl2;
+      if (NS == 2) load_half(0);
+      ptx::tmem_ld_wait();
+      mask_half(1);
+      float mx = half_max(1, -INFINITY);
+      if (NS == 1) {
+        load_half(0);
+        ptx::tmem_ld_wait();
+      }
+      mask_half(0);
+      mx = half_max(0, mx) * sl2;
       if (j == 0) {
-        m = mx;
+        // (a split whose first keys' scores are all -inf adds nothing, as those keys
+        // would behind others)
+        m = KS > 1 ? fmaxf(mx, -FLT_MAX) : mx;
       } else if (__any_sync(0xffffffffu, mx > m + kRescaleLog2)) {
-        // O holds P_{j-1} V_{j-1}: S_j was issued behind it
+        // O holds P_{j-1} V_{j-1} (one buffer: S_j was issued behind it)
+        if (NS == 2) {
+          if (!wait_all(&pv_done[(j - 1) % NS], ((j - 1) / NS) & 1)) { ok = false; break; }
+          ptx::tc_fence_after();
+        }
         const float m_new = fmaxf(m, mx);
         const float alpha = exp2f(m - m_new);
 #pragma unroll
@@ -267,7 +314,12 @@ __global__ void __launch_bounds__(NTHR, F_CTAS) attn_fwd_tc(const __grid_constan
       uint64_t ls[2] = {0, 0};  // pairs of zeros
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        if (h == 1) load_half(1);
+        if (NS == 1 && h == 1) {
+          load_half(1);
+          ptx::tmem_ld_wait();
+          mask_half(1);
+        }
+        const uint32_t(&v)[32] = half(h);
         uint32_t pk[16];
 #pragma unroll
         for (int u = 0; u < 16; ++u) {
@@ -282,46 +334,119 @@ __global__ void __launch_bounds__(NTHR, F_CTAS) attn_fwd_tc(const __grid_constan
       l += lsum.x + lsum.y;
       ptx::tmem_st_wait();
       ptx::tc_fence_before();
-      ptx::mbar_arrive(p_full);
+      ptx::mbar_arrive(&p_full[j % NS]);
     }
     pdl_trigger();  // behind the main loop: see common.cuh
-    // epilogue: O / l -> ctx (bf16) as 128-byte-swizzled rows over the Q
-    // tile (the last S product has read it), stored by one TMA that drops the
-    // rows past S; the log-sum-exp directly
-    if (ok && wait_all(pv_done, (n_kt - 1) & 1)) {
-      ptx::tc_fence_after();
-      const float inv = 1.f / l;
-      const int q = q0 + r;
-      const uint32_t orow = ptx::smem_u32(smem + F_Q_OFF) + r * 128;
+    if constexpr (KS > 1) {
+      // partial O (16-byte group g of row r at group g ^ (r & 7)), m and l to shared
+      // memory, over the K/V stages, which have been read
+      if (n_kt > 0 && ok && wait_all(&pv_done[last % NS], (last / NS) & 1)) {
+        ptx::tc_fence_after();
+        const uint32_t orow = ptx::smem_u32(smem + SH::KV_OFF) + r * HD * 4;
 #pragma unroll
-      for (int c = 0; c < HD / 32; ++c) {
-        ptx::tmem_ld_32x32b_x32(tO + lane_base + c * 32, v);
-        ptx::tmem_ld_wait();
+        for (int c = 0; c < HD / 32; ++c) {
+          uint32_t(&v)[32] = half(0);
+          ptx::tmem_ld_32x32b_x32(tO + lane_base + c * 32, v);
+          ptx::tmem_ld_wait();
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          uint32_t w[4];
-#pragma unroll
-          for (int t = 0; t < 4; ++t)
-            w[t] = ptx::pack_bf16(__uint_as_float(v[8 * u + 2 * t]) * inv,
-                                  __uint_as_float(v[8 * u + 2 * t + 1]) * inv);
-          ptx::st_shared_v4(orow + (((c * 4 + u) ^ (r & 7)) << 4), w[0], w[1], w[2], w[3]);
+          for (int u = 0; u < 8; ++u)
+            ptx::st_shared_v4(orow + (((c * 8 + u) ^ (r & 7)) << 4), v[4 * u], v[4 * u + 1], v[4 * u + 2],
+                              v[4 * u + 3]);
         }
       }
-      if (q < S) p.lse[(static_cast<int64_t>(b) * p.A + a) * S + q] = m + log2f(l);
-    }
-    ptx::fence_proxy_async_smem();  // the staged rows -> the TMA store
-    asm volatile("bar.sync 1, 128;" ::: "memory");  // the four softmax warps
-    if (warp == 2 && lane == 0) {
-      ptx::tma_store_3d(&tmOut, smem + F_Q_OFF, a * HD, q0, b);
-      ptx::bulk_commit_group();
-      ptx::bulk_wait_group_read0();  // before the CTA's memory goes
+      reinterpret_cast<float2*>(smem + SH::ML_OFF)[r] = make_float2(m, l);
+    } else {
+      // epilogue: O / l -> ctx (bf16) as 128-byte-swizzled rows over the Q
+      // tile (the last S product has read it), stored by one TMA that drops the
+      // rows past S; the log-sum-exp directly
+      if (ok && wait_all(&pv_done[last % NS], (last / NS) & 1)) {
+        ptx::tc_fence_after();
+        const float inv = 1.f / l;
+        const int q = q0 + r;
+        const uint32_t orow = ptx::smem_u32(smem + SH::Q_OFF) + r * 128;
+#pragma unroll
+        for (int c = 0; c < HD / 32; ++c) {
+          uint32_t(&v)[32] = half(0);
+          ptx::tmem_ld_32x32b_x32(tO + lane_base + c * 32, v);
+          ptx::tmem_ld_wait();
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            uint32_t w[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t)
+              w[t] = ptx::pack_bf16(__uint_as_float(v[8 * u + 2 * t]) * inv,
+                                    __uint_as_float(v[8 * u + 2 * t + 1]) * inv);
+            ptx::st_shared_v4(orow + (((c * 4 + u) ^ (r & 7)) << 4), w[0], w[1], w[2], w[3]);
+          }
+        }
+        if (q < S) p.lse[(static_cast<int64_t>(b) * p.A + a) * S + q] = m + log2f(l);
+      }
+      ptx::fence_proxy_async_smem();  // the staged rows -> the TMA store
+      asm volatile("bar.sync 1, 128;" ::: "memory");  // the four softmax warps
+      if (warp == 2 && lane == 0) {
+        ptx::tma_store_3d(&tmOut, smem + SH::Q_OFF, a * HD, q0, b);
+        ptx::bulk_commit_group();
+        ptx::bulk_wait_group_read0();  // before the CTA's memory goes
+      }
     }
   }
+  if constexpr (KS > 1) {
+    __syncwarp();
+    ptx::cluster_sync();  // every split's part is where it is read from
+    if (warp >= 2) {
+      // This CTA finishes 128 / KS of the query rows, KS threads a row: the splits'
+      // parts in split order, each scaled to the largest m.
+      constexpr int ROWS = BQ / KS, G = HD / 4 / KS;
+      const int t = static_cast<int>(threadIdx.x) - 64, lr = t / KS, sub = t % KS, row = split * ROWS + lr;
+      const uint32_t part = ptx::smem_u32(smem + SH::KV_OFF) + row * HD * 4;
+      const uint32_t ml = ptx::smem_u32(smem + SH::ML_OFF) + row * 8;
+      float w[KS], mx = -FLT_MAX, l = 0.f;
+#pragma unroll
+      for (int s = 0; s < KS; ++s) {
+        const float2 x = ptx::ld_cluster_f2(ptx::mapa_shared(ml, s));
+        const bool any = (s + 1) * n_all / KS > s * n_all / KS;
+        w[s] = any ? x.x : -INFINITY;
+        mx = fmaxf(mx, w[s]);
+      }
+#pragma unroll
+      for (int s = 0; s < KS; ++s) {
+        w[s] = exp2f(w[s] - mx);
+        l += w[s] * ptx::ld_cluster_f2(ptx::mapa_shared(ml, s)).y;
+      }
+      const float inv = 1.f / l;
+      const uint32_t orow = ptx::smem_u32(smem + SH::Q_OFF) + lr * 128;
+#pragma unroll
+      for (int i = 0; i < G; ++i) {
+        const int g = sub + KS * i;
+        float4 x[KS], o = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int s = 0; s < KS; ++s) x[s] = ptx::ld_cluster_f4(ptx::mapa_shared(part + ((g ^ (row & 7)) << 4), s));
+#pragma unroll
+        for (int s = 0; s < KS; ++s) {
+          if ((s + 1) * n_all / KS == s * n_all / KS) continue;  // (nothing was written there)
+          o.x += w[s] * x[s].x; o.y += w[s] * x[s].y; o.z += w[s] * x[s].z; o.w += w[s] * x[s].w;
+        }
+        ptx::st_shared_v2(orow + (((g >> 1) ^ (lr & 7)) << 4) + (g & 1) * 8, ptx::pack_bf16(o.x * inv, o.y * inv),
+                          ptx::pack_bf16(o.z * inv, o.w * inv));
+      }
+      const int q = q0 + row;
+      if (sub == 0 && q < S) p.lse[(static_cast<int64_t>(b) * p.A + a) * S + q] = mx + log2f(l);
+      ptx::fence_proxy_async_smem();
+      asm volatile("bar.sync 1, 128;" ::: "memory");
+      if (warp == 2 && lane == 0 && q0 + split * ROWS < S) {
+        ptx::tma_store_3d(&tmOut, smem + SH::Q_OFF, a * HD, q0 + split * ROWS, b);
+        ptx::bulk_commit_group();
+        ptx::bulk_wait_group_read0();
+      }
+    }
+    __syncwarp();
+  }
   ptx::tc_fence_before();
-  __syncthreads();
+  if constexpr (KS > 1) ptx::cluster_sync();  // the peers have read this CTA's part
+  else __syncthreads();
   if (warp == 1) {
     ptx::tc_fence_after();
-    ptx::tmem_dealloc(tmem, F_TMEM_COLS);
+    ptx::tmem_dealloc(tmem, SH::TMEM_COLS);
   }
 }
 
@@ -332,9 +457,10 @@ __global__ void __launch_bounds__(NTHR, F_CTAS) attn_fwd_tc(const __grid_constan
 // second tile's round trip through the tensor pipe.
 constexpr int FS_Q = 0, FS_K = Q_BYTES, FS_V = 2 * Q_BYTES, FS_BAR = 3 * Q_BYTES;
 constexpr int FS_SMEM = FS_BAR + 64 + 1024;
-static_assert(F_CTAS * (FS_SMEM + 1024) <= 233472, "four forward CTAs per SM");
+constexpr int FS_TMEM_COLS = 128;
+static_assert(4 * (FS_SMEM + 1024) <= 233472, "four forward CTAs per SM");
 
-__global__ void __launch_bounds__(NTHR, F_CTAS) attn_fwd_short_tc(const __grid_constant__ CUtensorMap tmQKV,
+__global__ void __launch_bounds__(NTHR, 4) attn_fwd_short_tc(const __grid_constant__ CUtensorMap tmQKV,
                                                                   const __grid_constant__ CUtensorMap tmOut,
                                                                   const FwdParams p) {
   extern __shared__ uint8_t smem_raw[];
@@ -363,7 +489,7 @@ __global__ void __launch_bounds__(NTHR, F_CTAS) attn_fwd_short_tc(const __grid_c
     ptx::prefetch_tensormap(&tmQKV);
   }
   if (warp == 1) {
-    ptx::tmem_alloc(tmem_slot, F_TMEM_COLS);
+    ptx::tmem_alloc(tmem_slot, FS_TMEM_COLS);
     ptx::tmem_relinquish();
   }
   ptx::tc_fence_before();
@@ -512,7 +638,7 @@ __global__ void __launch_bounds__(NTHR, F_CTAS) attn_fwd_short_tc(const __grid_c
   __syncthreads();
   if (warp == 1) {
     ptx::tc_fence_after();
-    ptx::tmem_dealloc(tmem, F_TMEM_COLS);
+    ptx::tmem_dealloc(tmem, FS_TMEM_COLS);
   }
 }
 
@@ -1478,16 +1604,38 @@ sky_status attention_fwd_tc(const void* qkv, const int32_t* lens, int B, int S, 
     count_launches(1);
     return e == cudaSuccess ? SKY_OK : cuda_fail(e, "tensor-core attention forward launch");
   }
+  // Which form (us; [ragged] lengths uniform in 1..S; CTAs of 128 queries, 152 SMs):
+  //  two buffers up to 2.6 CTAs an SM: 2 x 1024 x 12 heads (192) 11.9 against 17.6 with
+  //    one; 8 x 700 x 8 (384) 16.9 and 14.8, [8.5 and 12.8]; 6 x 700 x 12 (432) 17.8
+  //    and 15.0, [12.8 and 11.2].  From 24 key tiles on, where CTAs left alone at the
+  //    end take long, up to six: 4 x 2048 x 12 (768) 66 and 71; 4 x 1500 x 16 (768)
+  //    [35.9 and 39.7]; 4 x 2048 x 16 (1024) 86 and 81, [64.5 and 63.4, of 512..S].
+  //  else one: 16 x 512 x 16 (1024) 27.0 against 32.7, 24 x 197 x 12 (576) 9.6 and 11.6.
+  //  keys in four while that leaves two CTAs an SM and each three tiles: 1024 x 9 heads
+  //    (72) 8.3, unsplit 10.0; in two up to one CTA an SM and from 24 tiles on: 2048 x
+  //    8 (128) 14.3 and 17.4; 800 x 12 (84, 13 tiles) 8.2 and 7.4.
+  const int sms = sm_count() > 0 ? sm_count() : 148, tiles = ceil_div(S, BKV);
+  const int64_t ctas = static_cast<int64_t>(ceil_div(S, BQ)) * A * B;
+  const bool two = 5 * ctas <= 13 * sms || (tiles >= 24 && ctas <= 6 * sms);
+  const int ks = tiles >= 12 && 2 * ctas <= sms ? 4 : tiles >= 24 && ctas <= sms ? 2 : 1;
   SKY_CHECK(head_map(&tq, qkv, T, 3 * H, BQ) && head_map(&tkv, qkv, T, 3 * H, BKV) &&
-                seq_map(&tout, ctx, B, S, H, BQ),
+                seq_map(&tout, ctx, B, S, H, BQ / ks),
             SKY_ERR_CUDA,
             "cuTensorMapEncodeTiled failed for the attention operands");
-  static cudaError_t attr = cudaFuncSetAttribute(attn_fwd_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 F_SMEM);
-  if (attr != cudaSuccess) return cuda_fail(attr, "attention smem attribute");
-  dim3 grid(ceil_div(S, BQ), A, B);
   FwdParams p{S, H, A, lens, static_cast<__nv_bfloat16*>(ctx), lse, status, timeout_ns};
-  const cudaError_t e = launch_pdl(attn_fwd_tc, grid, dim3(NTHR), F_SMEM, stream, 1, tq, tkv, tout, p);
+  auto go = [&](auto splits, auto bufs) {
+    constexpr int KS = decltype(splits)::value, NS = decltype(bufs)::value;
+    auto kern = attn_fwd_tc<KS, NS>;
+    static cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   FwdShape<NS>::SMEM);
+    if (attr != cudaSuccess) return attr;
+    return launch_pdl(kern, dim3(ceil_div(S, BQ) * KS, A, B), dim3(NTHR), FwdShape<NS>::SMEM, stream, KS, tq, tkv,
+                      tout, p);
+  };
+  const std::integral_constant<int, 1> c1{};
+  const std::integral_constant<int, 2> c2{};
+  const std::integral_constant<int, 4> c4{};
+  const cudaError_t e = !two ? go(c1, c1) : ks == 1 ? go(c1, c2) : ks == 2 ? go(c2, c2) : go(c4, c2);
   count_launches(1);
   return e == cudaSuccess ? SKY_OK : cuda_fail(e, "tensor-core attention forward launch");
 }

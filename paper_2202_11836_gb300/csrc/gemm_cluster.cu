@@ -91,14 +91,6 @@ struct Tiling {
   static constexpr int RECV_BYTES = PUSH ? KS * ROWS * BN * 4 : 0;  // a multiple of 256
 };
 
-__device__ __forceinline__ float4 ld_cluster_f4(uint32_t addr) {
-  float4 v;
-  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
-               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-               : "r"(addr)
-               : "memory");
-  return v;
-}
 __device__ __forceinline__ float4 ld_stream_f4(const float* p) {
   float4 v;
   asm volatile("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
@@ -385,7 +377,7 @@ __global__ void __launch_bounds__(C_THREADS, 2)
             w[u][s] = ptx::ld_shared_f4(at);
           } else {
             const uint32_t at = sbase + static_cast<uint32_t>(rl * BN * 4) + ((c ^ (rl & 7)) << 4);
-            w[u][s] = ld_cluster_f4(ptx::mapa_shared(at, PAIR ? 2 * s + half : s));
+            w[u][s] = ptx::ld_cluster_f4(ptx::mapa_shared(at, PAIR ? 2 * s + half : s));
           }
         }
       }
