@@ -5,9 +5,10 @@
 // get probability exactly 0.
 //
 // bf16 (D = 64): the tensor-core kernels of attention_tc.cu, plus the
-// vectorised delta = rowsum(dO * O) pre-pass here.
-// fp32: one warp per query (or key) row with exact fp32 arithmetic, for the
-// small fp32 configuration.
+// vectorised delta = rowsum(dO * O) pre-pass here (sequences over 128; shorter
+// ones form it in their one backward launch).
+// fp32: blocks of query (or key) rows against tiles of the other side, exact
+// fp32 arithmetic.
 #include "common.cuh"
 #include "ptx.cuh"
 
@@ -130,27 +131,47 @@ __global__ void attn_delta(const T* __restrict__ ctx, const T* __restrict__ dctx
 constexpr int FR = 16, FC = 64, F_THR = 128;  // rows of a CTA, columns of a tile
 constexpr int FP_LD = FC + 4;                 // row stride of the probability tiles
 
-// Rows [r0, r0 + n) of X (row stride ld, D values each) into s[n][LD]; rows from
-// `rows` on and columns from D on are zeros.  vec: D, ld and X allow 16-byte loads.
-__device__ __forceinline__ void stage_rows(float* s, int LD, const float* __restrict__ X, int64_t ld, int r0,
-                                           int n, int rows, int D, bool vec) {
-  const int g4 = (D + 3) / 4;
-  for (int i = threadIdx.x; i < n * g4; i += F_THR) {
-    const int r = i / g4, c = (i - r * g4) * 4;
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (r0 + r < rows) {
-      const float* p = X + static_cast<int64_t>(r0 + r) * ld + c;
+// Rows are staged F_THR / G a pass, G threads a row (D <= 4 G), through registers, so
+// that a tile's loads are all in flight before the first is stored.  Loading and
+// storing in turn waited for each: 4 x 32 tokens, 2 heads of 64, forward 6.4 us,
+// now 3.8, backward 10.7 and 7.3; 4 x 101, 12 heads 17.0 and 12.2, 39.9 and 29.4; 4 x
+// 256, 24 heads of 32 52.6 and 48.7 (58.1 with 16 threads a row).
+template <int G>
+struct Stage {  // a tile's FC rows: BATCHES of PASSES passes, R rows each
+  static constexpr int PASSES = FC * G / F_THR < 8 ? FC * G / F_THR : 8;
+  static constexpr int R = PASSES * F_THR / G, BATCHES = FC / R;
+  static constexpr int OWN = FR * G / F_THR;  // passes of the CTA's FR rows
+  static constexpr int CC = G > 16 ? G / 16 : 1;  // 64-value column groups of an output row
+};
+// Rows from `rows` on are zeros.  vec: D, ld and X allow 16-byte loads.
+template <int G, int N>
+__device__ __forceinline__ void load_rows(const float* __restrict__ X, int64_t ld, int r0, int rows, int D, bool vec,
+                                          float4 (&v)[N]) {
+  const int c = (threadIdx.x % G) * 4;
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const int r = r0 + F_THR / G * i + threadIdx.x / G;
+    v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (r < rows && c < D) {
+      const float* p = X + static_cast<int64_t>(r) * ld + c;
       if (vec) {
-        v = *reinterpret_cast<const float4*>(p);
+        v[i] = *reinterpret_cast<const float4*>(p);
       } else {
-        v.x = p[0];
-        if (c + 1 < D) v.y = p[1];
-        if (c + 2 < D) v.z = p[2];
-        if (c + 3 < D) v.w = p[3];
+        v[i].x = p[0];
+        if (c + 1 < D) v[i].y = p[1];
+        if (c + 2 < D) v[i].z = p[2];
+        if (c + 3 < D) v[i].w = p[3];
       }
     }
-    *reinterpret_cast<float4*>(s + r * LD + c) = v;
   }
+}
+template <int G, int N>
+__device__ __forceinline__ void put_rows(float* s, int LD, int D, const float4 (&v)[N]) {
+  const int c = (threadIdx.x % G) * 4;
+  if (c >= D) return;
+#pragma unroll
+  for (int i = 0; i < N; ++i)
+    *reinterpret_cast<float4*>(s + (F_THR / G * i + threadIdx.x / G) * LD + c) = v[i];
 }
 // acc[i][c] = row (2 ty + i) . column row (tx + 16 c), over D (a multiple of 4 in shared memory)
 __device__ __forceinline__ void scores(const float* rows, const float* cols, int LD, int D, float (&acc)[2][4]) {
@@ -238,11 +259,13 @@ __device__ __forceinline__ float half_warp_sum(float v) {
   return v;
 }
 
-template <int CC>
+template <int G>
 __global__ void __launch_bounds__(F_THR) attn_fwd_f32(const float* __restrict__ qkv, const int32_t* __restrict__ lens,
                                                       int S, int H, int A, int D, int LD, bool vec,
                                                       float* __restrict__ ctx, float* __restrict__ lse,
                                                       int32_t* status) {
+  using ST = Stage<G>;
+  constexpr int CC = ST::CC;
   pdl_wait();
   extern __shared__ __align__(16) float sm[];
   float *sq = sm, *sk = sq + FR * LD, *sv = sk + FC * LD, *sp = sv + FC * LD;
@@ -257,13 +280,22 @@ __global__ void __launch_bounds__(F_THR) attn_fwd_f32(const float* __restrict__ 
   const int64_t rs = 3 * static_cast<int64_t>(H);
   const float* q = qkv + static_cast<int64_t>(b) * S * rs + a * D;
   const float sc = 1.f / sqrtf((float)D);
-  stage_rows(sq, LD, q, rs, q0, FR, S, D, vec);
+  float4 own[ST::OWN];
+  load_rows<G>(q, rs, q0, S, D, vec, own);
   float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};
   float4 o[2][CC] = {};
   for (int k0 = 0; k0 < len; k0 += FC) {
     __syncthreads();
-    stage_rows(sk, LD, q + H, rs, k0, FC, len, D, vec);
-    stage_rows(sv, LD, q + 2 * H, rs, k0, FC, len, D, vec);
+#pragma unroll
+    for (int h = 0; h < ST::BATCHES; ++h) {
+      constexpr int R = ST::R;
+      float4 kx[ST::PASSES], vx[ST::PASSES];
+      load_rows<G>(q + H, rs, k0 + R * h, len, D, vec, kx);
+      load_rows<G>(q + 2 * H, rs, k0 + R * h, len, D, vec, vx);
+      if (h == 0 && k0 == 0) put_rows<G>(sq, LD, D, own);
+      put_rows<G>(sk + R * h * LD, LD, D, kx);
+      put_rows<G>(sv + R * h * LD, LD, D, vx);
+    }
     __syncthreads();
     float s[2][4];
     scores(sq, sk, LD, D, s);
@@ -308,12 +340,16 @@ __global__ void __launch_bounds__(F_THR) attn_fwd_f32(const float* __restrict__ 
 // dK, dV (odd): own rows are keys (K, V), columns queries (Q, dO).  Either way
 //   P = exp2(s log2(e)/sqrt(D) - lse_q),  dS = P (dp - delta_q),
 // s and dp the products of the first and second operands; dQ or dK = dS . first
-// operand of the columns / sqrt(D), dV = P . dO.
-template <int CC>
-__global__ void __launch_bounds__(F_THR) attn_bwd_f32(const float* __restrict__ qkv, const float* __restrict__ dctx,
+// operand of the columns / sqrt(D), dV = P . dO.  Four CTAs an SM (128 registers) are
+// faster up to a head dim of 64 (29.8 us against 34.7 at 4 x 101, 12 heads), above it
+// the registers are (50.6 against 57.0 at 2 x 200, 6 heads of 128).
+template <int G>
+__global__ void __launch_bounds__(F_THR, G > 16 ? 1 : 4) attn_bwd_f32(const float* __restrict__ qkv, const float* __restrict__ dctx,
                                                       const float* __restrict__ lse, const float* __restrict__ delta,
                                                       const int32_t* __restrict__ lens, int S, int H, int A, int D,
                                                       int LD, bool vec, float* __restrict__ dqkv) {
+  using ST = Stage<G>;
+  constexpr int CC = ST::CC;
   pdl_wait();
   extern __shared__ __align__(16) float sm[];
   float *r0s = sm, *r1s = r0s + FR * LD, *c0s = r1s + FR * LD, *c1s = c0s + FC * LD;
@@ -334,9 +370,9 @@ __global__ void __launch_bounds__(F_THR) attn_bwd_f32(const float* __restrict__ 
   float4 o0[2][CC] = {}, o1[2][CC] = {};
   const int cols = keys ? S : len;
   if (!keys || r0 < len) {
-    stage_rows(r0s, LD, keys ? q + H : q, rs, r0, FR, S, D, vec);
-    if (keys) stage_rows(r1s, LD, q + 2 * H, rs, r0, FR, S, D, vec);
-    else stage_rows(r1s, LD, dO, H, r0, FR, S, D, vec);
+    float4 own0[ST::OWN], own1[ST::OWN];
+    load_rows<G>(keys ? q + H : q, rs, r0, S, D, vec, own0);
+    load_rows<G>(keys ? q + 2 * H : dO, keys ? rs : static_cast<int64_t>(H), r0, S, D, vec, own1);
     float lr[2], dr[2];
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
@@ -346,17 +382,30 @@ __global__ void __launch_bounds__(F_THR) attn_bwd_f32(const float* __restrict__ 
     }
     for (int c0 = 0; c0 < cols; c0 += FC) {
       __syncthreads();
-      if (keys) {
-        stage_rows(c0s, LD, q, rs, c0, FC, S, D, vec);
-        stage_rows(c1s, LD, dO, H, c0, FC, S, D, vec);
-        if (threadIdx.x < FC) {
-          const int c = min(c0 + static_cast<int>(threadIdx.x), S - 1);
-          sl[threadIdx.x] = lse_b[c];
-          sd[threadIdx.x] = del_b[c];
+      // columns: queries (Q, dO; all S) or keys (K, V; the valid ones)
+      const float *x0 = keys ? q : q + H, *x1 = keys ? dO : q + 2 * H;
+      float lc = 0.f, dc = 0.f;
+      if (keys && threadIdx.x < FC) {
+        const int c = min(c0 + static_cast<int>(threadIdx.x), S - 1);
+        lc = lse_b[c];
+        dc = del_b[c];
+      }
+#pragma unroll
+      for (int h = 0; h < ST::BATCHES; ++h) {
+        constexpr int R = ST::R;
+        float4 v0[ST::PASSES], v1[ST::PASSES];
+        load_rows<G>(x0, rs, c0 + R * h, cols, D, vec, v0);
+        load_rows<G>(x1, keys ? static_cast<int64_t>(H) : rs, c0 + R * h, cols, D, vec, v1);
+        if (h == 0 && c0 == 0) {
+          put_rows<G>(r0s, LD, D, own0);
+          put_rows<G>(r1s, LD, D, own1);
         }
-      } else {
-        stage_rows(c0s, LD, q + H, rs, c0, FC, len, D, vec);
-        stage_rows(c1s, LD, q + 2 * H, rs, c0, FC, len, D, vec);
+        put_rows<G>(c0s + R * h * LD, LD, D, v0);
+        put_rows<G>(c1s + R * h * LD, LD, D, v1);
+      }
+      if (keys && threadIdx.x < FC) {
+        sl[threadIdx.x] = lc;
+        sd[threadIdx.x] = dc;
       }
       __syncthreads();
       float s[2][4], dp[2][4];
@@ -429,16 +478,17 @@ sky_status attention_fwd(const void* qkv, const int32_t* lens, int B, int S, int
     SKY_CHECK(D <= 128, SKY_ERR_UNSUPPORTED, "fp32 attention needs head dim <= 128");
     SKY_CHECK(S <= 3072, SKY_ERR_UNSUPPORTED, "fp32 attention: sequence too long");
     const attn::F32Shape f(S, H, A, D, qkv, ctx, nullptr);
-    static const cudaError_t attr[2] = {  // once, for the largest head dim of each
-        cudaFuncSetAttribute(attn::attn_fwd_f32<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, attn::fwd_smem(64)),
-        cudaFuncSetAttribute(attn::attn_fwd_f32<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, attn::fwd_smem(128))};
+    static const cudaError_t attr[3] = {  // once, for the largest head dim of each
+        cudaFuncSetAttribute(attn::attn_fwd_f32<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, attn::fwd_smem(32)),
+        cudaFuncSetAttribute(attn::attn_fwd_f32<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, attn::fwd_smem(64)),
+        cudaFuncSetAttribute(attn::attn_fwd_f32<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, attn::fwd_smem(128))};
     const auto go = [&](auto kern) {
       return launch_pdl(kern, dim3(f.units, B), dim3(attn::F_THR), attn::fwd_smem(D), stream, 1,
                         static_cast<const float*>(qkv), lens, S, H, A, D, f.LD, f.vec, static_cast<float*>(ctx), lse,
                         status);
     };
-    cudaError_t le = attr[D > 64];
-    if (le == cudaSuccess) le = D <= 64 ? go(attn::attn_fwd_f32<1>) : go(attn::attn_fwd_f32<2>);
+    cudaError_t le = attr[(D > 32) + (D > 64)];
+    if (le == cudaSuccess) le = D <= 32 ? go(attn::attn_fwd_f32<8>) : D <= 64 ? go(attn::attn_fwd_f32<16>) : go(attn::attn_fwd_f32<32>);
     if (le != cudaSuccess) return cuda_fail(le, "attention forward launch");
   }
   count_launches(1);
@@ -490,16 +540,17 @@ sky_status attention_bwd(const void* qkv, const void* ctx, const void* dctx, con
                                 static_cast<const float*>(ctx), static_cast<const float*>(dctx), S, H, A, D, rows,
                                 delta);
     const attn::F32Shape f(S, H, A, D, qkv, dctx, dqkv);
-    static const cudaError_t attr[2] = {
-        cudaFuncSetAttribute(attn::attn_bwd_f32<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, attn::bwd_smem(64)),
-        cudaFuncSetAttribute(attn::attn_bwd_f32<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, attn::bwd_smem(128))};
-    if (le == cudaSuccess) le = attr[D > 64];
+    static const cudaError_t attr[3] = {
+        cudaFuncSetAttribute(attn::attn_bwd_f32<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, attn::bwd_smem(32)),
+        cudaFuncSetAttribute(attn::attn_bwd_f32<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, attn::bwd_smem(64)),
+        cudaFuncSetAttribute(attn::attn_bwd_f32<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, attn::bwd_smem(128))};
+    if (le == cudaSuccess) le = attr[(D > 32) + (D > 64)];
     const auto go = [&](auto kern) {
       return launch_pdl(kern, dim3(2 * f.units, B), dim3(attn::F_THR), attn::bwd_smem(D), stream, 1,
                         static_cast<const float*>(qkv), static_cast<const float*>(dctx), lse,
                         static_cast<const float*>(delta), lens, S, H, A, D, f.LD, f.vec, static_cast<float*>(dqkv));
     };
-    if (le == cudaSuccess) le = D <= 64 ? go(attn::attn_bwd_f32<1>) : go(attn::attn_bwd_f32<2>);
+    if (le == cudaSuccess) le = D <= 32 ? go(attn::attn_bwd_f32<8>) : D <= 64 ? go(attn::attn_bwd_f32<16>) : go(attn::attn_bwd_f32<32>);
     if (le != cudaSuccess) return cuda_fail(le, "attention backward launch");
   }
   count_launches(2);

@@ -55,7 +55,8 @@ def test_gemm(form, shape):
 
 @pytest.mark.parametrize("B,S,A,D,lens", [(1, 1, 1, 64, [1]), (2, 15, 3, 32, [15, 1]), (2, 17, 2, 20, [16, 17]),
                                           (1, 65, 2, 128, [64]), (3, 130, 1, 100, [130, 65, 63]),
-                                          (2, 64, 5, 3, [64, 9]), (1, 200, 4, 64, [129])])
+                                          (2, 64, 5, 3, [64, 9]), (1, 200, 4, 64, [129]), (2, 70, 3, 33, [70, 2]),
+                                          (1, 129, 2, 65, [129])])
 def test_attention(B, S, A, D, lens):
     H = A * D
     g = torch.Generator(device="cuda").manual_seed(S + D)
