@@ -166,8 +166,8 @@ sky_status sky_slice_backward(sky_slice* s, const void* dy, void* dx, void* stre
  * (0 <= slot < stash_slots); sky_slice_backward_slot is sky_slice_backward
  * for the most recent forward into that slot (its x, d_len, B, S).  With
  * accumulate == 0 the backward overwrites the gradients; with accumulate == 1
- * it adds this micro-batch's gradients to them (each layer's gradients are
- * formed in a scratch set and added on the device, in call order, so a
+ * it adds this micro-batch's gradients to them (on the device, in call order:
+ * each gets the number that an overwriting backward would store, so a
  * fixed order of calls gives the same bits).  sky_slice_forward /
  * sky_slice_backward are slot 0 without accumulation.  Slots are
  * independent: a forward into slot m leaves the other slots' stashes as

@@ -6,8 +6,8 @@
 // kernel serves all three contraction forms:
 //   warp 0      TMA producer: 128-byte-swizzled tiles of A and B into a
 //               STAGES-deep shared-memory ring (mbarrier complete_tx),
-//   warp 1      MMA issuer: one thread issues tcgen05.mma (M=128, N=256,
-//               K=16) into a TMEM accumulator; two accumulators (512 TMEM
+//   warp 1      MMA issuer: the warp walks the loop and one elected lane issues
+//               tcgen05.mma (M=128, N=256, K=16); two accumulators (512 TMEM
 //               columns) let the epilogue of one tile overlap the next,
 //   warps 2..9  epilogue (two warps per TMEM lane quarter, one per half of
 //               the tile's columns): tcgen05.ld of the accumulator, a
@@ -846,12 +846,6 @@ sky_status launch_bf16(sky_gemm_form form, int M, int N, int K, const void* A, c
   // the fuller last wave gained: QKV at T = 8192 took 47.1 instead of 43.1 us.)
   const int clusters = sms / 2;
   const int64_t m_t = ceil_div(M, pair ? 2 * BM : BM);
-  // 192-wide pair tiles for K-major B and the plain-store epilogue when the
-  // product is less than one wave of 256-wide tiles and still one wave of
-  // 192-wide ones: more SM pairs then share it.  (Over several waves the
-  // narrower tile's main loop, which reuses each A tile for fewer columns,
-  // lost more than the fuller last wave gained: QKV at T = 8192 took 47.1
-  // instead of 43.1 us.)
   const bool narrow = pair && form == SKY_GEMM_XWT && epi == SKY_EPI_STORE && !may_split &&
                       !colsum && !deferred_rows && N % 192 == 0 &&
                       m_t * ceil_div(N, BN) < clusters && m_t * (N / 192) <= clusters;
