@@ -507,16 +507,14 @@ __global__ void __launch_bounds__(RP_WARPS * 32) reduce_segments(const ColSegmen
 // with 16-byte loads (a warp reads 512 contiguous bytes of bf16 per row), the
 // CTA's 8 warps are added in order and part[g][n] is written.
 template <typename T>
-__global__ void __launch_bounds__(256) colsum_partial(const T* __restrict__ x, int rows, int N,
-                                                      float* __restrict__ part) {
-  pdl_wait();
-  pdl_trigger();
+__device__ __forceinline__ void colsum_rows(const T* __restrict__ x, int rows, int N, int groups,
+                                            float* __restrict__ part) {
   __shared__ float red[8][256];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int col = blockIdx.x * 256 + lane * 8;
   float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
   if (col < N) {
-    const int step = gridDim.y * 8;
+    const int step = groups * 8;
     int r = blockIdx.y * 8 + w;
     for (; r + 3 * step < rows; r += 4 * step) {
       float v[4][8];
@@ -544,6 +542,26 @@ __global__ void __launch_bounds__(256) colsum_partial(const T* __restrict__ x, i
     for (int k = 0; k < 8; ++k) s += red[k][threadIdx.x];
     part[(int64_t)blockIdx.y * N + c] = s;
   }
+}
+template <typename T>
+__global__ void __launch_bounds__(256) colsum_partial(const T* __restrict__ x, int rows, int N,
+                                                      float* __restrict__ part) {
+  pdl_wait();
+  pdl_trigger();
+  colsum_rows(x, rows, N, gridDim.y, part);
+}
+// Two matrices of the same rows; blockIdx.z picks one.
+struct ColPair {
+  const float* x[2];
+  float* part[2];
+  int N[2], groups[2];
+};
+__global__ void __launch_bounds__(256) colsum_partial_pair(const ColPair in, int rows) {
+  pdl_wait();
+  pdl_trigger();
+  const int z = blockIdx.z, N = in.N[z], groups = in.groups[z];
+  if (blockIdx.x * 256 >= N || blockIdx.y >= groups) return;  // uniform over the CTA
+  colsum_rows(in.x[z], rows, N, groups, in.part[z]);
 }
 
 template <typename T>
@@ -817,17 +835,28 @@ sky_status column_sum(const void* x, int rows, int N, sky_dtype dt, float* out, 
   SKY_CHECK(ws && ws_bytes >= (size_t)groups * N * sizeof(float), SKY_ERR_INVALID_ARG,
             "column-sum workspace too small");
   float* part = static_cast<float*>(ws);
-  dim3 grid(ceil_div(N, 256), groups);
-  if (dt == SKY_DTYPE_BF16)
-    launch_pdl(rw::colsum_partial<__nv_bfloat16>, dim3(grid), dim3(256), 0, st, 1, 
-        static_cast<const __nv_bfloat16*>(x), rows, N, part);
-  else
-    launch_pdl(rw::colsum_partial<float>, dim3(grid), dim3(256), 0, st, 1, static_cast<const float*>(x), rows, N, part);
-  launch_pdl(rw::reduce_partials, dim3(dim3(ceil_div(N, 32), 1)), dim3(rw::RP_WARPS * 32), 0, st, 1, part, groups, N, out, nullptr,
-                                                                nullptr);
-  count_launches(2);
-  const cudaError_t e = cudaGetLastError();
+  const dim3 grid(ceil_div(N, 256), groups);
+  cudaError_t e = dt == SKY_DTYPE_BF16
+                      ? launch_pdl(rw::colsum_partial<__nv_bfloat16>, grid, dim3(256), 0, st, 1,
+                                   static_cast<const __nv_bfloat16*>(x), rows, N, part)
+                      : launch_pdl(rw::colsum_partial<float>, grid, dim3(256), 0, st, 1, static_cast<const float*>(x),
+                                   rows, N, part);
+  count_launches(1);
+  if (e == cudaSuccess) e = gemm::reduce_rows_f32(part, groups, N, out, st);
   return e == cudaSuccess ? SKY_OK : cuda_fail(e, "column sum launch");
+}
+
+sky_status column_partials_f32(const float* x, int N, float* part, int* parts, const float* x2, int N2, float* part2,
+                               int* parts2, int rows, cudaStream_t st) {
+  SKY_CHECK(N % 8 == 0 && N2 % 8 == 0, SKY_ERR_UNSUPPORTED, "column sum needs N %% 8 == 0 (got %d, %d)", N, N2);
+  *parts = colsum_row_groups(rows, N);
+  *parts2 = colsum_row_groups(rows, N2);
+  const rw::ColPair in{{x, x2}, {part, part2}, {N, N2}, {*parts, *parts2}};
+  const cudaError_t e = launch_pdl(rw::colsum_partial_pair,
+                                   dim3(ceil_div(std::max(N, N2), 256), std::max(*parts, *parts2), 2), dim3(256), 0, st,
+                                   1, in, rows);
+  count_launches(1);
+  return e == cudaSuccess ? SKY_OK : cuda_fail(e, "column partials launch");
 }
 
 sky_status bias_gelu_fwd(const void* z, const void* bias, int rows, int N, sky_dtype dt,

@@ -57,6 +57,10 @@ sky_status to_f32(const void* x, int64_t n, sky_dtype dt, float* out, cudaStream
 size_t column_sum_ws(int rows, int N);
 sky_status column_sum(const void* x, int rows, int N, sky_dtype dt, float* out, void* ws,
                       size_t ws_bytes, cudaStream_t st);
+// Column partials of two fp32 matrices of `rows` rows in one launch, column_sum_ws
+// bytes each, and their counts, for reduce_column_segments.
+sky_status column_partials_f32(const float* x, int N, float* part, int* parts, const float* x2, int N2, float* part2,
+                               int* parts2, int rows, cudaStream_t st);
 sky_status bias_gelu_fwd(const void* z, const void* bias, int rows, int N, sky_dtype dt,
                          void* hpre, void* g, cudaStream_t st);
 sky_status gelu_bwd(const void* dg, const void* hpre, int rows, int N, sky_dtype dt, void* dh,

@@ -436,12 +436,14 @@ sky_status backward_layer(sky_slice* s, int i, const void* dY, sky_dtype dy_dt, 
   };
   void* ws2 = bf ? s->ws2 : nullptr;
   const size_t ws2b = s->ws2_bytes;
-  // bf16: the column sums behind this layer's bias and LayerNorm-parameter
-  // gradients (LN2 and LN1 partials per CTA, db1 partials per 32 rows from
-  // the FFN2 data-gradient epilogue, dbqkv partials per 128-row tile from the
-  // attention backward) land in partial buffers of set k and are added up by
-  // one fixed-order launch on sw at the end of the layer.  Set k was last
-  // used by the layer two above; wait for its reduction before reusing it.
+  // The column sums behind this layer's bias and LayerNorm-parameter gradients
+  // (LN2 and LN1 partials per CTA; db1 and dbqkv partials: bf16 per 32 rows from
+  // the FFN2 data-gradient epilogue and per 128-row tile from the attention
+  // backward, fp32 from one pass over dZ and dQKV) land in partial buffers of set
+  // k and are added up by one fixed-order launch on sw at the end of the layer.
+  // (Summed where each arises, they were eight launches of an fp32 layer instead
+  // of two: 2-layer slice of width 128 170 us a step, now 160.)  Set k was
+  // last used by the layer two above; wait for its reduction before reusing it.
   int ln2_parts = 0, ln1_parts = 0, db1_rows = 0;
   if (bf && two && s->ev_red_live[k]) SKY_CUDA(cudaStreamWaitEvent(st, s->ev_red[k], 0));
   // a9: LN2 backward -> dU2 (fp32 + dtype), dgamma2, dbeta2, db2
@@ -450,8 +452,7 @@ sky_status backward_layer(sky_slice* s, int i, const void* dY, sky_dtype dy_dt, 
     Timed t(s, st, P_LN_BWD, 0, (dye + 4.0 + 4.0 + (bf ? e : 0.0)) * T * H + 8.0 * T);
     SKY_TRY(layernorm_bwd(dY, dy_dt, dY2, Lb.U2, Lb.p[10], Lb.mean2, Lb.rstd2, T, H, dt,
                           bf ? s->dU2_32 : nullptr, s->dU2b, G[10], G[11], G[9],
-                          bf ? s->lnp[k][0] : s->ws, bf ? s->lnp_bytes : s->ws_bytes, st,
-                          bf ? &ln2_parts : nullptr, s->d_status));
+                          s->lnp[k][0], s->lnp_bytes, st, &ln2_parts, s->d_status));
   }
   SKY_TRY(fork(0));
   // a10 + a11: dW2 = dU2^T G (on sw, beside the data gradient);
@@ -469,8 +470,6 @@ sky_status backward_layer(sky_slice* s, int i, const void* dY, sky_dtype dy_dt, 
   } else {
     SKY_TRY(run_gemm(s, st, P_GEMM_DGRAD, SKY_GEMM_XW, T, F, H, s->dU2b, Lb.p[8], s->dH, false,
                      SKY_EPI_GELU_BWD, nullptr, Lb.Gp, nullptr));
-    Timed t(s, st, P_COLSUM, 0, e * T * F);
-    SKY_TRY(column_sum(s->dH, T, F, dt, G[7], s->ws, s->ws_bytes, st));
   }
   SKY_TRY(fork(1));
   // a12: dX1 = dZ W1 + dU2 (fp32; bf16: dU2 added by the GEMM epilogue, fp32:
@@ -487,8 +486,7 @@ sky_status backward_layer(sky_slice* s, int i, const void* dY, sky_dtype dy_dt, 
     Timed t(s, st, P_LN_BWD, 0, (bf ? 4.0 : 8.0) * T * H + (4.0 + 4.0 + (bf ? e : 0.0)) * T * H + 8.0 * T);
     SKY_TRY(layernorm_bwd(s->dP1, SKY_DTYPE_FP32, bf ? nullptr : static_cast<float*>(s->dU2b),
                           Lb.U1, Lb.p[4], Lb.mean1, Lb.rstd1, T, H, dt, bf ? s->dR[k] : nullptr,
-                          dU1b, G[4], G[5], G[3], bf ? s->lnp[k][1] : s->ws,
-                          bf ? s->lnp_bytes : s->ws_bytes, st, bf ? &ln1_parts : nullptr,
+                          dU1b, G[4], G[5], G[3], s->lnp[k][1], s->lnp_bytes, st, &ln1_parts,
                           s->d_status));
   }
   SKY_TRY(fork(2));
@@ -506,12 +504,16 @@ sky_status backward_layer(sky_slice* s, int i, const void* dY, sky_dtype dy_dt, 
                           s->delta, s->d_status, st, bf ? s->qkvp[k] : nullptr));
   }
   SKY_TRY(fork(3));
-  if (bf) {
+  int qkv_rows = B * ceil_div(S, 128);
+  if (!bf) {
+    Timed t(s, sw, P_COLSUM, 0, e * T * (F + 3.0 * H));
+    SKY_TRY(column_partials_f32(static_cast<const float*>(s->dH), F, s->db1p[k], &db1_rows,
+                                static_cast<const float*>(s->dqkv), 3 * H, s->qkvp[k], &qkv_rows, T, sw));
+  }
+  {
     // the layer's eight column reductions in one fixed-order launch on sw:
     // dgamma2, dbeta2, db2 and dgamma1, dbeta1, dbo from the LayerNorm
-    // partials, db1 from the FFN2 data-gradient partials, dbqkv from the
-    // attention backward's partials
-    const int qkv_rows = B * ceil_div(S, 128);
+    // partials, db1 and dbqkv from theirs
     const float* l2 = static_cast<const float*>(s->lnp[k][0]);
     const float* l1 = static_cast<const float*>(s->lnp[k][1]);
     ColSegments sg{};
@@ -524,7 +526,7 @@ sky_status backward_layer(sky_slice* s, int i, const void* dY, sky_dtype dy_dt, 
     sg.seg[6] = {s->db1p[k], G[7], db1_rows, F};
     sg.seg[7] = {s->qkvp[k], G[1], qkv_rows, 3 * H};
     sg.n = 8;
-    sg.add = s->accumulate;
+    sg.add = s->accumulate && bf;
     Timed t(s, sw, P_COLSUM, 0,
             4.0 * (3.0 * (ln2_parts + ln1_parts) * H + (double)db1_rows * F + qkv_rows * 3.0 * H));
     SKY_TRY(reduce_column_segments(sg, sw));
@@ -532,9 +534,6 @@ sky_status backward_layer(sky_slice* s, int i, const void* dY, sky_dtype dy_dt, 
       SKY_CUDA(cudaEventRecord(s->ev_red[k], sw));
       s->ev_red_live[k] = true;
     }
-  } else {  // dbqkv = column sums of dQKV
-    Timed t(s, sw, P_COLSUM, 0, e * T * 3.0 * H);
-    SKY_TRY(column_sum(s->dqkv, T, 3 * H, dt, G[1], s->ws, s->ws_bytes, sw));
   }
   // a16: dX = dQKV Wqkv + dU1;  dWqkv = dQKV^T X.  bf16: dU1 is added by the
   // GEMM epilogue (straight into dx for the slice's first layer with fp32
@@ -814,9 +813,10 @@ static sky_status plan_slice(sky_slice* s, size_t* total) {
   s->stash_bytes = stash * s->L * s->n_slots;
   s->ws_bytes = align_up(workspace_need(s, T));
   s->ws2_bytes = bf ? align_up(side_workspace_need(s, T)) : 0;
-  s->lnp_bytes = bf ? align_up(layernorm_bwd_ws((int)T, s->H)) : 0;
-  s->db1p_bytes = bf ? align_up((size_t)gemm::colpart_rows_max((int)T) * s->F * 4) : 0;
-  s->qkvp_bytes = bf ? align_up((size_t)c.max_batch * ceil_div(c.max_seq, 128) * 3 * s->H * 4) : 0;
+  s->lnp_bytes = align_up(layernorm_bwd_ws((int)T, s->H));
+  s->db1p_bytes = align_up(bf ? (size_t)gemm::colpart_rows_max((int)T) * s->F * 4 : column_sum_ws((int)T, s->F));
+  s->qkvp_bytes = align_up(bf ? (size_t)c.max_batch * ceil_div(c.max_seq, 128) * 3 * s->H * 4
+                              : column_sum_ws((int)T, 3 * s->H));
   // dP[2] dR[2] dU2_32 dP1 | dU2b dU1b dctx (bf16) | dH | dqkv | delta | ws | ws2 | lnp[2] |
   // db1p | qkvp | status | x32 (bf16)
   const size_t wk = (bf ? 7 : 6) * t32 + (bf ? 3 : 1) * th + align_up((size_t)T * s->F * s->esz) +
