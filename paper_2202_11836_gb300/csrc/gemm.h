@@ -61,7 +61,7 @@ int colpart_rows_max(int M);
 // out[n] = sum over r of part[r][n] in order r = 0, 1, ... (rowwise.cu).
 cudaError_t reduce_rows_f32(const float* part, int rows, int N, float* out, cudaStream_t stream);
 size_t workspace_bytes(sky_gemm_form form, int M, int N, int K, bool out_f32);
-int choose_splits(int tiles, int k_blocks, int sms);
+int choose_splits(int64_t mn, int tiles, int k_blocks, int sms);
 // Debug controls: per-wait timeout (0 = default 2 s) and the fault-injection
 // switch that makes the TMA producer skip its loads (waits then time out).
 void set_debug(uint64_t timeout_ns, int skip_loads);

@@ -748,16 +748,23 @@ int colpart_rows_max(int M) {
   return std::max(ceil_div(M, BM) * 4, ceil_div(M, 2 * BM) * 8);
 }
 
-int choose_splits(int tiles, int k_blocks, int sms) {
-  // Estimated makespan (in k-block units) of `tiles * s` units on `sms` CTAs
-  // plus a small per-unit cost; the fixed-order reduce is charged per split.
+int choose_splits(int64_t mn, int tiles, int k_blocks, int sms) {
+  // Estimated makespan (in k-blocks of 0.32 us) of `tiles * s` units on `sms`
+  // CTAs, with four for a unit's epilogue, plus the fixed-order reduction: 2 us,
+  // half a block a split and the bytes of s partials and the result at 8 TB/s (they
+  // are mostly in L2).
+  // Without the bytes, products of a wave or more were split too: 10000 x 768 x
+  // 3072 59.9 us, unsplit 35.1; 8192 x 768 x 3072 48.9 and 34.7; 6000 x 1024 x 4096
+  // 52.0 and 43.0.  Below a wave splits stay: 1024 x 1024 x 8192 40.3, in four 20.2;
+  // 3072 x 1024 x 6144 33.8, in three 32.3.
+  const double partial = static_cast<double>(mn) * 4 / 8e6 / 0.32;
   int best = 1;
   double best_cost = 1e30;
   for (int s = 1; s <= 32 && s <= k_blocks; ++s) {
     const int per = ceil_div(k_blocks, s);
     const int s_eff = ceil_div(k_blocks, per);
     const int waves = ceil_div((int64_t)tiles * s_eff, sms);
-    const double cost = waves * (per + 4.0) + (s_eff > 1 ? 2.0 + 0.5 * s_eff : 0.0);
+    const double cost = waves * (per + 4.0) + (s_eff > 1 ? 6.25 + 0.5 * s_eff + (s_eff + 1) * partial : 0.0);
     if (cost < best_cost - 1e-9) { best_cost = cost; best = s_eff; }
   }
   return best;
@@ -769,7 +776,7 @@ size_t workspace_bytes(sky_gemm_form form, int M, int N, int K, bool out_f32) {
   const int tiles = ceil_div(M, pair ? 2 * BM : BM) * ceil_div(N, BN);
   const int kb = ceil_div(K, BK);
   const int sms = sm_count() > 0 ? sm_count() : 148;
-  const int s = choose_splits(tiles, kb, pair ? sms / 2 : sms);
+  const int s = choose_splits(static_cast<int64_t>(M) * N, tiles, kb, pair ? sms / 2 : sms);
   (void)form;
   return s > 1 ? static_cast<size_t>(s) * M * N * sizeof(float) : 0;
 }
@@ -861,7 +868,7 @@ sky_status launch_bf16(sky_gemm_form form, int M, int N, int K, const void* A, c
   p.m_tiles = static_cast<int>(m_t);
   p.n_tiles = ceil_div(N, tbn);
   p.k_blocks = ceil_div(K, BK);
-  p.splits = may_split ? choose_splits(p.m_tiles * p.n_tiles, p.k_blocks, pair ? sms / 2 : sms) : 1;
+  p.splits = may_split ? choose_splits(static_cast<int64_t>(M) * N, p.m_tiles * p.n_tiles, p.k_blocks, pair ? sms / 2 : sms) : 1;
   if (p.splits > 1) {  // never more partials than the workspace holds
     const size_t cap = ws_bytes / (static_cast<size_t>(M) * N * sizeof(float));
     p.splits = cap < 2 ? 1 : (p.splits < (int)cap ? p.splits : (int)cap);
