@@ -204,16 +204,22 @@ sky_status launch_f32(sky_gemm_form form, int M, int N, int K, const float* A, c
   p.k_slabs = ceil_div(K, TK);
   const int64_t tiles = static_cast<int64_t>(ceil_div(M, TM)) * p.n_tiles;
   const int sms = sm_count() > 0 ? sm_count() : 148;
-  // Splits: a lone CTA waits for its loads, so an SM wants several.  Eight
-  // splits up to ten CTAs an SM, else four, each of two slabs or more (one,
-  // where the tiles are few); never two, whose pairs land on one SM.  us at 1 /
-  // 2 / 4 / 8 splits: 404 x 768 x 3072 146 / 134 / 77 / 52, 404 x 2304 x 768
-  // 65 / 44 / 40 / 41, 1000 x 2304 x 768 77 / 82 / 82 / 86, 128 x 384 x 128
-  // 5.6 / 7.7 / 4.8 / -, 512 x 2048 x 97 12.4 / 16.1 / 15.1 / - (all before the
-  // partial rows were sent rather than read).
+  // Splits: a lone CTA waits for its loads, so an SM wants several.  Eight splits up
+  // to eleven CTAs an SM, else four, each of two slabs or more.  Where the tiles are
+  // few, one slab is enough, and eight only if every CTA has an SM to itself or that
+  // halves the longest one's slabs.
+  // Never two, whose pairs land on one SM.  us at 1 / 2 / 4 / 8 splits: 404 x 768 x
+  // 3072 99 / - / 61 / 51, 404 x 2304 x 768 42 / - / 38 / 40, 1000 x 768 x 3072 171 / - /
+  // 115 / 106, 1000 x 2304 x 768 77 / 82 / 83 / 85, 512 x 2048 x 97 9.9 / 16.1 / 13.1 / -,
+  // 128 x 384 x 128 5.8 / 7.7 / 3.7 / -; 256 x 384 x 384 (12 slabs) 5.8 at four, 7.0 at
+  // eight, 384 x 384 x 256 (8) 6.5 and 6.0, 150 x 448 x 448 (14) 6.8 and 6.5.
   p.ks = 1;
-  for (int ks = 8; ks >= 4 && p.ks == 1; ks /= 2)
-    if (tiles * ks <= 10 * sms && p.k_slabs >= (4 * tiles <= sms ? ks : 2 * ks)) p.ks = ks;
+  const bool few = 4 * tiles <= sms;
+  const bool halves = 2 * ceil_div(p.k_slabs, 8) <= ceil_div(p.k_slabs, 4);
+  for (int ks = 8; ks >= 4 && p.ks == 1; ks /= 2) {
+    const bool one_slab = few && p.k_slabs >= ks && (ks == 4 || 8 * tiles <= sms || halves);
+    if (tiles * ks <= 11 * sms && (p.k_slabs >= 2 * ks || one_slab)) p.ks = ks;
+  }
   const bool vec = p.lda % 4 == 0 && p.ldb % 4 == 0 && (reinterpret_cast<uintptr_t>(A) & 15) == 0 &&
                    (reinterpret_cast<uintptr_t>(B) & 15) == 0;
   SKY_CHECK(tiles * p.ks <= 0x7fffffff, SKY_ERR_INVALID_ARG, "GEMM too large (M=%d N=%d)", M, N);
