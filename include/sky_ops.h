@@ -64,9 +64,9 @@ size_t sky_gemm_workspace_bytes(sky_gemm_form form, int32_t M, int32_t N, int32_
  * A, B, C 16-byte aligned, else UNSUPPORTED); FP32 runs the SIMT kernel.
  * out_dtype: the storage type of C (BF16 only with BF16 input); an FP32
  * output takes the STORE epilogue (with or without bias).  bias uses
- * in_dtype.  An FP32 output with no bias may split the K range over CTAs; the
- * partial sums go to `workspace` and are added in a fixed order
- * (deterministic). */
+ * in_dtype.  The K range may be split over CTAs, whose partial sums are added
+ * in a fixed order (deterministic): inside a thread-block cluster, or, for large
+ * products with an FP32 output and no bias, through `workspace`. */
 sky_status sky_gemm(sky_gemm_form form, int32_t M, int32_t N, int32_t K, sky_dtype in_dtype,
                     const void* A, const void* B, void* C, sky_dtype out_dtype,
                     sky_epilogue epilogue, const void* bias, const void* aux, void* aux_out,
