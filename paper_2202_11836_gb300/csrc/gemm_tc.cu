@@ -49,6 +49,7 @@ namespace gemm {
 constexpr int BM = 128, BN = 256, BK = 64, STAGES = 4;
 constexpr int A_BYTES = BM * BK * 2;        // 16 KiB
 constexpr int NUM_EPI_WARPS = 8;            // two per TMEM lane quarter (default)
+constexpr int SMEM_ALIGN = 128;             // of the dynamic shared memory, as declared
 constexpr int MN_CHUNK_BYTES = 64 * BK * 2; // one 64-wide MN-major box: 8 KiB
 // CTA-pair variant: per CTA and stage A 128 x 64 + B 128 x 64 (32 KiB).  Six
 // stages (192 KiB) for every epilogue but the GELU' data gradient, which
@@ -76,9 +77,12 @@ struct Shape {
   // two fp32 accumulators of 128 x TBN, in a power-of-two TMEM allocation
   static constexpr int TMEM_ALLOC = 2 * TBN <= 256 ? 256 : 512;
   static constexpr int EPI_OFF = NST * SBYTES;  // per epilogue warp: 32 x 32 staging, fp32 or two 16-bit outputs
-  static constexpr int BIAS_OFF = EPI_OFF + EW * 4096;       // bias+GELU: the tile's bias, one copy per accumulator
-  static constexpr int BAR_OFF = BIAS_OFF + (GELU ? 2 * TBN * 2 : 0);
-  static constexpr int SMEM = BAR_OFF + 256 /*barriers*/ + 1024 /*alignment slack*/;
+  static constexpr int BIAS_OFF = EPI_OFF + EW * 4096;       // bias+GELU: each warp's columns of the tile's bias
+  static constexpr int BIAS_BYTES = TBN / (EW / 4) * 2;      // of a warp
+  static constexpr int BAR_OFF = BIAS_OFF + (GELU ? EW * BIAS_BYTES : 0);
+  static constexpr int BAR_BYTES = GELU ? 128 : 256;         // barriers and the TMEM address
+  static constexpr int SMEM = BAR_OFF + BAR_BYTES + 1024 - SMEM_ALIGN /*alignment slack*/;
+  static_assert((2 * NST + 5) * 8 + 4 <= BAR_BYTES, "barrier block");
   static_assert(SMEM <= 232448, "shared memory per CTA");
 };
 constexpr uint32_t kSleepNs = 20000;         // suspend hint of the epilogue's accumulator wait
@@ -151,7 +155,7 @@ __global__ void __launch_bounds__(Shape<EPI, PAIR, TBN>::THREADS, 1)
   constexpr int B_ROWS = PAIR ? TBN / 2 : TBN;  // B rows (tile columns) this CTA loads
   static_assert(!B_MN || B_ROWS % 64 == 0, "MN-major B is loaded in 64-column boxes");
   constexpr int TILE_M = PAIR ? 2 * BM : BM;
-  extern __shared__ uint8_t smem_raw[];
+  extern __shared__ __align__(SMEM_ALIGN) uint8_t smem_raw[];
   const uint32_t raw_addr = ptx::smem_u32(smem_raw);
   uint8_t* smem = smem_raw + (((raw_addr + 1023u) & ~1023u) - raw_addr);
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + SH::BAR_OFF);
@@ -396,11 +400,14 @@ __global__ void __launch_bounds__(Shape<EPI, PAIR, TBN>::THREADS, 1)
         }
       }
       if constexpr (EPI == SKY_EPI_BIAS_GELU) {
-        // this warp's 64 columns of bias (the four warps of a column group write the
-        // same values; a copy per accumulator, as a warp may be one tile ahead)
+        // This warp's 64 columns of bias, in a copy of its own: the four warps of a
+        // column group may be two tiles apart (a tile's MMAs wait for the tile two
+        // before it, and a warp releases its accumulator before it has read the last
+        // chunk's bias), so a copy they shared could be overwritten under a reader.
         const int col = n0 + 2 * lane;
         const uint32_t b2 = col < p.N ? *reinterpret_cast<const uint32_t*>(p.bias + col) : 0u;
-        *reinterpret_cast<uint32_t*>(smem + SH::BIAS_OFF + (acc * TBN + hf * HALF + 2 * lane) * 2) = b2;
+        __syncwarp();  // every lane has read the tile before's
+        *reinterpret_cast<uint32_t*>(smem + SH::BIAS_OFF + (warp - 2) * SH::BIAS_BYTES + 4 * lane) = b2;
         __syncwarp();
       }
       if (!ptx::mbar_wait(&tfull[acc], aphase, lim, p.status, kSleepNs)) break;
@@ -418,7 +425,7 @@ __global__ void __launch_bounds__(Shape<EPI, PAIR, TBN>::THREADS, 1)
         // loop; this takes 4.  4096 x 3072 x 768: 25.3 -> 23.7 us, FFN forward block on
         // 4999 rows, large width, 97.2 -> 94.8.
         uint8_t* sg = reinterpret_cast<uint8_t*>(stage);
-        const uint32_t sbias = ptx::smem_u32(smem + SH::BIAS_OFF) + (acc * TBN + hf * HALF) * 2;
+        const uint32_t sbias = ptx::smem_u32(smem + SH::BIAS_OFF) + (warp - 2) * SH::BIAS_BYTES;
         const uint32_t srow = ptx::smem_u32(sg) + lane * 64;
 #pragma unroll
         for (int c = 0; c < HALF; c += 32) {

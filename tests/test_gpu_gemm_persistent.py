@@ -1,0 +1,53 @@
+"""The persistent GEMM's bias + GELU epilogue over many tiles a CTA with a short K,
+where its warps run tiles apart: every element against float64, and the same bits
+again."""
+import ctypes as C
+import math
+
+import pytest
+
+from paper_2202_11836_gb300 import _lib as L
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+def P(t):
+    return C.c_void_p(0 if t is None else int(t.data_ptr()))
+
+
+def bias_gelu(M, N, K, a, w, bias):
+    c = torch.full((M, N), -7.0, dtype=torch.bfloat16, device="cuda")
+    gp = torch.full((M, N), -7.0, dtype=torch.float16, device="cuda")
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    L.call("sky_gemm", L.SKY_GEMM_XWT, M, N, K, L.SKY_DTYPE_BF16, P(a), P(w), P(c), L.SKY_DTYPE_BF16,
+           L.SKY_EPI_BIAS_GELU, P(bias), None, P(gp), None, 0, P(st),
+           C.c_void_p(int(torch.cuda.current_stream().cuda_stream)))
+    torch.cuda.synchronize()
+    assert int(st.item()) == 0
+    return c, gp
+
+
+# 27 tiles a pair (every row tile crosses all eight column tiles); 5 a pair with a
+# ragged last row and column tile; 3 to 4 a single CTA
+@pytest.mark.parametrize("M,N,K", [(65536, 2048, 256), (2000, 10000, 72), (200, 60000, 72)])
+def test_bias_of_many_tiles(M, N, K):
+    g = torch.Generator(device="cuda").manual_seed(M + N)
+    a = torch.randn(M, K, device="cuda", generator=g).bfloat16()
+    w = (0.05 * torch.randn(N, K, device="cuda", generator=g)).bfloat16()
+    # another value in every column, and a step between column tiles
+    bias = torch.randn(N, device="cuda", generator=g)
+    bias = (bias + (torch.arange(N, device="cuda") // 256 % 5 - 2)).bfloat16()
+    c, gp = bias_gelu(M, N, K, a, w, bias)
+    for r in range(0, M, 8192):
+        z = a[r:r + 8192].double() @ w.double().T + bias.double()
+        phi = 0.5 * (1 + torch.erf(z / math.sqrt(2)))
+        ref, dref = z * phi, phi + z * torch.exp(-0.5 * z * z) / math.sqrt(2 * math.pi)
+        # half an ulp of the outputs (2^-9 bf16, 2^-11 fp16) and as much for the sums;
+        # the erf formula: 2.5e-5, half of it in Phi
+        assert bool(((c[r:r + 8192] - ref).abs() <= 2.0 ** -8 * ref.abs() + 2e-5 * (1 + z.abs())).all())
+        assert bool(((gp[r:r + 8192] - dref).abs() <= 2.0 ** -10 * dref.abs() + 3e-5).all())
+    for _ in range(3):
+        c2, gp2 = bias_gelu(M, N, K, a, w, bias)
+        assert torch.equal(c, c2) and torch.equal(gp, gp2)
