@@ -61,7 +61,8 @@ size_t sky_gemm_workspace_bytes(sky_gemm_form form, int32_t M, int32_t N, int32_
 /* C = epilogue(op(A) * op(B)) with fp32 accumulation (Sec. II-C linear
  * layers).  in_dtype: BF16 runs the tcgen05/TMEM tensor-core kernel (the
  * contiguous dimensions -- K for XWT/XW, M for XTW, and N -- multiples of 8,
- * A, B, C 16-byte aligned, else UNSUPPORTED); FP32 runs the SIMT kernel.
+ * A, B, C 16-byte and bias, aux, aux_out 8-byte aligned, else UNSUPPORTED);
+ * FP32 runs the SIMT kernel.
  * out_dtype: the storage type of C (BF16 only with BF16 input); an FP32
  * output takes the STORE epilogue (with or without bias).  bias uses
  * in_dtype.  The K range may be split over CTAs, whose partial sums are added

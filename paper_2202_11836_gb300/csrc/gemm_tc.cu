@@ -811,6 +811,10 @@ sky_status launch_bf16(sky_gemm_form form, int M, int N, int K, const void* A, c
   SKY_CHECK(epi != SKY_EPI_BIAS_GELU || (bias && aux_out), SKY_ERR_INVALID_ARG,
             "BIAS_GELU epilogue needs bias and aux_out");
   SKY_CHECK(epi != SKY_EPI_GELU_BWD || aux, SKY_ERR_INVALID_ARG, "GELU' epilogue needs aux");
+  // the epilogues read and write these in groups of four 16-bit values
+  const auto a8 = [](const void* q) { return (reinterpret_cast<uintptr_t>(q) & 7) == 0; };
+  SKY_CHECK(a8(bias) && (epi != SKY_EPI_GELU_BWD || a8(aux)) && (epi != SKY_EPI_BIAS_GELU || a8(aux_out)),
+            SKY_ERR_UNSUPPORTED, "GEMM bias, aux and aux_out must be 8-byte aligned");
   SKY_CHECK(!resid || (out_f32 && epi == SKY_EPI_STORE && !colsum && !deferred_rows &&
                        (reinterpret_cast<uintptr_t>(resid) & 15) == 0),
             SKY_ERR_UNSUPPORTED, "a residual needs a 16-byte aligned fp32 output of the STORE epilogue");
