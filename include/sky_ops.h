@@ -47,7 +47,8 @@ typedef enum { SKY_GEMM_XWT = 0, SKY_GEMM_XW = 1, SKY_GEMM_XTW = 2 } sky_gemm_fo
  *               derivative the backward pass needs, stored as IEEE fp16 for
  *               bf16 inputs (finer than bf16 on its range [-0.17, 1.13]) and
  *               as fp32 for fp32 inputs
- *   GELU_BWD  : C = acc * aux[m,n], aux = GELU'(z) as stored by BIAS_GELU
+ *   GELU_BWD  : C = (acc (+ bias[n])) * aux[m,n], aux = GELU'(z) as stored by
+ *               BIAS_GELU
  * sky_gemm takes no residual operand: with the ops of this header the
  * residual is added by sky_layernorm_fwd (its r operand).  The slice
  * (sky_slice.h) adds its residuals inside its own GEMM epilogues. */

@@ -114,7 +114,7 @@ __device__ __forceinline__ float4 bf4(const __nv_bfloat16* p) {
 }
 
 // Epilogues, one instantiation each: bias only (fp32 or bf16 output), bias +
-// GELU, GELU', bias + fp32 residual or LayerNorm residual (fp32 output), and
+// GELU, bias then GELU', bias + fp32 residual or LayerNorm residual (fp32 output), and
 // C += product (fp32).
 enum { E_STORE, E_GELU, E_GELU_BWD, E_RESID, E_ADD };
 
@@ -275,7 +275,7 @@ __global__ void __launch_bounds__(C_THREADS, 2)
   } else {
     const int col = n0 + 4 * (et % GPR);
     if (col < p.N) {
-      if (EP != E_GELU_BWD && p.bias) bias4 = bf4(p.bias + col);
+      if (p.bias) bias4 = bf4(p.bias + col);
       if (EP == E_RESID && p.ln_mean) {
         gm4 = bf4(p.ln_gamma + col);
         be4 = bf4(p.ln_beta + col);
@@ -398,9 +398,7 @@ __global__ void __launch_bounds__(C_THREADS, 2)
           continue;
         }
         const int64_t off = static_cast<int64_t>(row) * p.N + col;
-        if constexpr (EP != E_GELU_BWD) {
-          v[u].x += bias4.x; v[u].y += bias4.y; v[u].z += bias4.z; v[u].w += bias4.w;
-        }
+        v[u].x += bias4.x; v[u].y += bias4.y; v[u].z += bias4.z; v[u].w += bias4.w;
         if constexpr (EP == E_GELU) {
           float gp[4];
           gelu_and_grad_as(v[u].x, v[u].x, gp[0]);

@@ -1,6 +1,6 @@
 """The persistent GEMM's bias + GELU epilogue over many tiles a CTA with a short K,
 where its warps run tiles apart: every element against float64, and the same bits
-again."""
+again.  And what it has to share with the kernels that take the other sizes."""
 import ctypes as C
 import math
 
@@ -51,3 +51,22 @@ def test_bias_of_many_tiles(M, N, K):
     for _ in range(3):
         c2, gp2 = bias_gelu(M, N, K, a, w, bias)
         assert torch.equal(c, c2) and torch.equal(gp, gp2)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("M,N,K", [(70, 136, 840), (1100, 1152, 2240), (2000, 3000, 72), (200, 20000, 72)])
+def test_bias_before_the_gelu_gradient(M, N, K, dtype):
+    """A bias given with GELU_BWD is added first, in every kernel."""
+    g = torch.Generator(device="cuda").manual_seed(M + N)
+    dt, at = (torch.bfloat16, torch.float16) if dtype == "bf16" else (torch.float32, torch.float32)
+    a = torch.randn(M, K, device="cuda", generator=g).to(dt)
+    w = (0.05 * torch.randn(N, K, device="cuda", generator=g)).to(dt)
+    bias = torch.randn(N, device="cuda", generator=g).to(dt)
+    aux = (0.5 + 0.3 * torch.randn(M, N, device="cuda", generator=g)).to(at)
+    c = torch.full((M, N), -7.0, dtype=dt, device="cuda")
+    code = L.SKY_DTYPE_BF16 if dtype == "bf16" else L.SKY_DTYPE_FP32
+    L.call("sky_gemm", L.SKY_GEMM_XWT, M, N, K, code, P(a), P(w), P(c), code, L.SKY_EPI_GELU_BWD, P(bias), P(aux),
+           None, None, 0, None, C.c_void_p(int(torch.cuda.current_stream().cuda_stream)))
+    ref = (a.double() @ w.double().T + bias.double()) * aux.double()
+    # an output's rounding (2^-9 at most for bf16); fp32 sums of K terms
+    assert float((c - ref).norm() / ref.norm()) <= (4e-3 if dtype == "bf16" else 1e-5)
