@@ -111,6 +111,7 @@ __device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
 // gelu_and_grad_as of two values, in packed arithmetic where it pairs up, with
 // the sign handled without branches: with q = Phi(-|h|),
 //   GELU(h) = max(h, 0) - |h| q,   Phi(h) = 1/2 + sign(h) (1/2 - q).
+// The factor of q stops at 64, where q is 0 long since, so that GELU(+inf) is +inf.
 __device__ __forceinline__ void gelu_and_grad_as2(float h0, float h1, float2& g, float2& gp) {
   const auto both = [](float v) { return pack2(v, v); };
   float t0, t1, e0, e1;
@@ -127,8 +128,8 @@ __device__ __forceinline__ void gelu_and_grad_as2(float h0, float h1, float2& g,
   poly = mul2(t, fma2(t, poly, both(0.5f * 0.3480242f)));
   const uint64_t q = mul2(poly, E);
   const float2 qq = unpack2(q);
-  g.x = fmaf(-fabsf(h0), qq.x, fmaxf(h0, 0.f));
-  g.y = fmaf(-fabsf(h1), qq.y, fmaxf(h1, 0.f));
+  g.x = fmaf(-fabsf(fminf(h0, 64.f)), qq.x, fmaxf(h0, 0.f));
+  g.y = fmaf(-fabsf(fminf(h1, 64.f)), qq.y, fmaxf(h1, 0.f));
   const uint64_t s = pack2(copysignf(1.f, h0), copysignf(1.f, h1));
   const uint64_t Phi = fma2(s, fma2(q, both(-1.f), both(0.5f)), both(0.5f));
   gp = unpack2(fma2(mul2(h, both(0.3989422804014327f)), E, Phi));

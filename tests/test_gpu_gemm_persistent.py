@@ -70,3 +70,22 @@ def test_bias_before_the_gelu_gradient(M, N, K, dtype):
     ref = (a.double() @ w.double().T + bias.double()) * aux.double()
     # an output's rounding (2^-9 at most for bf16); fp32 sums of K terms
     assert float((c - ref).norm() / ref.norm()) <= (4e-3 if dtype == "bf16" else 1e-5)
+
+
+@pytest.mark.parametrize("M,N", [(64, 256), (300, 8008), (129, 20000)])
+def test_gelu_of_infinities(M, N):
+    """GELU of an overflowed pre-activation is the same in both kernels (the cluster
+    kernel takes the first shape): +inf of +inf, NaN of NaN."""
+    K = 64
+    g = torch.Generator(device="cuda").manual_seed(N)
+    a = torch.randn(M, K, device="cuda", generator=g).bfloat16()
+    w = (0.05 * torch.randn(N, K, device="cuda", generator=g)).bfloat16()
+    bias = torch.randn(N, device="cuda", generator=g).bfloat16()
+    bias[3::17], bias[5::17], bias[7::17] = math.inf, math.nan, 1e30
+    c, _ = bias_gelu(M, N, K, a, w, bias)
+    z = a.double() @ w.double().T + bias.double()
+    ref = z * 0.5 * (1 + torch.erf(z / math.sqrt(2)))
+    inf, nan = torch.isinf(ref), torch.isnan(ref)
+    assert torch.equal(torch.isnan(c), nan) and bool((c[inf] == math.inf).all())
+    f = ~(inf | nan)
+    assert bool(((c[f] - ref[f]).abs() <= 2.0 ** -8 * ref[f].abs() + 2e-5 * (1 + z[f].abs())).all())
