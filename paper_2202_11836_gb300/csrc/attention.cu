@@ -9,6 +9,8 @@
 // ones form it in their one backward launch).
 // fp32: blocks of query (or key) rows against tiles of the other side, exact
 // fp32 arithmetic.
+#include <cfloat>
+
 #include "common.cuh"
 #include "ptx.cuh"
 
@@ -307,7 +309,8 @@ __global__ void __launch_bounds__(F_THR) attn_fwd_f32(const float* __restrict__ 
         s[i][c] = k0 + tx + 16 * c < len ? s[i][c] * sc : -INFINITY;
         mx = fmaxf(mx, s[i][c]);
       }
-      const float mn = fmaxf(m[i], half_warp_max(mx));
+      // (finite also while every score so far is -inf: those keys then add nothing)
+      const float mn = fmaxf(fmaxf(m[i], half_warp_max(mx)), -FLT_MAX);
       const float al = expf(m[i] - mn);  // 0 in the first tile
       m[i] = mn;
       float sum = 0.f;

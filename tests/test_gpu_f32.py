@@ -85,3 +85,33 @@ def test_attention(B, S, A, D, lens):
     assert l2rel(to_host(d), ref_d.cpu().numpy()) <= 3e-6
     for i, n in enumerate(lens):  # padded keys: exactly zero
         assert not d[i, n:, H:].any()
+
+
+@pytest.mark.parametrize("S,len_,hidden", [(130, 130, 64), (130, 129, 128), (64, 40, 20), (200, 200, 1)])
+def test_attention_first_scores_overflow(S, len_, hidden):
+    """Keys whose scores overflow to -inf get probability 0, also where they fill the
+    first tiles of 64 keys; a row that sees only such keys is NaN, as 0 / 0 is."""
+    A, D = 2, 32
+    H = A * D
+    g = torch.Generator(device="cuda").manual_seed(S + hidden)
+    qkv = torch.randn(2, S, 3 * H, device="cuda", generator=g)
+    z = qkv.view(2, S, 3, A, D)
+    z[:, :, 0, :, 0] = 1e20
+    z[:, :, 1, :, 0] = 0.0
+    z[:, :hidden, 1, 0, 0] = -1e20  # head 0's first keys, both sequences
+    z[1, :, 1, 1, 0] = -1e20        # head 1 of sequence 1: every key
+    ln = torch.tensor([len_, len_], dtype=torch.int32, device="cuda")
+    ctx, lse = torch.empty(2, S, H, device="cuda"), torch.empty(2, A, S, device="cuda")
+    L.call("sky_attention_fwd", P(qkv), P(ln), 2, S, H, A, F32, P(ctx), P(lse), None, stream())
+    torch.cuda.synchronize()
+    q, k, v = qkv.double().view(2, S, 3, A, D).permute(2, 0, 3, 1, 4)
+    s = q[..., 1:] @ k[..., 1:].transpose(-1, -2) / D ** 0.5
+    s = s.masked_fill((torch.arange(S, device="cuda") >= len_)[None, None, None, :], -np.inf)
+    s[:, 0, :, :hidden] = -np.inf
+    ref = (torch.softmax(s, -1) @ v).permute(0, 2, 1, 3)
+    ref_lse = torch.logsumexp(s, -1) / np.log(2.0)
+    c = ctx.view(2, S, A, D)
+    for b, a in ((0, 0), (0, 1), (1, 0)):
+        assert l2rel(to_host(c[b, :, a]), ref[b, :, a].cpu().numpy()) <= 2e-6
+        assert maxrel(to_host(lse[b, a]), ref_lse[b, a].cpu().numpy()) <= 2e-6
+    assert bool(torch.isnan(c[1, :, 1]).all())
