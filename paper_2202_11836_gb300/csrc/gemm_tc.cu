@@ -410,7 +410,8 @@ __global__ void __launch_bounds__(Shape<EPI, PAIR, TBN>::THREADS, 1)
         *reinterpret_cast<uint32_t*>(smem + SH::BIAS_OFF + (warp - 2) * SH::BIAS_BYTES + 4 * lane) = b2;
         __syncwarp();
       }
-      if (!ptx::mbar_wait(&tfull[acc], aphase, lim, p.status, kSleepNs)) break;
+      // (one verdict a warp: the loads of the accumulator take all its lanes)
+      if (!__all_sync(0xffffffffu, ptx::mbar_wait(&tfull[acc], aphase, lim, p.status, kSleepNs))) break;
       ptx::tc_fence_after();
       const uint32_t taddr = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + acc * TBN + hf * HALF;
       float* outf = OUT_F32 ? static_cast<float*>(p.C) +

@@ -72,3 +72,43 @@ def test_slice_reports_timeout_then_recovers():
         y = s.forward(x, ln)
         s.sync()  # OK again
         assert torch.isfinite(y.float()).all()
+
+
+# of the persistent kernel: SM pairs and single CTAs, bf16 and fp32 output, each epilogue
+@pytest.mark.parametrize("M,N", [(2048, 4096), (200, 25000)])
+@pytest.mark.parametrize("epi,f32", [(L.SKY_EPI_STORE, False), (L.SKY_EPI_STORE, True), (L.SKY_EPI_BIAS_GELU, False),
+                                     (L.SKY_EPI_GELU_BWD, False)])
+def test_persistent_gemm_timeout(M, N, epi, f32):
+    """More than two 128 x 64 tiles an SM: the persistent kernel.  Its producer, MMA
+    and epilogue warps give up, nothing is stored, and the next call is right."""
+    K = 192
+    g = torch.Generator(device="cuda").manual_seed(N + epi)
+    a = torch.randn(M, K, device="cuda", generator=g).bfloat16()
+    w = (0.05 * torch.randn(N, K, device="cuda", generator=g)).bfloat16()
+    bias = torch.randn(N, device="cuda", generator=g).bfloat16()
+    aux = torch.randn(M, N, device="cuda", generator=g).half()
+    out = torch.full((M, N), -7.0, dtype=torch.float32 if f32 else torch.bfloat16, device="cuda")
+    gp = torch.full((M, N), -7.0, dtype=torch.float16, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+
+    def go():
+        L.call("sky_gemm", L.SKY_GEMM_XWT, M, N, K, 0, P(a), P(w), P(out), int(f32), epi, P(bias), P(aux), P(gp), None,
+               0, P(status), stream())
+        torch.cuda.synchronize()
+
+    L.lib().sky_debug_gemm_fault(20_000_000, 1)
+    try:
+        go()
+    finally:
+        L.lib().sky_debug_gemm_fault(0, 0)
+    assert int(status.item()) & 2, "timeout bit not set"
+    assert bool((out == -7.0).all()) and bool((gp == -7.0).all())
+    status.zero_()
+    go()
+    assert int(status.item()) == 0
+    z = a.double() @ w.double().T + bias.double()
+    if epi == L.SKY_EPI_BIAS_GELU:
+        z = z * 0.5 * (1 + torch.erf(z / 2 ** 0.5))
+    elif epi == L.SKY_EPI_GELU_BWD:
+        z = z * aux.double()
+    assert float((out - z).norm() / z.norm()) <= (1e-5 if f32 else 4e-3)
