@@ -181,7 +181,10 @@ sky_status sky_column_sum_noalloc(const void* x, int32_t T, int32_t N, sky_dtype
  * (0 restores the default, 2 s).  skip_loads != 0 makes the TMA producer
  * arrive on its barriers without issuing the copies, so the consumers' waits
  * run out: the kernel then sets the timeout bit (2) of the status word it was
- * given, frees its tensor memory and exits, and the context stays usable.
+ * given, frees its tensor memory and exits without storing the tiles
+ * concerned, and the context stays usable.  skip_loads == 2: of a product
+ * whose K range is split over a cluster only the last part's copies are left
+ * out.
  * Process-wide setting; pass (0, 0) to restore normal operation. */
 void sky_debug_gemm_fault(uint64_t limit_ns, int32_t skip_loads);
 

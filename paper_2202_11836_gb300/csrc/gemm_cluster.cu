@@ -66,7 +66,7 @@ struct ClusterParams {
   const __nv_bfloat16* ln_beta;
   int32_t* status;
   uint64_t timeout_ns;
-  int skip_loads;
+  int skip_loads;  // fault injection: no TMA copies (2: only the last split's are left out)
 };
 
 // Tile and split of an instantiation, and what follows from them.
@@ -130,7 +130,11 @@ __global__ void __launch_bounds__(C_THREADS, 2)
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + p.bar_off);
   uint64_t* empty = full + C_MAX_STAGES;
   uint64_t* tfull = empty + C_MAX_STAGES;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tfull + 1);
+  uint64_t* done = tfull + 1;  // after a time-out: the issued MMAs have finished
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
+  // Set in every CTA of the cluster by one whose accumulator did not come: no part
+  // of the tile is stored then.
+  const uint32_t lost = ptx::smem_u32(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t crank = ptx::cluster_ctarank();
@@ -149,6 +153,9 @@ __global__ void __launch_bounds__(C_THREADS, 2)
       ptx::mbar_init(&empty[s], 1);
     }
     ptx::mbar_init(tfull, 1);
+    ptx::mbar_init(done, 1);
+    ptx::st_shared_u32(lost, 0);
+    if (TL::PUSH) ptx::fence_cluster();  // with the arrival below: before a peer writes it
     ptx::fence_mbar_init_cluster();
     ptx::fence_proxy_async_smem();
     ptx::prefetch_tensormap(&tmA);
@@ -187,6 +194,7 @@ __global__ void __launch_bounds__(C_THREADS, 2)
 
   if (warp == 0) {
     const bool issuer = ptx::elect_one();
+    const bool skip = p.skip_loads != 0 && (p.skip_loads != 2 || split == KS - 1);  // fault injection
     int stage = 0, issued = 0;
     uint32_t phase = 0;
     for (int kb = kb0; kb < kb1; ++kb) {
@@ -196,7 +204,7 @@ __global__ void __launch_bounds__(C_THREADS, 2)
         uint8_t* sb = sa + C_A_BYTES;
         // a pair's leader barrier expects both CTAs' bytes
         if (half == 0) ptx::mbar_arrive_expect_tx(&full[stage], (PAIR ? 2 : 1) * SBYTES);
-        if (!p.skip_loads) {
+        if (!skip) {
           const int k0 = kb * CBK;
           auto load = [&](void* dst, const CUtensorMap* map, int c0, int c1) {
             if constexpr (PAIR)
@@ -235,10 +243,9 @@ __global__ void __launch_bounds__(C_THREADS, 2)
     // one elected lane issues.
     if (half == 0) {
       constexpr uint32_t idesc = ptx::idesc_bf16_f32(TL::TILE_M, BN, A_MN, B_MN);
-      const uint16_t mask = static_cast<uint16_t>(3u << lead_rank);
       const bool issuer = ptx::elect_one();
-      auto commit = [&](uint64_t* bar) {
-        if constexpr (PAIR) ptx::tc_commit_pair(bar, mask);
+      auto commit = [&](uint64_t* bar, uint32_t to = 3) {  // pair: bit 0 this CTA, bit 1 its peer
+        if constexpr (PAIR) ptx::tc_commit_pair(bar, static_cast<uint16_t>(to << lead_rank));
         else ptx::tc_commit(bar);
       };
       const uint32_t s0 = ptx::smem_u32(smem);
@@ -266,11 +273,14 @@ __global__ void __launch_bounds__(C_THREADS, 2)
         __syncwarp();
         if (++stage == p.stages) { stage = 0; phase ^= 1u; }
       }
-      // on a timeout the issued MMAs still have to finish before TMEM is released
+      // The issued MMAs have to finish before TMEM is released.  On a timeout they
+      // do so behind a barrier that no epilogue waits for.
       if (issuer) {
-        commit(tfull);
-        if (!good) ptx::mbar_wait(tfull, 0, lim, p.status);
+        if (good) commit(tfull);
+        else commit(done, 1);
+        ptx::mbar_wait(good ? tfull : done, 0, lim, p.status);
       }
+      __syncwarp();
     }
   } else {
     const int col = n0 + 4 * (et % GPR);
@@ -300,6 +310,9 @@ __global__ void __launch_bounds__(C_THREADS, 2)
     }
     // ---------------------- accumulator rows -> their owners' shared memory
     const int q = warp & 3, hf = (warp - 2) >> 2;
+    auto give_up = [&]() {
+      if (lane < TL::CL) ptx::st_cluster_u32(ptx::mapa_shared(lost, lane), 1);
+    };
     ok = ptx::mbar_wait(tfull, 0, lim, p.status, kClusterHint);
     ok = __all_sync(0xffffffffu, ok);
     if (ok) {
@@ -318,11 +331,14 @@ __global__ void __launch_bounds__(C_THREADS, 2)
           ptx::st_shared_v4(dst + (((hf * (BN / 8) + (c >> 2) + j) ^ (r & 7)) << 4), v[4 * j], v[4 * j + 1],
                             v[4 * j + 2], v[4 * j + 3]);
       }
+    } else if (!TL::PUSH) {
+      give_up();
     }
     if constexpr (TL::PUSH) {
       // rows to their owners, half a warp a row (a row a lane, straight from the
       // accumulator, took 1.3 us instead of 0.5)
       ptx::cluster_wait();  // every peer runs
+      if (!ok) give_up();
       asm volatile("bar.sync 1, 256;" ::: "memory");
       const uint32_t sm0 = ptx::smem_u32(smem);
       constexpr int N = CBM * GPR / C_EPI;
@@ -381,6 +397,7 @@ __global__ void __launch_bounds__(C_THREADS, 2)
           }
         }
       }
+      if (b == 0) ok = ptx::ld_shared_u32(lost) == 0;  // (behind the first sums' loads)
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         v[u] = w[u][0];

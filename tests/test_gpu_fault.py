@@ -112,3 +112,35 @@ def test_persistent_gemm_timeout(M, N, epi, f32):
     elif epi == L.SKY_EPI_GELU_BWD:
         z = z * aux.double()
     assert float((out - z).norm() / z.norm()) <= (1e-5 if f32 else 4e-3)
+
+
+# of the cluster kernel: unsplit, two, three and six splits, pairs, 128-wide tiles
+@pytest.mark.parametrize("form,M,N,K", [(L.SKY_GEMM_XWT, 256, 512, 256), (L.SKY_GEMM_XWT, 700, 768, 1024),
+                                        (L.SKY_GEMM_XWT, 384, 768, 1024), (L.SKY_GEMM_XWT, 64, 768, 3072),
+                                        (L.SKY_GEMM_XWT, 2048, 768, 3072), (L.SKY_GEMM_XTW, 1024, 4096, 512)])
+@pytest.mark.parametrize("skip", [1, 2])
+def test_cluster_gemm_timeout_stores_nothing(form, M, N, K, skip):
+    """Also where the others' parts of a tile are complete (skip = 2), their sum is
+    not stored."""
+    g = torch.Generator(device="cuda").manual_seed(M + K)
+    a = torch.randn((K, M) if form == L.SKY_GEMM_XTW else (M, K), device="cuda", generator=g).bfloat16()
+    w = (0.05 * torch.randn((K, N) if form == L.SKY_GEMM_XTW else (N, K), device="cuda", generator=g)).bfloat16()
+    out = torch.full((M, N), -7.0, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+
+    def go():
+        L.call("sky_gemm", form, M, N, K, 0, P(a), P(w), P(out), 1, 0, None, None, None, None, 0, P(status), stream())
+        torch.cuda.synchronize()
+
+    L.lib().sky_debug_gemm_fault(20_000_000, skip)
+    try:
+        go()
+    finally:
+        L.lib().sky_debug_gemm_fault(0, 0)
+    assert int(status.item()) & 2, "timeout bit not set"
+    assert bool((out == -7.0).all())
+    status.zero_()
+    go()
+    assert int(status.item()) == 0
+    ref = a.double().T @ w.double() if form == L.SKY_GEMM_XTW else a.double() @ w.double().T
+    assert float((out - ref).norm() / ref.norm()) <= 1e-5
