@@ -10,6 +10,7 @@
 // fp32: blocks of query (or key) rows against tiles of the other side, exact
 // fp32 arithmetic.
 #include <cfloat>
+#include <type_traits>
 
 #include "common.cuh"
 #include "ptx.cuh"
@@ -443,6 +444,8 @@ __global__ void __launch_bounds__(F_THR, G > 16 ? 1 : 4) attn_bwd_f32(const floa
 constexpr int row_stride(int D) { return (D + 3) / 4 * 4 + 4; }
 constexpr int fwd_smem(int D) { return ((FR + 2 * FC) * row_stride(D) + FR * FP_LD) * 4; }
 constexpr int bwd_smem(int D) { return ((2 * FR + 2 * FC) * row_stride(D) + 2 * FR * FP_LD + 2 * FC) * 4; }
+template <int G>
+using Group = std::integral_constant<int, G>;
 struct F32Shape {
   unsigned units;
   int LD;
@@ -481,17 +484,17 @@ sky_status attention_fwd(const void* qkv, const int32_t* lens, int B, int S, int
     SKY_CHECK(D <= 128, SKY_ERR_UNSUPPORTED, "fp32 attention needs head dim <= 128");
     SKY_CHECK(S <= 3072, SKY_ERR_UNSUPPORTED, "fp32 attention: sequence too long");
     const attn::F32Shape f(S, H, A, D, qkv, ctx, nullptr);
-    static const cudaError_t attr[3] = {  // once, for the largest head dim of each
-        cudaFuncSetAttribute(attn::attn_fwd_f32<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, attn::fwd_smem(32)),
-        cudaFuncSetAttribute(attn::attn_fwd_f32<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, attn::fwd_smem(64)),
-        cudaFuncSetAttribute(attn::attn_fwd_f32<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, attn::fwd_smem(128))};
-    const auto go = [&](auto kern) {
+    const auto go = [&](auto group, auto kern) {  // `group` threads a row: head dims up to four times that
+      static OncePerDevice once;
+      const cudaError_t e = allow_smem(once, kern, attn::fwd_smem(4 * decltype(group)::value));
+      if (e != cudaSuccess) return e;
       return launch_pdl(kern, dim3(f.units, B), dim3(attn::F_THR), attn::fwd_smem(D), stream, 1,
                         static_cast<const float*>(qkv), lens, S, H, A, D, f.LD, f.vec, static_cast<float*>(ctx), lse,
                         status);
     };
-    cudaError_t le = attr[(D > 32) + (D > 64)];
-    if (le == cudaSuccess) le = D <= 32 ? go(attn::attn_fwd_f32<8>) : D <= 64 ? go(attn::attn_fwd_f32<16>) : go(attn::attn_fwd_f32<32>);
+    const cudaError_t le = D <= 32   ? go(attn::Group<8>{}, attn::attn_fwd_f32<8>)
+                           : D <= 64 ? go(attn::Group<16>{}, attn::attn_fwd_f32<16>)
+                                     : go(attn::Group<32>{}, attn::attn_fwd_f32<32>);
     if (le != cudaSuccess) return cuda_fail(le, "attention forward launch");
   }
   count_launches(1);
@@ -543,17 +546,18 @@ sky_status attention_bwd(const void* qkv, const void* ctx, const void* dctx, con
                                 static_cast<const float*>(ctx), static_cast<const float*>(dctx), S, H, A, D, rows,
                                 delta);
     const attn::F32Shape f(S, H, A, D, qkv, dctx, dqkv);
-    static const cudaError_t attr[3] = {
-        cudaFuncSetAttribute(attn::attn_bwd_f32<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, attn::bwd_smem(32)),
-        cudaFuncSetAttribute(attn::attn_bwd_f32<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, attn::bwd_smem(64)),
-        cudaFuncSetAttribute(attn::attn_bwd_f32<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, attn::bwd_smem(128))};
-    if (le == cudaSuccess) le = attr[(D > 32) + (D > 64)];
-    const auto go = [&](auto kern) {
+    const auto go = [&](auto group, auto kern) {
+      static OncePerDevice once;
+      const cudaError_t e = allow_smem(once, kern, attn::bwd_smem(4 * decltype(group)::value));
+      if (e != cudaSuccess) return e;
       return launch_pdl(kern, dim3(2 * f.units, B), dim3(attn::F_THR), attn::bwd_smem(D), stream, 1,
                         static_cast<const float*>(qkv), static_cast<const float*>(dctx), lse,
                         static_cast<const float*>(delta), lens, S, H, A, D, f.LD, f.vec, static_cast<float*>(dqkv));
     };
-    if (le == cudaSuccess) le = D <= 32 ? go(attn::attn_bwd_f32<8>) : D <= 64 ? go(attn::attn_bwd_f32<16>) : go(attn::attn_bwd_f32<32>);
+    if (le == cudaSuccess)
+      le = D <= 32   ? go(attn::Group<8>{}, attn::attn_bwd_f32<8>)
+           : D <= 64 ? go(attn::Group<16>{}, attn::attn_bwd_f32<16>)
+                     : go(attn::Group<32>{}, attn::attn_bwd_f32<32>);
     if (le != cudaSuccess) return cuda_fail(le, "attention backward launch");
   }
   count_launches(2);

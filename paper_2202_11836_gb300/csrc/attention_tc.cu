@@ -1597,7 +1597,8 @@ sky_status attention_fwd_tc(const void* qkv, const int32_t* lens, int B, int S, 
   if (S <= 128 && B <= 65535) {  // one tile a sequence
     SKY_CHECK(head_map(&tq, qkv, T, 3 * H, BQ) && seq_map(&tout, ctx, B, S, H, BQ), SKY_ERR_CUDA,
               "cuTensorMapEncodeTiled failed for the attention operands");
-    static cudaError_t at = cudaFuncSetAttribute(attn_fwd_short_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, FS_SMEM);
+    static OncePerDevice once;
+    const cudaError_t at = allow_smem(once, attn_fwd_short_tc, FS_SMEM);
     if (at != cudaSuccess) return cuda_fail(at, "attention smem attribute");
     FwdParams p{S, H, A, lens, static_cast<__nv_bfloat16*>(ctx), lse, status, timeout_ns};
     const cudaError_t e = launch_pdl(attn_fwd_short_tc, dim3(A, B), dim3(NTHR), FS_SMEM, stream, 1, tq, tout, p);
@@ -1626,8 +1627,8 @@ sky_status attention_fwd_tc(const void* qkv, const int32_t* lens, int B, int S, 
   auto go = [&](auto splits, auto bufs) {
     constexpr int KS = decltype(splits)::value, NS = decltype(bufs)::value;
     auto kern = attn_fwd_tc<KS, NS>;
-    static cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   FwdShape<NS>::SMEM);
+    static OncePerDevice once;
+    const cudaError_t attr = allow_smem(once, kern, FwdShape<NS>::SMEM);
     if (attr != cudaSuccess) return attr;
     return launch_pdl(kern, dim3(ceil_div(S, BQ) * KS, A, B), dim3(NTHR), FwdShape<NS>::SMEM, stream, KS, tq, tkv,
                       tout, p);
@@ -1651,8 +1652,8 @@ sky_status attention_bwd_short_tc(const void* qkv, const void* ctx, const void* 
   SKY_CHECK(head_map(&tq, qkv, T, 3 * H, BQ) && head_map(&to, dctx, T, H, BQ) && head_map(&tc, ctx, T, H, BQ) &&
                 seq_map(&tout, dqkv, B, S, 3 * H, BQ),
             SKY_ERR_CUDA, "cuTensorMapEncodeTiled failed for the attention backward operands");
-  static cudaError_t attr =
-      cudaFuncSetAttribute(attn_bwd_short_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, SH_SMEM);
+  static OncePerDevice once;
+  const cudaError_t attr = allow_smem(once, attn_bwd_short_tc, SH_SMEM);
   if (attr != cudaSuccess) return cuda_fail(attr, "attention backward smem attribute");
   BwdParams p{S, H, A, lens, lse, nullptr, nullptr, static_cast<__nv_bfloat16*>(dqkv), colpart, status, timeout_ns};
   const cudaError_t e = launch_pdl(attn_bwd_short_tc, dim3(A, B), dim3(SH_THR), SH_SMEM, stream, 1, tq, to, tc,
@@ -1675,8 +1676,8 @@ sky_status attention_bwd_tc(const void* qkv, const void* dctx, const float* lse,
                 head_map(&tq64, qkv, T, 3 * H, BQ2) && head_map(&to64, dctx, T, H, BQ2) &&
                 seq_map(&tout, dqkv, B, S, 3 * H, BK2),
             SKY_ERR_CUDA, "cuTensorMapEncodeTiled failed for the attention backward operands");
-  static cudaError_t a1 = cudaFuncSetAttribute(attn_bwd_dq_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, DQ_SMEM);
-  static cudaError_t a2 = cudaFuncSetAttribute(attn_bwd_dkdv_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, KV_SMEM);
+  static OncePerDevice once1, once2;
+  const cudaError_t a1 = allow_smem(once1, attn_bwd_dq_tc, DQ_SMEM), a2 = allow_smem(once2, attn_bwd_dkdv_tc, KV_SMEM);
   if (a1 != cudaSuccess) return cuda_fail(a1, "attention dQ smem attribute");
   if (a2 != cudaSuccess) return cuda_fail(a2, "attention dK/dV smem attribute");
   SKY_CHECK((reinterpret_cast<uintptr_t>(xtab) & 15) == 0, SKY_ERR_INVALID_ARG,

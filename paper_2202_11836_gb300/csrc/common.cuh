@@ -10,6 +10,7 @@
 
 #include "../../include/sky_ops.h"
 #include "../../include/sky_slice.h"
+#include "device_once.h"
 
 namespace sky {
 
@@ -179,6 +180,18 @@ __device__ __forceinline__ void pdl_trigger() {
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 bool pdl_enabled();
+
+// Allows a kernel `bytes` of dynamic shared memory, which is a setting of each
+// device: `once` is the kernel's own, static at its launch site.
+template <typename K>
+cudaError_t allow_smem(OncePerDevice& once, K* kern, size_t bytes) {
+  int device = -1;
+  const cudaError_t e = cudaGetDevice(&device);
+  if (e != cudaSuccess) return e;
+  return once(device, [&] {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+  });
+}
 
 // cudaLaunchKernelEx with the programmatic-serialization attribute (when
 // enabled) and optionally a cluster of `cluster_x` CTAs.

@@ -479,7 +479,8 @@ __global__ void __launch_bounds__(C_THREADS, 2)
 template <bool A_MN, bool B_MN, class TL, int EP>
 cudaError_t launch_one(ClusterParams& p, const CUtensorMap& ta, const CUtensorMap& tb, cudaStream_t st) {
   auto kern = gemm_cluster_kernel<A_MN, B_MN, TL, EP>;
-  static cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C_SMEM);
+  static OncePerDevice once;
+  const cudaError_t attr = allow_smem(once, kern, C_SMEM);
   if (attr != cudaSuccess) return attr;
   // Ring: as deep as two CTAs an SM allow, also where no SM gets a second: the
   // next kernel's CTAs then fit beside this one's (1024 x 768 x 3072 in three

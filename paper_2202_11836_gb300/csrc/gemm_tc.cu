@@ -689,8 +689,8 @@ cudaError_t launch_variant(const Params& p, int sms, const CUtensorMap& ta, cons
                            cudaStream_t stream, const CUtensorMap* tc = nullptr, const CUtensorMap* tx = nullptr) {
   auto kern = gemm_tc_kernel<A_MN, B_MN, EPI, OUT_F32, PAIR, TBN>;
   using SH = Shape<EPI, PAIR, TBN>;
-  static cudaError_t attr =
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SH::SMEM);
+  static OncePerDevice once;
+  const cudaError_t attr = allow_smem(once, kern, SH::SMEM);
   if (attr != cudaSuccess) return attr;
   int ctas = sms;
   if constexpr (PAIR) {

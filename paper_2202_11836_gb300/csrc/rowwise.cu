@@ -696,19 +696,19 @@ sky_status layernorm_bwd(const void* dy, sky_dtype dy_dt, const float* dy2, cons
     const size_t fixed = (size_t)rw::SB_RING * rw::SB_ROW_BYTES + 2 * rw::SB_RING * 8 +
                          (size_t)rw::SB_PAIRS * 2 * 2 * 4 * 4 + 128;
     const size_t smem = fixed + (size_t)H * 4;
-    // the attribute is set once, for the largest H this variant takes
+    // the attribute is set once a device, for the largest H this variant takes
     const size_t smem_max = fixed + 1024 * 4;
     const int threads = 32 * (rw::SB_WARPS + 1);
     if (dy_dt == SKY_DTYPE_BF16) {
-      static cudaError_t a = cudaFuncSetAttribute(rw::ln_bwd_stream_kernel<__nv_bfloat16>,
-                                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max);
+      static OncePerDevice once;
+      const cudaError_t a = allow_smem(once, rw::ln_bwd_stream_kernel<__nv_bfloat16>, smem_max);
       if (a != cudaSuccess) return cuda_fail(a, "LayerNorm backward smem attribute");
       launch_pdl(rw::ln_bwd_stream_kernel<__nv_bfloat16>, dim3(sb), dim3(threads), smem, st, 1, 
           static_cast<const __nv_bfloat16*>(dy), dy2, u, static_cast<const __nv_bfloat16*>(gamma),
           mean, rstd, rows, H, du32, static_cast<__nv_bfloat16*>(du), part, status);
     } else {
-      static cudaError_t a = cudaFuncSetAttribute(rw::ln_bwd_stream_kernel<float>,
-                                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max);
+      static OncePerDevice once;
+      const cudaError_t a = allow_smem(once, rw::ln_bwd_stream_kernel<float>, smem_max);
       if (a != cudaSuccess) return cuda_fail(a, "LayerNorm backward smem attribute");
       launch_pdl(rw::ln_bwd_stream_kernel<float>, dim3(sb), dim3(threads), smem, st, 1, 
           static_cast<const float*>(dy), dy2, u, static_cast<const __nv_bfloat16*>(gamma), mean,
