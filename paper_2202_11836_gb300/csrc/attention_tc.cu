@@ -1170,8 +1170,8 @@ __global__ void __maxnreg__(80) attn_bwd_dkdv_tc(const __grid_constant__ CUtenso
     const int r = q4 * 32 + lane;    // key row within the tile == TMEM lane
     const int key = k0 + r;
     const uint32_t lane_base = static_cast<uint32_t>(q4 * 32) << 16;
-    const float sl2 = LOG2E * 0.125f, pad = key < len ? 0.f : -INFINITY;
-    const uint64_t sc2 = pack2(sl2, sl2), off = pack2(pad, pad);
+    const float sl2 = LOG2E * 0.125f;
+    const uint64_t sc2 = pack2(sl2, sl2);
     bool ok = true;
     auto wait_all = [&](uint64_t* bar, uint32_t parity) {
       const bool mine = ptx::mbar_wait(bar, parity, lim, p.status, kWaitHint);
@@ -1188,8 +1188,8 @@ __global__ void __maxnreg__(80) attn_bwd_dkdv_tc(const __grid_constant__ CUtenso
       uint32_t pp[16], dd[16];
 #pragma unroll
       for (int t = 0; t < 32; t += 2) {
-        // (a key past the valid length: exp2(-inf) = 0)
-        const float2 x = unpack2(fma2(pack2(__uint_as_float(sv[t]), __uint_as_float(sv[t + 1])), sc2, off));
+        // (a key past the valid length gets a row of its own, which the epilogue drops)
+        const float2 x = unpack2(mul2(pack2(__uint_as_float(sv[t]), __uint_as_float(sv[t + 1])), sc2));
         const float2 pt = make_float2(ptx::ex2_ftz(x.x), ptx::ex2_ftz(x.y));
         const float2 ds = unpack2(mul2(pack2(pt.x, pt.y), pack2(__uint_as_float(dv[t]), __uint_as_float(dv[t + 1]))));
         pp[t >> 1] = ptx::pack_bf16(pt.x, pt.y);
@@ -1225,6 +1225,12 @@ __global__ void __maxnreg__(80) attn_bwd_dkdv_tc(const __grid_constant__ CUtenso
       ptx::tmem_ld_32x32b_x32(tacc + lane_base, o[0]);
       ptx::tmem_ld_32x32b_x32(tacc + lane_base + 32, o[1]);
       ptx::tmem_ld_wait();
+      if (k0 + q4 * 32 + 32 > len) {  // warp-uniform: rows of keys past the valid length are zero
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+#pragma unroll
+          for (int j = 0; j < 32; ++j) o[c][j] = key < len ? o[c][j] : 0u;
+      }
 #pragma unroll
       for (int c = 0; c < 2; ++c)
 #pragma unroll
