@@ -1397,14 +1397,21 @@ __global__ void __launch_bounds__(SH_THR, 2) attn_bwd_short_tc(const __grid_cons
       ptx::tc_fence_after();
       const uint64_t pt = mnmaj(SH_P), dst = mnmaj(SH_DS), ds = kmaj(SH_DS);
       const uint64_t bo = mnmaj(SH_O), bq = mnmaj(SH_Q), bk = mnmaj(SH_K);
+      // Only the 16-row blocks that hold a query (of dO and Q) or a valid key (of K):
+      // the rows behind are other sequences' or padding, and a zero of P or dS
+      // times an infinity or NaN there would reach this sequence's gradients.
+      const int nq = (S + 15) / 16, nk = (len + 15) / 16;
       if (issuer) {
 #pragma unroll
-        for (int kk = 0; kk < 8; ++kk) ptx::tc_mma_f16(tdV, pt + kk * 128, bo + kk * 128, idT, kk > 0 ? 1u : 0u);
+        for (int kk = 0; kk < 8; ++kk)
+          if (kk < nq) ptx::tc_mma_f16(tdV, pt + kk * 128, bo + kk * 128, idT, kk > 0 ? 1u : 0u);
 #pragma unroll
-        for (int kk = 0; kk < 8; ++kk) ptx::tc_mma_f16(tdK, dst + kk * 128, bq + kk * 128, idT, kk > 0 ? 1u : 0u);
+        for (int kk = 0; kk < 8; ++kk)
+          if (kk < nq) ptx::tc_mma_f16(tdK, dst + kk * 128, bq + kk * 128, idT, kk > 0 ? 1u : 0u);
 #pragma unroll
         for (int kk = 0; kk < 8; ++kk)  // keys 16 kk ..: chunk kk / 4
-          ptx::tc_mma_f16(tdQ, ds + (kk >> 2) * (Q_BYTES >> 4) + (kk & 3) * 2, bk + kk * 128, idN, kk > 0 ? 1u : 0u);
+          if (kk < nk)
+            ptx::tc_mma_f16(tdQ, ds + (kk >> 2) * (Q_BYTES >> 4) + (kk & 3) * 2, bk + kk * 128, idN, kk > 0 ? 1u : 0u);
       }
       __syncwarp();
     }

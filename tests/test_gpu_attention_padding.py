@@ -53,3 +53,33 @@ def test_scores_of_padded_keys_may_overflow(S, lens):
     for b, n in enumerate(lens):
         assert not got[2][b, n:, 1:].any()  # dK and dV of padded keys: exactly zero
     assert torch.equal(got[2], want[2])
+
+
+@pytest.mark.parametrize("S", [32, 64, 96, 128, 192])
+def test_other_sequences_may_be_nan(S):
+    """Lengths of whole 32-row blocks (the forward's step; from 129 tokens on 64-row
+    ones): no row of the next sequence meets this one's."""
+    A, B = 2, 3
+    qkv, dctx = inputs(B, S, A, S)
+    lens = [S, S, max(1, S - 5)]
+    want = attention(qkv, dctx, lens)
+    q2, d2 = qkv.clone(), dctx.clone()
+    q2[1], d2[1] = float("nan"), float("inf")
+    got = attention(q2, d2, lens)
+    for b in (0, 2):
+        for g, w in zip(got, want):
+            assert torch.equal(g[b], w[b])
+
+
+@pytest.mark.parametrize("S,n", [(128, 64), (128, 32), (100, 64), (64, 32), (256, 128), (200, 64)])
+def test_padded_keys_may_be_nan(S, n):
+    """The same for keys past a valid length of whole blocks."""
+    A = 2
+    qkv, dctx = inputs(2, S, A, S + n)
+    want = attention(qkv, dctx, [n, n])
+    nan = qkv.clone()
+    nan[:, n:, 1:] = float("nan")
+    if S % 64:  # the last sequence only: its rows meet no other's queries
+        nan[0] = qkv[0]
+    for g, w in zip(attention(nan, dctx, [n, n]), want):
+        assert torch.equal(g, w)
