@@ -45,9 +45,10 @@ struct ClusterPlan {
   int bn, ks;
 };
 // Whether a product goes to the cluster kernel, and with which tiles.
-// may_split: an fp32 output without bias or residual (C += product is none); colpart: column sums per
-// 32 rows are wanted.
-bool plan_cluster(sky_gemm_form form, int M, int N, int K, bool may_split, bool colpart, int sms,
+// may_split: an fp32 output without bias or residual (C += product is none); ws_split: of
+// those, with a workspace that holds the persistent kernel's partial sums; colpart: column
+// sums per 32 rows are wanted.
+bool plan_cluster(sky_gemm_form form, int M, int N, int K, bool may_split, bool ws_split, bool colpart, int sms,
                   ClusterPlan* out);
 // Arguments as launch_bf16, already checked there.
 sky_status launch_cluster(sky_gemm_form form, const ClusterPlan& pl, int M, int N, int K, const void* A,

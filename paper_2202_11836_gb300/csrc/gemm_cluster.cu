@@ -577,13 +577,31 @@ sky_status launch_cluster(sky_gemm_form form, const ClusterPlan& pl, int M, int 
 //     decides, and a 256 x 128 tile on two pairs reads the least.
 //   half to one CTA an SM: the same from 24 k-blocks on (2048 x 768 x 3072 old
 //     18.3, unsplit 15.9, here 13.2); a split of 64-wide tiles, with more CTAs
-//     than SMs, loses.  Weight gradients over 88 k-blocks: old, level or better.
-//   fewer: two splits, and three or six while the clusters fill no more than
-//     three quarters of the SMs (they have to fit the SMs' groups): 64 x 768 x
-//     3072 old 18.7, six splits 5.2; 1024 x 768 x 768 old 8.0, unsplit 5.1.
+//     than SMs, loses.
+//   fewer: from 12 k-blocks on two splits, and three or six while the clusters
+//     fill no more than three quarters of the SMs (they have to fit the SMs'
+//     groups): 64 x 768 x 3072 old 18.7, six splits 5.2; 1024 x 768 x 768 old 8.0,
+//     unsplit 5.1.  Six also on all SMs from 64 k-blocks on (256 x 768 x 4096 in
+//     three 7.4, six 7.5; x 6144 9.4 and 8.8), and three also with up to one and a
+//     half CTAs an SM over 96 (768 x 768 x 6144 in two 14.3, three 13.7; x 8192 23.5
+//     and 18.6).  Under 12 a split gains nothing (64 x 768 x 512 3.5, in two 4.0, six
+//     3.8; x 640 3.9, 4.1 and 3.8).
+// Long K ranges whose partial sums the workspace can take (weight gradients of
+// many tokens; others have no other split and stay): few CTAs do not draw the
+// operands from memory fast enough, and the persistent kernel's splits, on all SM
+// pairs, are level or better.  M x N x K, old and here with the operands in L2 / in
+// memory:
+//   under half a CTA an SM, over 32 k-blocks a CTA and SM, or over 200: 768 x 768 x
+//     4096 12.5 13.4 / 9.7 13.5, x 8192 15.1 15.9 / 17.0 19.0; 512 x 512 x 8192 12.8
+//     14.1 / 11.5 17.5, x 16384 16.6 18.1 / 19.7 30.8; 128 x 768 x 12288 12.7 14.6 / 9.7
+//     14.6, x 16384 14.1 16.3 / 11.7 18.3.
+//   up to one CTA an SM, over 88: level or better.
+//   above, over 88 where the pairs' last wave is less than a third full: 1024 x
+//     1536 x 5000 18.0 19.0 / 17.8 19.2, x 8192 22.5 23.4 / 24.4 26.6; fuller ones stay:
+//     768 x 2304 x 8192 27.6 28.4 / 24.9 27.6.
 // Over the sweep the choice is twice as fast as before at 64 and 128 rows, 1.8
 // times at 404, 1.6 at 1024, 1.34 at 2048, 1.15 at 4096.
-bool plan_cluster(sky_gemm_form form, int M, int N, int K, bool may_split, bool colpart, int sms,
+bool plan_cluster(sky_gemm_form form, int M, int N, int K, bool may_split, bool ws_split, bool colpart, int sms,
                   ClusterPlan* out) {
   const int kb = ceil_div(K, CBK);
   const int64_t t64 = static_cast<int64_t>(ceil_div(M, CBM)) * ceil_div(N, 64);
@@ -595,7 +613,11 @@ bool plan_cluster(sky_gemm_form form, int M, int N, int K, bool may_split, bool 
     return kb <= (full ? 24 : 48);
   }
   const bool many = t64 > sms / 2;
-  if (may_split && kb > 88 && many && t64 <= sms) return false;
+  if (ws_split) {
+    const int64_t pairs = std::max(1, sms / 2), units = 2 * static_cast<int64_t>(ceil_div(M, 2 * CBM)) * ceil_div(N, 128);
+    if (!many && (kb * t64 > 32 * sms || kb > 200)) return false;
+    if (many && kb > 88 && (t64 <= sms || 3 * units < 2 * pairs * ceil_div(units, pairs))) return false;
+  }
   if (many) {
     const bool pair = M >= 2 * CBM && !colpart && kb >= (t64 <= sms ? 24 : 40);
     *out = pair ? ClusterPlan{true, 128, 2} : ClusterPlan{false, 64, 1};
@@ -608,7 +630,7 @@ bool plan_cluster(sky_gemm_form form, int M, int N, int K, bool may_split, bool 
     if (!colpart) {
       if (6 * t64 <= (kb >= 64 ? sms : room)) ks = 6;
       else if (3 * t64 <= room) ks = 3;
-      else if (kb > 96) ks = 4 * t64 <= sms ? 6 : 3;
+      else if (kb > 96) ks = 3;
     }
   }
   *out = ClusterPlan{false, 64, ks};

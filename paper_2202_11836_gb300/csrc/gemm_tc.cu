@@ -832,7 +832,9 @@ sky_status launch_bf16(sky_gemm_form form, int M, int N, int K, const void* A, c
   const bool may_split = out_f32 && epi == SKY_EPI_STORE && bias == nullptr && (!resid || add);
   if (!colsum) {  // small and mid-sized products: the cluster kernel
     ClusterPlan pl;
-    bool here = plan_cluster(form, M, N, K, may_split, deferred_rows != nullptr, sms, &pl);
+    const size_t partials = may_split && ws ? workspace_bytes(form, M, N, K, true) : 0;
+    const bool ws_split = partials > 0 && ws_bytes >= partials;
+    bool here = plan_cluster(form, M, N, K, may_split, ws_split, deferred_rows != nullptr, sms, &pl);
     // GELU' off the 16-byte grid cannot be written by TMA: 8-byte stores do it
     if (!here && epi == SKY_EPI_BIAS_GELU && (reinterpret_cast<uintptr_t>(aux_out) & 15) != 0) {
       pl = ClusterPlan{false, 64, 1};

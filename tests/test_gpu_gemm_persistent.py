@@ -89,3 +89,30 @@ def test_gelu_of_infinities(M, N):
     assert torch.equal(torch.isnan(c), nan) and bool((c[inf] == math.inf).all())
     f = ~(inf | nan)
     assert bool(((c[f] - ref[f]).abs() <= 2.0 ** -8 * ref[f].abs() + 2e-5 * (1 + z[f].abs())).all())
+
+
+# both sides of the lines for long K ranges (152 SMs, k-blocks of 64): 36 tiles to 135,
+# 12 to 200, 96 to 88, 192 to 88 (their pairs' last wave is a quarter full), 256: none
+@pytest.mark.parametrize("M,N,kb", [(384, 768, 135), (384, 768, 136), (128, 768, 200), (128, 768, 201), (768, 1024, 88),
+                                    (768, 1024, 89), (1024, 1536, 88), (1024, 1536, 89), (1024, 2048, 89)])
+@pytest.mark.parametrize("ragged", [False, True])
+def test_long_weight_gradients(M, N, kb, ragged):
+    """With a workspace for split sums and without one; each repeats itself."""
+    K = 64 * kb - (3 if ragged else 0)
+    g = torch.Generator(device="cuda").manual_seed(M + N + K)
+    a = torch.randn(K, M, device="cuda", generator=g).bfloat16()
+    b = (0.05 * torch.randn(K, N, device="cuda", generator=g)).bfloat16()
+    ref = a.double().T @ b.double()
+    nb = L.lib().sky_gemm_workspace_bytes(L.SKY_GEMM_XTW, M, N, K, L.SKY_DTYPE_BF16, L.SKY_DTYPE_FP32)
+    ws = torch.empty(max(16, nb), dtype=torch.uint8, device="cuda")
+    for w, n in ((ws, nb), (None, 0), (ws, max(0, nb - 16))):
+        outs = []
+        for _ in range(2):
+            c = torch.full((M, N), -7.0, device="cuda")
+            L.call("sky_gemm", L.SKY_GEMM_XTW, M, N, K, L.SKY_DTYPE_BF16, P(a), P(b), P(c), L.SKY_DTYPE_FP32,
+                   L.SKY_EPI_STORE, None, None, None, P(w), n, None,
+                   C.c_void_p(int(torch.cuda.current_stream().cuda_stream)))
+            outs.append(c)
+        # fp32 sums of K products of bf16 values
+        assert float((outs[0] - ref).norm() / ref.norm()) <= 1e-5
+        assert torch.equal(*outs)
