@@ -133,16 +133,18 @@ __global__ void attn_delta(const T* __restrict__ ctx, const T* __restrict__ dctx
 // heads of 64.
 constexpr int FR = 16, FC = 64, F_THR = 128;  // rows of a CTA, columns of a tile
 constexpr int FP_LD = FC + 4;                 // row stride of the probability tiles
+// (the backward of sequences up to 16 tokens: tiles of 16 columns, NC = 1 of 4)
 
 // Rows are staged F_THR / G a pass, G threads a row (D <= 4 G), through registers, so
 // that a tile's loads are all in flight before the first is stored.  Loading and
 // storing in turn waited for each: 4 x 32 tokens, 2 heads of 64, forward 6.4 us,
 // now 3.8, backward 10.7 and 7.3; 4 x 101, 12 heads 17.0 and 12.2, 39.9 and 29.4; 4 x
 // 256, 24 heads of 32 52.6 and 48.7 (58.1 with 16 threads a row).
-template <int G>
-struct Stage {  // a tile's FC rows: BATCHES of PASSES passes, R rows each
-  static constexpr int PASSES = FC * G / F_THR < 8 ? FC * G / F_THR : 8;
-  static constexpr int R = PASSES * F_THR / G, BATCHES = FC / R;
+template <int G, int NC = FC / 16>
+struct Stage {  // a tile's 16 NC rows: BATCHES of PASSES passes, R rows each
+  static constexpr int ROWS = 16 * NC;
+  static constexpr int PASSES = ROWS * G / F_THR < 8 ? ROWS * G / F_THR : 8;
+  static constexpr int R = PASSES * F_THR / G, BATCHES = ROWS / R;
   static constexpr int OWN = FR * G / F_THR;  // passes of the CTA's FR rows
   static constexpr int CC = G > 16 ? G / 16 : 1;  // 64-value column groups of an output row
 };
@@ -177,33 +179,34 @@ __device__ __forceinline__ void put_rows(float* s, int LD, int D, const float4 (
     *reinterpret_cast<float4*>(s + (F_THR / G * i + threadIdx.x / G) * LD + c) = v[i];
 }
 // acc[i][c] = row (2 ty + i) . column row (tx + 16 c), over D (a multiple of 4 in shared memory)
-__device__ __forceinline__ void scores(const float* rows, const float* cols, int LD, int D, float (&acc)[2][4]) {
+template <int NC>
+__device__ __forceinline__ void scores(const float* rows, const float* cols, int LD, int D, float (&acc)[2][NC]) {
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
 #pragma unroll
   for (int i = 0; i < 2; ++i)
 #pragma unroll
-    for (int c = 0; c < 4; ++c) acc[i][c] = 0.f;
+    for (int c = 0; c < NC; ++c) acc[i][c] = 0.f;
   for (int d = 0; d < D; d += 4) {
-    float4 r[2], k[4];
+    float4 r[2], k[NC];
 #pragma unroll
     for (int i = 0; i < 2; ++i) r[i] = *reinterpret_cast<const float4*>(rows + (2 * ty + i) * LD + d);
 #pragma unroll
-    for (int c = 0; c < 4; ++c) k[c] = *reinterpret_cast<const float4*>(cols + (tx + 16 * c) * LD + d);
+    for (int c = 0; c < NC; ++c) k[c] = *reinterpret_cast<const float4*>(cols + (tx + 16 * c) * LD + d);
 #pragma unroll
     for (int i = 0; i < 2; ++i)
 #pragma unroll
-      for (int c = 0; c < 4; ++c)
+      for (int c = 0; c < NC; ++c)
         acc[i][c] = fmaf(r[i].w, k[c].w, fmaf(r[i].z, k[c].z, fmaf(r[i].y, k[c].y, fmaf(r[i].x, k[c].x, acc[i][c]))));
   }
 }
 // o[i][cc] += sum_j w[2 ty + i][j] cols[j][4 tx + 64 cc ..] over the tile's first n columns (n <= 64)
-template <int CC>
+template <int CC, int W_LD = FP_LD>
 __device__ __forceinline__ void accumulate(const float* w, const float* cols, int LD, int D, int n, float4 (&o)[2][CC]) {
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   for (int j = 0; j < n; j += 4) {
     float4 p[2];
 #pragma unroll
-    for (int i = 0; i < 2; ++i) p[i] = *reinterpret_cast<const float4*>(w + (2 * ty + i) * FP_LD + j);
+    for (int i = 0; i < 2; ++i) p[i] = *reinterpret_cast<const float4*>(w + (2 * ty + i) * W_LD + j);
 #pragma unroll
     for (int cc = 0; cc < CC; ++cc) {
       const int d = 4 * tx + 64 * cc;
@@ -347,17 +350,17 @@ __global__ void __launch_bounds__(F_THR) attn_fwd_f32(const float* __restrict__ 
 // operand of the columns / sqrt(D), dV = P . dO.  Four CTAs an SM (128 registers) are
 // faster up to a head dim of 64 (29.8 us against 34.7 at 4 x 101, 12 heads), above it
 // the registers are (50.6 against 57.0 at 2 x 200, 6 heads of 128).
-template <int G>
+template <int G, int NC>
 __global__ void __launch_bounds__(F_THR, G > 16 ? 1 : 4) attn_bwd_f32(const float* __restrict__ qkv, const float* __restrict__ dctx,
                                                       const float* __restrict__ lse, const float* __restrict__ delta,
                                                       const int32_t* __restrict__ lens, int S, int H, int A, int D,
                                                       int LD, bool vec, float* __restrict__ dqkv) {
-  using ST = Stage<G>;
-  constexpr int CC = ST::CC;
+  using ST = Stage<G, NC>;
+  constexpr int CC = ST::CC, TC = ST::ROWS, P_LD = TC + 4;
   pdl_wait();
   extern __shared__ __align__(16) float sm[];
-  float *r0s = sm, *r1s = r0s + FR * LD, *c0s = r1s + FR * LD, *c1s = c0s + FC * LD;
-  float *sds = c1s + FC * LD, *sp = sds + FR * FP_LD, *sl = sp + FR * FP_LD, *sd = sl + FC;
+  float *r0s = sm, *r1s = r0s + FR * LD, *c0s = r1s + FR * LD, *c1s = c0s + TC * LD;
+  float *sds = c1s + TC * LD, *sp = sds + FR * P_LD, *sl = sp + FR * P_LD, *sd = sl + TC;
   const int tiles = (S + FR - 1) / FR;
   const bool keys = blockIdx.x & 1;  // own rows are keys
   const int u = static_cast<int>(blockIdx.x) >> 1;
@@ -384,12 +387,12 @@ __global__ void __launch_bounds__(F_THR, G > 16 ? 1 : 4) attn_bwd_f32(const floa
       lr[i] = lse_b[r];
       dr[i] = del_b[r];
     }
-    for (int c0 = 0; c0 < cols; c0 += FC) {
+    for (int c0 = 0; c0 < cols; c0 += TC) {
       __syncthreads();
       // columns: queries (Q, dO; all S) or keys (K, V; the valid ones)
       const float *x0 = keys ? q : q + H, *x1 = keys ? dO : q + 2 * H;
       float lc = 0.f, dc = 0.f;
-      if (keys && threadIdx.x < FC) {
+      if (keys && threadIdx.x < TC) {
         const int c = min(c0 + static_cast<int>(threadIdx.x), S - 1);
         lc = lse_b[c];
         dc = del_b[c];
@@ -407,28 +410,28 @@ __global__ void __launch_bounds__(F_THR, G > 16 ? 1 : 4) attn_bwd_f32(const floa
         put_rows<G>(c0s + R * h * LD, LD, D, v0);
         put_rows<G>(c1s + R * h * LD, LD, D, v1);
       }
-      if (keys && threadIdx.x < FC) {
+      if (keys && threadIdx.x < TC) {
         sl[threadIdx.x] = lc;
         sd[threadIdx.x] = dc;
       }
       __syncthreads();
-      float s[2][4], dp[2][4];
+      float s[2][NC], dp[2][NC];
       scores(r0s, c0s, LD, D, s);
       scores(r1s, c1s, LD, D, dp);
 #pragma unroll
       for (int i = 0; i < 2; ++i)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
+        for (int c = 0; c < NC; ++c) {
           const int cl = tx + 16 * c;
           const bool live = c0 + cl < cols && (!keys || r0 + 2 * ty + i < len);
           const float p = live ? exp2f(fmaf(s[i][c], sl2, -(keys ? sl[cl] : lr[i]))) : 0.f;
-          sds[(2 * ty + i) * FP_LD + cl] = live ? p * (dp[i][c] - (keys ? sd[cl] : dr[i])) : 0.f;
-          if (keys) sp[(2 * ty + i) * FP_LD + cl] = p;
+          sds[(2 * ty + i) * P_LD + cl] = live ? p * (dp[i][c] - (keys ? sd[cl] : dr[i])) : 0.f;
+          if (keys) sp[(2 * ty + i) * P_LD + cl] = p;
         }
       __syncwarp();
-      const int n = min(FC, cols - c0);
-      accumulate<CC>(sds, c0s, LD, D, n, o0);
-      if (keys) accumulate<CC>(sp, c1s, LD, D, n, o1);
+      const int n = min(TC, cols - c0);
+      accumulate<CC, P_LD>(sds, c0s, LD, D, n, o0);
+      if (keys) accumulate<CC, P_LD>(sp, c1s, LD, D, n, o1);
       __syncwarp();
     }
   }
@@ -443,7 +446,9 @@ __global__ void __launch_bounds__(F_THR, G > 16 ? 1 : 4) attn_bwd_f32(const floa
 // 16-byte accesses.
 constexpr int row_stride(int D) { return (D + 3) / 4 * 4 + 4; }
 constexpr int fwd_smem(int D) { return ((FR + 2 * FC) * row_stride(D) + FR * FP_LD) * 4; }
-constexpr int bwd_smem(int D) { return ((2 * FR + 2 * FC) * row_stride(D) + 2 * FR * FP_LD + 2 * FC) * 4; }
+constexpr int bwd_smem(int D, int NC) {
+  return ((2 * FR + 32 * NC) * row_stride(D) + 2 * FR * (16 * NC + 4) + 32 * NC) * 4;
+}
 template <int G>
 using Group = std::integral_constant<int, G>;
 struct F32Shape {
@@ -546,18 +551,25 @@ sky_status attention_bwd(const void* qkv, const void* ctx, const void* dctx, con
                                 static_cast<const float*>(ctx), static_cast<const float*>(dctx), S, H, A, D, rows,
                                 delta);
     const attn::F32Shape f(S, H, A, D, qkv, dctx, dqkv);
-    const auto go = [&](auto group, auto kern) {
+    const auto go = [&](auto group, auto nc, auto kern) {
+      constexpr int G = decltype(group)::value, NC = decltype(nc)::value;
       static OncePerDevice once;
-      const cudaError_t e = allow_smem(once, kern, attn::bwd_smem(4 * decltype(group)::value));
+      const cudaError_t e = allow_smem(once, kern, attn::bwd_smem(4 * G, NC));
       if (e != cudaSuccess) return e;
-      return launch_pdl(kern, dim3(2 * f.units, B), dim3(attn::F_THR), attn::bwd_smem(D), stream, 1,
+      return launch_pdl(kern, dim3(2 * f.units, B), dim3(attn::F_THR), attn::bwd_smem(D, NC), stream, 1,
                         static_cast<const float*>(qkv), static_cast<const float*>(dctx), lse,
                         static_cast<const float*>(delta), lens, S, H, A, D, f.LD, f.vec, static_cast<float*>(dqkv));
     };
+    // Up to 16 tokens a 64-column tile is mostly empty: 128 x 8 tokens, 6 heads of 128
+    // 52.4 us with it, 27.8 with 16 columns (a warp a row 28.8); 12 of 64 45.2 and 25.5
+    // (41.1); 64 x 16, 12 of 64 29.8 and 18.3 (70.4).
+    const auto width = [&](auto group) {
+      constexpr int G = decltype(group)::value;
+      return S <= 16 ? go(group, std::integral_constant<int, 1>{}, attn::attn_bwd_f32<G, 1>)
+                     : go(group, std::integral_constant<int, 4>{}, attn::attn_bwd_f32<G, 4>);
+    };
     if (le == cudaSuccess)
-      le = D <= 32   ? go(attn::Group<8>{}, attn::attn_bwd_f32<8>)
-           : D <= 64 ? go(attn::Group<16>{}, attn::attn_bwd_f32<16>)
-                     : go(attn::Group<32>{}, attn::attn_bwd_f32<32>);
+      le = D <= 32 ? width(attn::Group<8>{}) : D <= 64 ? width(attn::Group<16>{}) : width(attn::Group<32>{});
     if (le != cudaSuccess) return cuda_fail(le, "attention backward launch");
   }
   count_launches(2);

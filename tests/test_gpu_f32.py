@@ -115,3 +115,10 @@ def test_attention_first_scores_overflow(S, len_, hidden):
         assert l2rel(to_host(c[b, :, a]), ref[b, :, a].cpu().numpy()) <= 2e-6
         assert maxrel(to_host(lse[b, a]), ref_lse[b, a].cpu().numpy()) <= 2e-6
     assert bool(torch.isnan(c[1, :, 1]).all())
+
+
+@pytest.mark.parametrize("B,S,A,D,lens", [(3, 16, 2, 128, [16, 1, 9]), (2, 8, 3, 64, [8, 5]), (2, 16, 1, 100, [16, 15]),
+                                          (1, 3, 2, 32, [2]), (2, 16, 2, 7, [4, 16]), (2, 17, 1, 128, [17, 16])])
+def test_attention_of_tiny_sequences(B, S, A, D, lens):
+    """Both sides of the backward's narrow tiles."""
+    test_attention(B, S, A, D, lens)
