@@ -9,11 +9,9 @@ namespace sky {
 namespace gemm {
 
 // bf16 inputs on tcgen05; C is bf16 unless out_f32.
-// colsum (optional, bf16 output, no split): also writes out[n] = sum_m C[m, n]
-// (before rounding), with fixed-order partials (one row per 32 rows of C) in
-// `ws`.  With `deferred_rows`, the partials go to `colpart` instead, no sum is
-// launched and *deferred_rows reports their row count (for reduce_rows_f32,
-// possibly on another stream ordered after this launch).
+// colpart (optional, GELU_BWD epilogue): also writes partial column sums of C
+// (before rounding), one row per 32 rows of C; *colpart_rows reports how many (for
+// a fixed-order reduction, possibly on another stream ordered after this launch).
 // resid (optional, fp32 output of the STORE epilogue, no split): C = acc +
 // bias + resid[m, n], added in that order (the residual branch of Sec. II-C).
 // resid == C (XTW form, no bias): C += product, which may be split.
@@ -31,8 +29,8 @@ struct LnResid {
 sky_status launch_bf16(sky_gemm_form form, int M, int N, int K, const void* A, const void* B,
                        void* C, bool out_f32, int epi, const void* bias, const void* aux,
                        void* aux_out, void* ws, size_t ws_bytes, int32_t* status,
-                       cudaStream_t stream, float* colsum = nullptr, float* colpart = nullptr,
-                       size_t colpart_bytes = 0, int* deferred_rows = nullptr,
+                       cudaStream_t stream, float* colpart = nullptr, size_t colpart_bytes = 0,
+                       int* colpart_rows = nullptr,
                        const float* resid = nullptr, const LnResid* ln = nullptr);
 // 2-D bf16 tensor map over a row-major [rows, cols] matrix, box {64, box_rows},
 // 128-byte swizzle; out-of-range elements read as zero.

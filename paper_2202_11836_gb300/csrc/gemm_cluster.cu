@@ -500,10 +500,7 @@ template <bool A_MN, bool B_MN, class TL>
 cudaError_t launch_epi(int epi, ClusterParams& p, const CUtensorMap& ta, const CUtensorMap& tb, cudaStream_t st) {
   if (epi == SKY_EPI_BIAS_GELU) return launch_one<A_MN, B_MN, TL, E_GELU>(p, ta, tb, st);
   if (epi == SKY_EPI_GELU_BWD) return launch_one<A_MN, B_MN, TL, E_GELU_BWD>(p, ta, tb, st);
-  if constexpr (A_MN) {
-    if (p.resid && p.resid == p.C) return launch_one<A_MN, B_MN, TL, E_ADD>(p, ta, tb, st);
-  }
-  if (p.resid) return launch_one<A_MN, B_MN, TL, E_RESID>(p, ta, tb, st);
+  if (p.resid) return launch_one<A_MN, B_MN, TL, A_MN ? E_ADD : E_RESID>(p, ta, tb, st);
   return launch_one<A_MN, B_MN, TL, E_STORE>(p, ta, tb, st);
 }
 

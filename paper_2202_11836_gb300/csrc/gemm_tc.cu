@@ -741,7 +741,7 @@ cudaError_t launch_form(const Params& p, int sms, const CUtensorMap& ta, const C
 }
 
 // The pair variant serves every problem with at least one full 256-row tile.
-bool use_pair(int M, int /*epi*/) { return M >= 2 * BM; }
+bool use_pair(int M) { return M >= 2 * BM; }
 
 uint64_t g_timeout_ns = 2000000000ull;  // 2 s per wait
 int g_skip_loads = 0;
@@ -780,7 +780,7 @@ int choose_splits(int64_t mn, int tiles, int k_blocks, int sms) {
 
 size_t workspace_bytes(sky_gemm_form form, int M, int N, int K, bool out_f32) {
   if (!out_f32) return 0;
-  const bool pair = use_pair(M, SKY_EPI_STORE);  // fp32 outputs use the STORE epilogue
+  const bool pair = use_pair(M);
   const int tiles = ceil_div(M, pair ? 2 * BM : BM) * ceil_div(N, BN);
   const int kb = ceil_div(K, BK);
   const int sms = sm_count() > 0 ? sm_count() : 148;
@@ -792,8 +792,8 @@ size_t workspace_bytes(sky_gemm_form form, int M, int N, int K, bool out_f32) {
 sky_status launch_bf16(sky_gemm_form form, int M, int N, int K, const void* A, const void* B,
                        void* C, bool out_f32, int epi, const void* bias, const void* aux,
                        void* aux_out, void* ws, size_t ws_bytes, int32_t* status,
-                       cudaStream_t stream, float* colsum, float* colpart, size_t colpart_bytes,
-                       int* deferred_rows, const float* resid, const LnResid* ln) {
+                       cudaStream_t stream, float* colpart, size_t colpart_bytes, int* colpart_rows,
+                       const float* resid, const LnResid* ln) {
   // TMA row pitches and the 16-byte epilogue stores need the contiguous
   // dimensions to be multiples of 8 elements; the token dimension is free.
   const bool dims_ok = N % 8 == 0 && (form == SKY_GEMM_XTW ? M % 8 == 0 : K % 8 == 0);
@@ -816,7 +816,9 @@ sky_status launch_bf16(sky_gemm_form form, int M, int N, int K, const void* A, c
   const auto a8 = [](const void* q) { return (reinterpret_cast<uintptr_t>(q) & 7) == 0; };
   SKY_CHECK(a8(bias) && (epi != SKY_EPI_GELU_BWD || a8(aux)) && (epi != SKY_EPI_BIAS_GELU || a8(aux_out)),
             SKY_ERR_UNSUPPORTED, "GEMM bias, aux and aux_out must be 8-byte aligned");
-  SKY_CHECK(!resid || (out_f32 && epi == SKY_EPI_STORE && !colsum && !deferred_rows &&
+  SKY_CHECK(!colpart || (epi == SKY_EPI_GELU_BWD && colpart_rows), SKY_ERR_UNSUPPORTED,
+            "column sums come with the GELU' epilogue");
+  SKY_CHECK(!resid || (out_f32 && epi == SKY_EPI_STORE &&
                        (reinterpret_cast<uintptr_t>(resid) & 15) == 0),
             SKY_ERR_UNSUPPORTED, "a residual needs a 16-byte aligned fp32 output of the STORE epilogue");
   SKY_CHECK(!ln || (resid && ln->mean && ln->rstd && ln->gamma && ln->beta &&
@@ -827,38 +829,36 @@ sky_status launch_bf16(sky_gemm_form form, int M, int N, int K, const void* A, c
   SKY_CHECK(sms > 0, SKY_ERR_CUDA, "no CUDA device");
 
   const bool add = resid && resid == C;  // C += product
-  SKY_CHECK(!add || (form == SKY_GEMM_XTW && !bias && !ln), SKY_ERR_UNSUPPORTED,
-            "only a weight gradient is added to its output");
+  SKY_CHECK(!resid || add == (form == SKY_GEMM_XTW), SKY_ERR_UNSUPPORTED,
+            "only a weight gradient is added to its output, and nothing else to a weight gradient");
+  SKY_CHECK(!add || (!bias && !ln), SKY_ERR_UNSUPPORTED, "a weight gradient is added without a bias");
   const bool may_split = out_f32 && epi == SKY_EPI_STORE && bias == nullptr && (!resid || add);
-  if (!colsum) {  // small and mid-sized products: the cluster kernel
+  {  // small and mid-sized products: the cluster kernel
     ClusterPlan pl;
     const size_t partials = may_split && ws ? workspace_bytes(form, M, N, K, true) : 0;
     const bool ws_split = partials > 0 && ws_bytes >= partials;
-    bool here = plan_cluster(form, M, N, K, may_split, ws_split, deferred_rows != nullptr, sms, &pl);
+    bool here = plan_cluster(form, M, N, K, may_split, ws_split, colpart != nullptr, sms, &pl);
     // GELU' off the 16-byte grid cannot be written by TMA: 8-byte stores do it
     if (!here && epi == SKY_EPI_BIAS_GELU && (reinterpret_cast<uintptr_t>(aux_out) & 15) != 0) {
       pl = ClusterPlan{false, 64, 1};
       here = true;
     }
     if (here) {
-      float* part = nullptr;
-      if (deferred_rows) {
-        SKY_CHECK(!out_f32, SKY_ERR_UNSUPPORTED, "fused column sum needs a bf16 output");
+      if (colpart) {
         const int rows = ceil_div(M, pl.pair ? 2 * BM : BM) * (pl.pair ? 8 : 4);  // one per 32 rows
-        SKY_CHECK(colpart && colpart_bytes >= static_cast<size_t>(rows) * N * sizeof(float),
-                  SKY_ERR_INVALID_ARG, "GEMM column-sum workspace too small");
-        part = colpart;
-        *deferred_rows = rows;
+        SKY_CHECK(colpart_bytes >= static_cast<size_t>(rows) * N * sizeof(float), SKY_ERR_INVALID_ARG,
+                  "GEMM column-sum workspace too small");
+        *colpart_rows = rows;
       }
       return launch_cluster(form, pl, M, N, K, A, B, C, out_f32, epi, bias, aux, aux_out, status,
-                            g_timeout_ns, g_skip_loads, stream, part, resid, ln);
+                            g_timeout_ns, g_skip_loads, stream, colpart, resid, ln);
     }
   }
 
   CUtensorMap ta, tb, tc{}, tx{};
   const bool a_mn = form == SKY_GEMM_XTW;
   const bool b_mn = form != SKY_GEMM_XWT;
-  const bool pair = use_pair(M, epi);
+  const bool pair = use_pair(M);
   // 192-wide pair tiles for K-major B and the plain-store epilogue (bf16 or
   // fp32 output, bias and residual allowed; no split-K) when the product is
   // less than one wave of 256-wide tiles and still one wave of 192-wide ones:
@@ -867,8 +867,7 @@ sky_status launch_bf16(sky_gemm_form form, int M, int N, int K, const void* A, c
   // the fuller last wave gained: QKV at T = 8192 took 47.1 instead of 43.1 us.)
   const int clusters = sms / 2;
   const int64_t m_t = ceil_div(M, pair ? 2 * BM : BM);
-  const bool narrow = pair && form == SKY_GEMM_XWT && epi == SKY_EPI_STORE && !may_split &&
-                      !colsum && !deferred_rows && N % 192 == 0 &&
+  const bool narrow = pair && form == SKY_GEMM_XWT && epi == SKY_EPI_STORE && !may_split && N % 192 == 0 &&
                       m_t * ceil_div(N, BN) < clusters && m_t * (N / 192) <= clusters;
   const int tbn = narrow ? 192 : BN;
   bool ok = a_mn ? make_map(&ta, A, K, M, 64) : make_map(&ta, A, M, K, BM);
@@ -893,17 +892,12 @@ sky_status launch_bf16(sky_gemm_form form, int M, int N, int K, const void* A, c
   SKY_CHECK(ws_bytes >= need && (need == 0 || ws), SKY_ERR_INVALID_ARG,
             "GEMM workspace too small (%zu < %zu)", ws_bytes, need);
   p.C = p.splits > 1 ? ws : C;
-  // optional fused column sum of C (bf16 outputs only): per-warp partials in
-  // the workspace, added in a fixed order after the kernel
-  const int colpart_rows = p.m_tiles * (pair ? 8 : 4);  // one per 32 rows of every tile
-  if (colsum || deferred_rows) {
-    SKY_CHECK(!out_f32 && p.splits == 1, SKY_ERR_UNSUPPORTED, "fused column sum needs a bf16 output");
-    float* buf = deferred_rows ? colpart : static_cast<float*>(ws);
-    const size_t cap = deferred_rows ? colpart_bytes : ws_bytes;
-    SKY_CHECK(buf && cap >= static_cast<size_t>(colpart_rows) * N * sizeof(float),
-              SKY_ERR_INVALID_ARG, "GEMM column-sum workspace too small");
-    p.colpart = buf;
-    if (deferred_rows) *deferred_rows = colpart_rows;
+  if (colpart) {
+    const int rows = p.m_tiles * (pair ? 8 : 4);  // one per 32 rows of every tile
+    SKY_CHECK(colpart_bytes >= static_cast<size_t>(rows) * N * sizeof(float), SKY_ERR_INVALID_ARG,
+              "GEMM column-sum workspace too small");
+    p.colpart = colpart;
+    *colpart_rows = rows;
   }
   p.bias = static_cast<const __nv_bfloat16*>(bias);
   p.resid = add && p.splits > 1 ? nullptr : resid;
@@ -940,10 +934,6 @@ sky_status launch_bf16(sky_gemm_form form, int M, int N, int K, const void* A, c
   }
   count_launches(1);
   if (e != cudaSuccess) return cuda_fail(e, "gemm_tc_kernel launch");
-  if (colsum && !deferred_rows) {
-    e = reduce_rows_f32(p.colpart, colpart_rows, N, colsum, stream);
-    if (e != cudaSuccess) return cuda_fail(e, "column-sum reduce launch");
-  }
   if (p.splits > 1) {
     const int64_t n = static_cast<int64_t>(M) * N;
     const int blocks = static_cast<int>(std::min<int64_t>(ceil_div(n / 4 + 1, 256), sms * 8));

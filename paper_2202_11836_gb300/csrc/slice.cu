@@ -118,8 +118,6 @@ struct sky_slice {
   float *dP[2], *dR[2], *dU2_32, *dP1;
   void *dU2b, *dU1b, *dH, *dctx, *dqkv;           // dtype copies / branch gradients
   float* delta;
-  void* ws;
-  size_t ws_bytes;
   int32_t* d_status;
   // bf16 slices: the first layer's fp32 residual input (the caller's x when it
   // is fp32 and 16-byte aligned, else the fp32 copy x32 made at the start of
@@ -234,27 +232,11 @@ size_t param_elems(const sky_slice* s, int k) {
 
 size_t align_up(size_t x) { return (x + 255) & ~size_t(255); }
 
-// Scratch needed by the backward pass at T tokens (shared by all steps).
-size_t workspace_need(const sky_slice* s, int64_t T) {
-  const int H = s->H, F = s->F;
-  size_t need = 0;
-  if (s->cfg.dtype == SKY_DTYPE_BF16) {
-    const int64_t shapes[4][2] = {{3 * H, H}, {H, H}, {F, H}, {H, F}};
-    for (auto& sh : shapes)
-      need = std::max(need, gemm::workspace_bytes(SKY_GEMM_XTW, (int)sh[0], (int)sh[1], (int)T, true));
-  }
-  need = std::max(need, layernorm_bwd_ws((int)T, H));
-  need = std::max(need, (size_t)ceil_div(T, 128) * 4 * F * sizeof(float));  // fused db1 partials
-  need = std::max(need, column_sum_ws((int)T, F));
-  need = std::max(need, column_sum_ws((int)T, 3 * H));
-  return need;
-}
-
 // Split-K scratch of the weight-gradient GEMMs (their own, so they can run
 // beside the main stream's kernels).
 size_t side_workspace_need(const sky_slice* s, int64_t T) {
   const int H = s->H, F = s->F;
-  size_t need = column_sum_ws((int)T, 3 * H);  // dbqkv
+  size_t need = 0;
   const int64_t shapes[4][2] = {{3 * H, H}, {H, H}, {F, H}, {H, F}};
   for (auto& sh : shapes)
     need = std::max(need, gemm::workspace_bytes(SKY_GEMM_XTW, (int)sh[0], (int)sh[1], (int)T, true));
@@ -297,17 +279,13 @@ struct Timed {
 
 sky_status run_gemm(sky_slice* s, cudaStream_t st, int cat, sky_gemm_form form, int M, int N,
                     int K, const void* A, const void* Bm, void* C, bool out_f32, int epi,
-                    const void* bias, const void* aux, void* aux_out, float* colsum = nullptr,
-                    void* ws = nullptr, size_t ws_bytes = 0, const float* resid = nullptr,
+                    const void* bias, const void* aux, void* aux_out, void* ws = nullptr,
+                    size_t ws_bytes = 0, const float* resid = nullptr,
                     const gemm::LnResid* ln = nullptr) {
   Timed t(s, st, cat, 2.0 * M * N * K, 0);
-  if (!ws) {
-    ws = s->ws;
-    ws_bytes = s->ws_bytes;
-  }
   if (s->cfg.dtype == SKY_DTYPE_BF16)
     return gemm::launch_bf16(form, M, N, K, A, Bm, C, out_f32, epi, bias, aux, aux_out, ws,
-                             ws_bytes, s->d_status, st, colsum, nullptr, 0, nullptr, resid, ln);
+                             ws_bytes, s->d_status, st, nullptr, 0, nullptr, resid, ln);
   return gemm::launch_f32(form, M, N, K, static_cast<const float*>(A),
                           static_cast<const float*>(Bm), static_cast<float*>(C), epi,
                           static_cast<const float*>(bias), static_cast<const float*>(aux),
@@ -351,7 +329,7 @@ sky_status forward_layer(sky_slice* s, int i, void* y_out, cudaStream_t st) {
       r = Pv.U2;
     }
     SKY_TRY(run_gemm(s, st, P_GEMM_FWD, SKY_GEMM_XWT, T, H, H, Lb.ctx, Lb.p[2], Lb.U1, true,
-                     SKY_EPI_STORE, Lb.p[3], nullptr, nullptr, nullptr, nullptr, 0,
+                     SKY_EPI_STORE, Lb.p[3], nullptr, nullptr, nullptr, 0,
                      bf ? r : nullptr, ln));
   }
   {
@@ -369,7 +347,7 @@ sky_status forward_layer(sky_slice* s, int i, void* y_out, cudaStream_t st) {
   {
     const gemm::LnResid ln1{Lb.mean1, Lb.rstd1, Lb.p[4], Lb.p[5]};
     SKY_TRY(run_gemm(s, st, P_GEMM_FWD, SKY_GEMM_XWT, T, H, F, Lb.G, Lb.p[8], Lb.U2, true,
-                     SKY_EPI_STORE, Lb.p[9], nullptr, nullptr, nullptr, nullptr, 0,
+                     SKY_EPI_STORE, Lb.p[9], nullptr, nullptr, nullptr, 0,
                      bf ? Lb.U1 : nullptr, bf ? &ln1 : nullptr));
   }
   {
@@ -459,14 +437,14 @@ sky_status backward_layer(sky_slice* s, int i, const void* dY, sky_dtype dy_dt, 
   //            dZ = (dU2 W2) * GELU'(Z);
   //            db1 = sum_rows dZ (fused into the bf16 epilogue; a column-sum pass for fp32)
   SKY_TRY(run_gemm(s, sw, P_GEMM_WGRAD, SKY_GEMM_XTW, H, F, T, s->dU2b, Lb.G, G[8], true,
-                   SKY_EPI_STORE, nullptr, nullptr, nullptr, nullptr, ws2, ws2b, acc(8)));
+                   SKY_EPI_STORE, nullptr, nullptr, nullptr, ws2, ws2b, acc(8)));
   SKY_TRY(done(0));
   SKY_TRY(reuse(1));
   if (bf) {
     Timed t(s, st, P_GEMM_DGRAD, 2.0 * T * F * H, 0);
     SKY_TRY(gemm::launch_bf16(SKY_GEMM_XW, T, F, H, s->dU2b, Lb.p[8], s->dH, false,
-                              SKY_EPI_GELU_BWD, nullptr, Lb.Gp, nullptr, s->ws, s->ws_bytes,
-                              s->d_status, st, nullptr, s->db1p[k], s->db1p_bytes, &db1_rows));
+                              SKY_EPI_GELU_BWD, nullptr, Lb.Gp, nullptr, nullptr, 0, s->d_status, st,
+                              s->db1p[k], s->db1p_bytes, &db1_rows));
   } else {
     SKY_TRY(run_gemm(s, st, P_GEMM_DGRAD, SKY_GEMM_XW, T, F, H, s->dU2b, Lb.p[8], s->dH, false,
                      SKY_EPI_GELU_BWD, nullptr, Lb.Gp, nullptr));
@@ -475,10 +453,10 @@ sky_status backward_layer(sky_slice* s, int i, const void* dY, sky_dtype dy_dt, 
   // a12: dX1 = dZ W1 + dU2 (fp32; bf16: dU2 added by the GEMM epilogue, fp32:
   // by the LN1 backward);  dW1 = dZ^T X1
   SKY_TRY(run_gemm(s, st, P_GEMM_DGRAD, SKY_GEMM_XW, T, H, F, s->dH, Lb.p[6], s->dP1, true,
-                   SKY_EPI_STORE, nullptr, nullptr, nullptr, nullptr, nullptr, 0,
+                   SKY_EPI_STORE, nullptr, nullptr, nullptr, nullptr, 0,
                    bf ? s->dU2_32 : nullptr));
   SKY_TRY(run_gemm(s, sw, P_GEMM_WGRAD, SKY_GEMM_XTW, F, H, T, s->dH, Lb.X1b, G[6], true,
-                   SKY_EPI_STORE, nullptr, nullptr, nullptr, nullptr, ws2, ws2b, acc(6)));
+                   SKY_EPI_STORE, nullptr, nullptr, nullptr, ws2, ws2b, acc(6)));
   SKY_TRY(done(1));
   // a13: LN1 backward of dX1 = P1 + dU2 -> dU1 (fp32 + dtype), dgamma1, dbeta1, dbo
   SKY_TRY(reuse(2));
@@ -494,7 +472,7 @@ sky_status backward_layer(sky_slice* s, int i, const void* dY, sky_dtype dy_dt, 
   SKY_TRY(run_gemm(s, st, P_GEMM_DGRAD, SKY_GEMM_XW, T, H, H, dU1b, Lb.p[2], s->dctx, false,
                    SKY_EPI_STORE, nullptr, nullptr, nullptr));
   SKY_TRY(run_gemm(s, sw, P_GEMM_WGRAD, SKY_GEMM_XTW, H, H, T, dU1b, Lb.ctx, G[2], true,
-                   SKY_EPI_STORE, nullptr, nullptr, nullptr, nullptr, ws2, ws2b, acc(2)));
+                   SKY_EPI_STORE, nullptr, nullptr, nullptr, ws2, ws2b, acc(2)));
   SKY_TRY(done(2));
   // a15: attention backward -> dQKV
   SKY_TRY(reuse(3));
@@ -540,8 +518,8 @@ sky_status backward_layer(sky_slice* s, int i, const void* dY, sky_dtype dy_dt, 
   // I/O); fp32: by the next LayerNorm backward, or here for the first layer
   const bool direct = bf && dx && s->cfg.io_fp32 && (reinterpret_cast<uintptr_t>(dx) & 15) == 0;
   SKY_TRY(run_gemm(s, st, P_GEMM_DGRAD, SKY_GEMM_XW, T, H, 3 * H, s->dqkv, Lb.p[0],
-                   direct ? dx : s->dP[k], true, SKY_EPI_STORE, nullptr, nullptr, nullptr, nullptr,
-                   nullptr, 0, bf ? s->dR[k] : nullptr));
+                   direct ? dx : s->dP[k], true, SKY_EPI_STORE, nullptr, nullptr, nullptr, nullptr, 0,
+                   bf ? s->dR[k] : nullptr));
   if (dx && !direct) {
     const sky_dtype odt = s->cfg.io_fp32 ? SKY_DTYPE_FP32 : dt;
     Timed t(s, st, P_COPY, 0, ((bf ? 4.0 : 8.0) + (odt == SKY_DTYPE_BF16 ? 2.0 : 4.0)) * T * H);
@@ -553,7 +531,7 @@ sky_status backward_layer(sky_slice* s, int i, const void* dY, sky_dtype dy_dt, 
       SKY_CUDA(cudaMemcpyAsync(dx, s->dP[k], (size_t)T * H * 4, cudaMemcpyDeviceToDevice, st));
   }
   SKY_TRY(run_gemm(s, sw, P_GEMM_WGRAD, SKY_GEMM_XTW, 3 * H, H, T, s->dqkv, Lb.Xb, G[0], true,
-                   SKY_EPI_STORE, nullptr, nullptr, nullptr, nullptr, ws2, ws2b, acc(0)));
+                   SKY_EPI_STORE, nullptr, nullptr, nullptr, ws2, ws2b, acc(0)));
   SKY_TRY(done(3));
   if (s->accumulate && !bf) {  // Lb.g += scratch: both are the 12 tensors laid out alike, contiguous
     const int64_t n = (Lb.g[SKY_NUM_PARAMS - 1] + param_elems(s, SKY_NUM_PARAMS - 1)) - Lb.g[0];
@@ -811,18 +789,17 @@ static sky_status plan_slice(sky_slice* s, size_t* total) {
   s->param_bytes = pb * s->L;
   s->grad_bytes = gb * s->L;
   s->stash_bytes = stash * s->L * s->n_slots;
-  s->ws_bytes = align_up(workspace_need(s, T));
   s->ws2_bytes = bf ? align_up(side_workspace_need(s, T)) : 0;
   s->lnp_bytes = align_up(layernorm_bwd_ws((int)T, s->H));
   s->db1p_bytes = align_up(bf ? (size_t)gemm::colpart_rows_max((int)T) * s->F * 4 : column_sum_ws((int)T, s->F));
   s->qkvp_bytes = align_up(bf ? (size_t)c.max_batch * ceil_div(c.max_seq, 128) * 3 * s->H * 4
                               : column_sum_ws((int)T, 3 * s->H));
-  // dP[2] dR[2] dU2_32 dP1 | dU2b dU1b dctx (bf16) | dH | dqkv | delta | ws | ws2 | lnp[2] |
+  // dP[2] dR[2] dU2_32 dP1 | dU2b dU1b dctx (bf16) | dH | dqkv | delta | ws2 | lnp[2] |
   // db1p | qkvp | status | x32 (bf16)
   const size_t wk = (bf ? 7 : 6) * t32 + (bf ? 3 : 1) * th + align_up((size_t)T * s->F * s->esz) +
                     align_up((size_t)T * 3 * s->H * s->esz) +
-                    align_up(attention_bwd_ws(c.max_batch, c.max_seq, s->A)) + s->ws_bytes +
-                    s->ws2_bytes + 4 * s->lnp_bytes + 2 * s->db1p_bytes + 2 * s->qkvp_bytes + 256 +
+                    align_up(attention_bwd_ws(c.max_batch, c.max_seq, s->A)) + s->ws2_bytes +
+                    4 * s->lnp_bytes + 2 * s->db1p_bytes + 2 * s->qkvp_bytes + 256 +
                     (s->n_slots > 1 && !bf ? gb : 0);  // gradient-accumulation scratch (one layer)
   s->ws_bytes_total = wk;
   *total = s->param_bytes + s->grad_bytes + s->stash_bytes + wk;
@@ -932,7 +909,6 @@ sky_status sky_slice_create(const sky_slice_config* cfg, sky_slice** out) {
   s->dH = take((size_t)T * s->F * s->esz);
   s->dqkv = take((size_t)T * 3 * s->H * s->esz);
   s->delta = static_cast<float*>(take(attention_bwd_ws(c.max_batch, c.max_seq, s->A)));
-  s->ws = take(s->ws_bytes);
   if (s->ws2_bytes) s->ws2 = take(s->ws2_bytes);
   for (int k = 0; k < 2; ++k) {
     if (s->lnp_bytes) {
