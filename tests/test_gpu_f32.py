@@ -26,11 +26,12 @@ def stream():
 
 
 # (1, 1, 1): all remainder; 33 / 65 / 130: past a slab, a tile; (5, 7, 1000): eight
-# splits of a ragged K; (2432, 640, 256) and (2496, 640, 256): 380 and 390 tiles, the
-# last split and the first unsplit size on 152 SMs; (63, 640, 96): three slabs
+# splits of a ragged K; (2624, 640, 256) and (2688, 640, 256): 410 and 420 tiles, either
+# side of the last split (eleven CTAs an SM, 152 SMs); (63, 640, 96): three slabs
 @pytest.mark.parametrize("form", [L.SKY_GEMM_XWT, L.SKY_GEMM_XW, L.SKY_GEMM_XTW])
 @pytest.mark.parametrize("shape", [(1, 1, 1), (65, 33, 130), (5, 7, 1000), (128, 384, 128), (63, 640, 96),
-                                   (404, 768, 516), (2432, 640, 256), (2496, 640, 256), (130, 65, 33)],
+                                   (404, 768, 516), (2432, 640, 256), (2496, 640, 256), (2624, 640, 256),
+                                   (2688, 640, 256), (130, 65, 33)],
                          ids=lambda s: "x".join(map(str, s)))
 def test_gemm(form, shape):
     M, N, K = shape
