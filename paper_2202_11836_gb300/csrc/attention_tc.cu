@@ -45,6 +45,7 @@
 
 #include "common.cuh"
 #include "ptx.cuh"
+#include "residency.h"
 
 namespace sky {
 namespace attn_tc {
@@ -1640,11 +1641,12 @@ sky_status attention_fwd_tc(const void* qkv, const int32_t* lens, int B, int S, 
   auto go = [&](auto splits, auto bufs) {
     constexpr int KS = decltype(splits)::value, NS = decltype(bufs)::value;
     auto kern = attn_fwd_tc<KS, NS>;
+    constexpr int SMEM = KS > 1 ? kSplitAttentionSmem : FwdShape<NS>::SMEM;
+    static_assert(SMEM >= FwdShape<NS>::SMEM && (KS == 1 || FwdShape<NS>::TMEM_COLS <= 256), "see residency.h");
     static OncePerDevice once;
-    const cudaError_t attr = allow_smem(once, kern, FwdShape<NS>::SMEM);
+    const cudaError_t attr = allow_smem(once, kern, SMEM);
     if (attr != cudaSuccess) return attr;
-    return launch_pdl(kern, dim3(ceil_div(S, BQ) * KS, A, B), dim3(NTHR), FwdShape<NS>::SMEM, stream, KS, tq, tkv,
-                      tout, p);
+    return launch_pdl(kern, dim3(ceil_div(S, BQ) * KS, A, B), dim3(NTHR), SMEM, stream, KS, tq, tkv, tout, p);
   };
   const std::integral_constant<int, 1> c1{};
   const std::integral_constant<int, 2> c2{};

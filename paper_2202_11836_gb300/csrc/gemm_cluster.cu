@@ -35,6 +35,7 @@
 #include "common.cuh"
 #include "gemm.h"
 #include "ptx.cuh"
+#include "residency.h"
 
 namespace sky {
 namespace gemm {
@@ -493,7 +494,9 @@ cudaError_t launch_one(ClusterParams& p, const CUtensorMap& ta, const CUtensorMa
   p.bar_off = ring + TL::RECV_BYTES;
   p.red_off = p.bar_off + 256;
   const int tiles = ceil_div(p.M, TL::TILE_M) * p.n_tiles;
-  return launch_pdl(kern, dim3(tiles * TL::CL), dim3(C_THREADS), p.bar_off + tail, st, TL::CL, ta, tb, p);
+  static_assert(kClusterProductSmem <= C_SMEM && TL::BN <= 128, "see residency.h");
+  const int smem = std::max(p.bar_off + tail, TL::CL > 1 ? kClusterProductSmem : 0);
+  return launch_pdl(kern, dim3(tiles * TL::CL), dim3(C_THREADS), smem, st, TL::CL, ta, tb, p);
 }
 
 template <bool A_MN, bool B_MN, class TL>
